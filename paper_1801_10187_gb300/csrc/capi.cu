@@ -284,8 +284,10 @@ struct Engine {
   // per kernel variant: thermostat (1) | walls or beads (2) | warp-spread members (4);
   // for the warp-spread kernel bit 2 means a nonzero body force, bit 8 beads
   // and bit 16 the Andersen rule
-  // per-cell kernel: bit 16 the Andersen rule, bit 32 the angular correction
-  static constexpr int NVAR = 64;
+  // per-cell kernel: bit 16 the Andersen rule, bit 32 the angular correction;
+  // bit 64: the register kernel of periodic mixed SRD boxes (bits 1, 2 and 8
+  // as for the warp-spread kernel)
+  static constexpr int NVAR = 128;
   int2* d_spans[NVAR] = {};
   int n_spans[NVAR] = {};
   ScanSeg* d_bsegs = nullptr;
@@ -304,14 +306,8 @@ struct Engine {
   bool any_beads = false;
   int wca_substeps = 0;  // most MD substeps of a box with the WCA repulsion (0: none)
   int cells_bps[3][NVAR] = {};
-  // F mode of the mixed SRD warp variants: blocks per SM for each pass-2 chunk
-  // depth (2, 3, 4), and the depth in use (a launch-tuner choice)
-  int bps_chunk[5][NVAR] = {};
-  int tuned_chunk = 3;
-  // the same variants with 16 and 8 cells per warp (chunks of 3), and the
-  // cells per warp in use (a launch-tuner choice)
-  int bps_narrow[2][NVAR] = {};
-  int tuned_cpw = 32;
+  // k_srd: cells per warp chosen by the launch tuner (0: by size)
+  int tuned_cpw = 0;
 
   cudaGraphExec_t gexec[3] = {nullptr, nullptr, nullptr};  // MODE_P, MODE_F, MODE_C
   bool tables_ok = false;
@@ -332,37 +328,22 @@ struct Engine {
     for (int m = 0; m < 3; ++m)
       for (int v = 0; v < NVAR; ++v) {
         const bool at = (v & 16) != 0, ang = (v & 32) != 0;
-        if ((v & 4) && ang)  // warp-spread angular correction: mixed SRD without beads
-          cells_bps[m][v] = (mixed && !(v & (8 | 16)))
-                                ? cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, false,
-                                                           true, m, 3, 32)
-                                : 1;
-        else if ((v & 4) && !(at && (v & 1)))
+        cells_bps[m][v] = 1;
+        if (v & 64) {
+          if (mixed && !(v & (4 | 16 | 32)))
+            cells_bps[m][v] = srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, m);
+        } else if ((v & 4) && ang) {  // warp-spread angular correction: mixed SRD without beads
+          if (mixed && !(v & (8 | 16)))
+            cells_bps[m][v] = cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, false, true, m);
+        } else if ((v & 4) && !(at && (v & 1))) {
           cells_bps[m][v] =
-              mixed ? cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, false, m, 3, 32)
+              mixed ? cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, false, m)
                     : cells_warpd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, m);
-        else if (!(v & 4))
+        } else if (!(v & 4)) {
           cells_bps[m][v] = cells_blocks_per_sm(mixed, v, m);
-        else
-          cells_bps[m][v] = 1;
+        }
         if (cells_bps[m][v] < 1) cells_bps[m][v] = 1;
       }
-    for (int v = 0; v < NVAR; ++v) {
-      for (int ch = 2; ch <= 4; ++ch) {
-        bps_chunk[ch][v] = cells_bps[MODE_F][v];
-        if (chunk_tunable(v))
-          bps_chunk[ch][v] = std::max(1, cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0,
-                                                                  (v & 8) != 0, false, false,
-                                                                  MODE_F, ch, 32));
-      }
-      for (int k = 0; k < 2; ++k) {
-        bps_narrow[k][v] = cells_bps[MODE_F][v];
-        if (chunk_tunable(v))
-          bps_narrow[k][v] = std::max(1, cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0,
-                                                                  (v & 8) != 0, false, false,
-                                                                  MODE_F, 3, k == 0 ? 16 : 8));
-      }
-    }
     CUDA_TRY((cudaError_t)md_bin_prepare());
     CUDA_TRY(cudaMalloc(&d_err, sizeof(int)));
     CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), stream));
@@ -504,8 +485,9 @@ struct Engine {
       if ((!d.angular || warp_ang) && !d.walls && d.K <= WARP_MAX_K &&
           std::max(d.n[0], std::max(d.n[1], d.n[2])) < (1 << 22)) {
         const bool force = d.g[0] != 0.0 || d.g[1] != 0.0 || d.g[2] != 0.0;
-        variant = 4 | (d.thermostat ? 1 : 0) | (force ? 2 : 0) | (d.nbead > 0 ? 8 : 0) |
-                  (d.collision == RULE_AT ? 16 : 0) | (d.angular ? 32 : 0);
+        const bool reg = mixed && !at && !d.angular && d.K <= SRD_SLOTS;
+        variant = (reg ? 64 : 4) | (d.thermostat ? 1 : 0) | (force ? 2 : 0) |
+                  (d.nbead > 0 ? 8 : 0) | (at ? 16 : 0) | (d.angular ? 32 : 0);
       }
       for (int c0 = 0; c0 < d.ncells; c0 += BLOCK) sp[variant].push_back(make_int2((int)i, c0));
       if (d.nbead > 0) {
@@ -544,27 +526,31 @@ struct Engine {
     return MPCD_OK;
   }
 
-  // variants whose F-mode launch takes the tuned pass-2 chunk depth
-  bool chunk_tunable(int v) const { return mixed && (v & 4) && !(v & (16 | 32)); }
-
   int grid_for(int n, int per_sm) const {
     const int g = nsm * per_sm;
     return n < g ? std::max(n, 1) : g;
   }
 
+  // Cells per warp of the register kernel: as chosen by the tuner, else the
+  // most of 32, 16, 8 and 4 that still gives every SM SRD_MIN_WARPS warps.
+  int srd_cpw() const {
+    if (tuned_cpw) return tuned_cpw;
+    int64_t cells = 0;
+    for (int v = 64; v < NVAR; ++v) cells += (int64_t)n_spans[v] * BLOCK;
+    int cpw = 32;
+    while (cpw > 4 && cells < (int64_t)cpw * SRD_MIN_WARPS * nsm) cpw >>= 1;
+    return cpw;
+  }
+
   // Grid of the fused pass: tuned_grid 0 = the occupancy limit (blocks per
   // SM that fit), k > 0 = at most k blocks per SM, -1 = one block per span
-  // part (a 256-cell span has 32 / cells-per-warp parts).
+  // part (the register kernel takes a 256-cell span in parts).
   int tuned_grid = 0;
   int grid_of(int v, int mode) const {
-    const bool narrow = mode == MODE_F && chunk_tunable(v) && tuned_cpw != 32;
-    const int items = n_spans[v] * (narrow ? 32 / tuned_cpw : 1);
+    const int items = n_spans[v] * ((v & 64) ? srd_parts(srd_cpw()) : 1);
     if (mode == MODE_F && tuned_grid == -1) return std::max(items, 1);
-    const int limit = (mode != MODE_F) ? cells_bps[mode][v]
-                      : narrow         ? bps_narrow[tuned_cpw == 16 ? 0 : 1][v]
-                                       : bps_chunk[tuned_chunk][v];
-    const int bps = (mode == MODE_F && tuned_grid > 0) ? std::min(tuned_grid, limit) : limit;
-    return grid_for(items, bps);
+    const int limit = cells_bps[mode][v];
+    return grid_for(items, (mode == MODE_F && tuned_grid > 0) ? std::min(tuned_grid, limit) : limit);
   }
 
   void launch_cells_all(int mode) {
@@ -572,10 +558,12 @@ struct Engine {
       if (n_spans[v] == 0) continue;
       const int grid = grid_of(v, mode);
       const bool at = (v & 16) != 0;
-      if ((v & 4) && mixed)
+      if (v & 64)
+        launch_srd((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, mode, d_boxes, d_spans[v], n_spans[v],
+                   grid, srd_cpw(), d_err, stream);
+      else if ((v & 4) && mixed)
         launch_cells_warp((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, (v & 32) != 0, mode,
-                          d_boxes, d_spans[v], n_spans[v], grid, tuned_chunk, tuned_cpw, d_err,
-                          stream);
+                          d_boxes, d_spans[v], n_spans[v], grid, d_err, stream);
       else if (v & 4)
         launch_cells_warpd((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, mode, d_boxes,
                            d_spans[v], n_spans[v], grid, d_err, stream);
@@ -681,29 +669,21 @@ struct Engine {
       pending = true;
       taken += 1;
     }
-    bool any_chunk = false;
-    for (int v = 0; v < NVAR; ++v)
-      if (n_spans[v] > 0 && chunk_tunable(v)) any_chunk = true;
-    // (cells per warp, chunk depth) pairs
-    std::vector<std::pair<int, int>> shapes;
-    if (any_chunk)
-      shapes = {{32, 2}, {32, 3}, {32, 4}, {16, 3}, {8, 3}};
-    else
-      shapes = {{32, 3}};
+    bool any_reg = false;
+    for (int v = 64; v < NVAR; ++v)
+      if (n_spans[v] > 0) any_reg = true;
+    std::vector<int> widths = {32};  // cells per warp
+    if (any_reg) widths = {32, 16, 8};
     cudaEvent_t e0, e1;
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));
     double best = 1e30;
-    int best_c = 0, best_ch = 3, best_cpw = 32;
-    for (const auto& shape : shapes) {
-      const int ch = shape.second;
-      tuned_cpw = shape.first;
-      tuned_chunk = ch;
+    int best_c = 0, best_cpw = 32;
+    for (int width : widths) {
+      tuned_cpw = width;
       int maxbps = 1;
       for (int v = 0; v < NVAR; ++v)
-        if (n_spans[v] > 0)
-          maxbps = std::max(maxbps, tuned_cpw == 32 ? bps_chunk[ch][v]
-                                                    : bps_narrow[tuned_cpw == 16 ? 0 : 1][v]);
+        if (n_spans[v] > 0) maxbps = std::max(maxbps, cells_bps[MODE_F][v]);
       std::vector<int> cand;
       for (int k = 1; k <= maxbps; ++k) cand.push_back(k);
       cand.push_back(-1);
@@ -719,7 +699,6 @@ struct Engine {
         if (ms / (double)reps < best) {
           best = ms / (double)reps;
           best_c = c;
-          best_ch = ch;
           best_cpw = tuned_cpw;
         }
       }
@@ -727,12 +706,11 @@ struct Engine {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     tuned_grid = best_c;
-    tuned_chunk = best_ch;
     tuned_cpw = best_cpw;
     drop_graphs();
     CUDA_TRY(cudaGetLastError());
     if (chosen) *chosen = best_c;
-    if (chosen_chunk) *chosen_chunk = best_ch;
+    if (chosen_chunk) *chosen_chunk = 3;
     if (chosen_cpw) *chosen_cpw = best_cpw;
     if (best_ms) *best_ms = best;
     if (steps_taken) *steps_taken = taken;
@@ -826,6 +804,14 @@ struct Engine {
     d.collision = p.collision;
     d.K = row_capacity(p, nsol);
     d.angular = p.angular ? 1 : 0;
+    // k_srd: cells per sub-tile, as many as rarely have more members than the
+    // staging area holds
+    d.subc = 32;
+    while (d.subc > 1) {
+      const double mean = (double)nsol / (double)C * d.subc;
+      if (mean + 2.5 * std::sqrt(mean) <= SRD_SLOTS) break;
+      d.subc >>= 1;
+    }
     if (d.collision == RULE_AT && nbead > 0 &&
         (d.K > WARP_MAX_K || std::max(p.n[0], std::max(p.n[1], p.n[2])) >= (1 << 22)))
       return fail(MPCD_EINVAL, "the Andersen rule with solute needs a row capacity <= 448 "

@@ -4,10 +4,11 @@
 // Sec. 3.6 rotation and thermostat, algorithm "SRD collision rule").
 //
 // Same modes, records and results as k_cells (one thread per cell), for boxes
-// without walls (solute beads allowed).  A warp owns 32 consecutive cells (or
-// 16 or 8, a launch-tuner choice; see CPW below).  Their row members are
-// numbered 0 .. N-1 in cell order (a warp prefix sum of the row counts); a
-// byte map gives each member's cell.
+// without walls (solute beads allowed): the Andersen rule, the angular
+// correction, and SRD with rows beyond the SRD_SLOTS records that k_srd, the
+// faster kernel for plain SRD, takes.  A warp owns 32 consecutive cells.  Their
+// row members are numbered 0 .. N-1 in cell order (a warp prefix sum of the row
+// counts); a byte map gives each member's cell.
 //   pass 1   the (v, tag) words of up to 192 members are copied into shared
 //            memory asynchronously in member order (neighbouring lanes,
 //            neighbouring records), issued as soon as the counts are scanned
@@ -25,7 +26,7 @@
 //            moment of the split velocities) and the factor xi; the axis and
 //            the Gamma pair were drawn before pass 1 (they need only the
 //            member count).  u, xi and the axis go to shared memory
-//   pass 2   members in order across the lanes, in chunks of two to four
+//   pass 2   members in order across the lanes, in chunks of three
 //            windows of 32: the chunk's records are copied into shared memory
 //            asynchronously (all in flight at once), each is collided with its
 //            cell's parameters, streamed and binned under the next shift while
@@ -63,7 +64,7 @@ constexpr int MAP_MEMBERS = 640;  // members per warp with a byte owner map
 constexpr int STAGE = 256;        // member velocities staged per block of pass 1
 constexpr int STAGE4 = 192;       // the same for the SRD variants (whole 16-byte words)
 constexpr int STAGE_PAD = STAGE + STAGE / 32;
-constexpr int CHUNK = 3;          // windows of 32 members per chunk of pass 2 (default)
+constexpr int CH = 3;             // windows of 32 members per chunk of pass 2
 
 // The wait for all of this thread's outstanding asynchronous copies (16-byte
 // global -> shared copies that bypass L1, issued below with an L2 policy).
@@ -79,9 +80,6 @@ struct BeadSums {
   unsigned long long E[32];
 };
 
-// CH: windows of 32 members per chunk of pass 2 (the launch tuner picks 2, 3
-// or 4 for the F mode of the SRD variants; 3 elsewhere).
-template <int CH>
 struct WarpShared {
   float4 prm[2][32];               // (u, xi), (axis, 0) per cell
   float2 gdv[32];                  // thermostat: accepted Gamma pair (d, v); d < 0: none
@@ -144,8 +142,7 @@ constexpr int DV_CAP_BEADS = 320;  // with the bead accumulators (two blocks per
 // Shared memory of one block: the span parameters, then one area per warp;
 // kept under 48 KB so that four blocks (the register limit) fit on an SM with
 // room left for L1.
-template <int CH>
-constexpr size_t WARP_SMEM = sizeof(WarpShared<CH>);
+constexpr size_t WARP_SMEM = sizeof(WarpShared);
 
 // Per-span parameters shared by the block.
 struct SpanParams {
@@ -162,8 +159,7 @@ struct SpanParams {
   int ovf_cap, pad;
 };
 constexpr size_t SPAN_SMEM = (sizeof(SpanParams) + 15) & ~(size_t)15;
-template <int CH>
-constexpr size_t BLOCK_SMEM = SPAN_SMEM + WARPS * WARP_SMEM<CH>;
+constexpr size_t BLOCK_SMEM = SPAN_SMEM + WARPS * WARP_SMEM;
 
 // Angular-momentum correction (SRD without beads): the float
 // frame of the collision step's shift (per block), and per warp the staged
@@ -183,10 +179,9 @@ struct AngWarp {
   float4 om[32];  // (omega, 0)
 };
 
-template <int CH = CHUNK>
 __host__ __device__ constexpr size_t block_smem(bool beads, bool at, bool ang = false,
                                                 bool thermo = false) {
-  return BLOCK_SMEM<CH> + (beads ? WARPS * sizeof(BeadShared) : 0) +
+  return BLOCK_SMEM + (beads ? WARPS * sizeof(BeadShared) : 0) +
          (at ? WARPS * (beads ? sizeof(ATShared<DV_CAP_BEADS>) : sizeof(ATShared<DV_CAP>)) : 0) +
          (ang ? sizeof(AngBlock) + WARPS * sizeof(AngWarp) : 0) +
          (thermo ? WARPS * sizeof(ThermoShared) : 0);
@@ -202,16 +197,10 @@ __host__ __device__ constexpr size_t block_smem(bool beads, bool at, bool ang = 
 // AT selects the Andersen rule (then THERMO is false): its two Box-Muller
 // draws per member want registers for independent chains, and its cache of
 // random velocities wants shared memory, so it runs two blocks per SM.
-// CPW: cells per warp (32, or 16 or 8 for the F mode of the SRD variants, a
-// launch-tuner choice).  A warp of CPW < 32 cells leaves lanes CPW..31
-// without a cell (they still take members in the member passes); a 256-cell
-// span is then taken in 32 / CPW parts, each by one block, which puts more
-// blocks on a small box.  Results do not depend on CPW (exact sums).
 // ANG adds the angular-momentum correction to SRD, with or without the
 // thermostat (then BEADS and AT are false); its shared memory allows two
 // blocks per SM.
-template <bool THERMO, int MODE, bool FORCE, bool BEADS, bool AT, bool ANG, int CH = CHUNK,
-          int CPW = 32>
+template <bool THERMO, int MODE, bool FORCE, bool BEADS, bool AT, bool ANG>
 __global__ void __launch_bounds__(BLOCK, (AT || ANG) ? 2 : 4) k_cells_warp(const BoxDev* __restrict__ boxes,
                                                          const int2* __restrict__ spans,
                                                          int nspans, int* err) {
@@ -219,24 +208,21 @@ __global__ void __launch_bounds__(BLOCK, (AT || ANG) ? 2 : 4) k_cells_warp(const
   extern __shared__ __align__(16) unsigned char smem_[];
   SpanParams& sp_ = *reinterpret_cast<SpanParams*>(smem_);
   const int lane = threadIdx.x & 31;
-  WarpShared<CH>& W =
-      reinterpret_cast<WarpShared<CH>*>(smem_ + SPAN_SMEM)[threadIdx.x >> 5];
-  BeadShared& BS = reinterpret_cast<BeadShared*>(smem_ + BLOCK_SMEM<CH>)[threadIdx.x >> 5];
+  WarpShared& W =
+      reinterpret_cast<WarpShared*>(smem_ + SPAN_SMEM)[threadIdx.x >> 5];
+  BeadShared& BS = reinterpret_cast<BeadShared*>(smem_ + BLOCK_SMEM)[threadIdx.x >> 5];
   constexpr int DVC = BEADS ? DV_CAP_BEADS : DV_CAP;
-  ATShared<DVC>& AS = reinterpret_cast<ATShared<DVC>*>(smem_ + block_smem<CH>(BEADS, false))[threadIdx.x >> 5];
-  AngBlock& AB = *reinterpret_cast<AngBlock*>(smem_ + block_smem<CH>(BEADS, AT));
-  AngWarp& AG = reinterpret_cast<AngWarp*>(smem_ + block_smem<CH>(BEADS, AT) + sizeof(AngBlock))[threadIdx.x >> 5];
-  ThermoShared& TS = reinterpret_cast<ThermoShared*>(smem_ + block_smem<CH>(BEADS, AT, ANG))[threadIdx.x >> 5];
+  ATShared<DVC>& AS = reinterpret_cast<ATShared<DVC>*>(smem_ + block_smem(BEADS, false))[threadIdx.x >> 5];
+  AngBlock& AB = *reinterpret_cast<AngBlock*>(smem_ + block_smem(BEADS, AT));
+  AngWarp& AG = reinterpret_cast<AngWarp*>(smem_ + block_smem(BEADS, AT) + sizeof(AngBlock))[threadIdx.x >> 5];
+  ThermoShared& TS = reinterpret_cast<ThermoShared*>(smem_ + block_smem(BEADS, AT, ANG))[threadIdx.x >> 5];
   const SpanParams& H = sp_;
   // SRD variants stage pass 1 by asynchronous copies issued early (above);
   // the Andersen and angular variants load and convert in stage()
   constexpr bool EARLY = !AT && !ANG;
   constexpr int SB = EARLY ? STAGE4 : STAGE;
   int box_of_params = -1;  // the span parameters depend on the box only
-  static_assert(CPW == 32 || CPW == 16 || CPW == 8, "cells per warp");
-  constexpr int PARTS = 32 / CPW;  // parts of a 256-cell span
-  for (int it = blockIdx.x; it < nspans * PARTS; it += gridDim.x) {
-    const int sp = it / PARTS, part = it - sp * PARTS;
+  for (int sp = blockIdx.x; sp < nspans; sp += gridDim.x) {
     const int2 tt = spans[sp];
     const BoxDev& B = boxes[tt.x];
     const unsigned long long t = B.step;
@@ -271,10 +257,10 @@ __global__ void __launch_bounds__(BLOCK, (AT || ANG) ? 2 : 4) k_cells_warp(const
       __syncthreads();
       box_of_params = tt.x;
     }
-    const int c0 = tt.y + part * (WARPS * CPW) + (int)(threadIdx.x >> 5) * CPW;
+    const int c0 = tt.y + (int)(threadIdx.x & ~31u);
     if (c0 >= B.ncells) continue;  // warp-uniform
     const int cell = c0 + lane;
-    const bool valid = (CPW == 32 || lane < CPW) && cell < B.ncells;
+    const bool valid = cell < B.ncells;
     const int cur = B.cur;
     const int K = H.K;
     const uint32_t n = valid ? B.cnt[cur][cell] : 0u;
@@ -408,19 +394,15 @@ __global__ void __launch_bounds__(BLOCK, (AT || ANG) ? 2 : 4) k_cells_warp(const
     if (EARLY && MODE != MODE_P) stage_async(0, min(STAGE4, N));
 
     // Solute beads join their cell's collision with mass M (Sec. 3.6).  The
-    // warp's cells lie in one bead group of 32 cells (all of it when CPW is
-    // 32); the group's beads are handled one per lane (grouped copies of cell
-    // and velocity), those of this warp's cells only: first their count and
-    // exact int64 momentum per cell, into shared sums.
+    // warp's cells are one bead group of 32 cells; the group's beads are
+    // handled one per lane (grouped copies of cell and velocity): first their
+    // count per cell.
     const int gnb = gb1 - gb0;
     int nb = 0;
     auto for_beads = [&](auto&& f) {  // f(slot in the group order, local cell)
       for (int j0 = 0; j0 < gnb; j0 += 32) {
         const int j = gb0 + j0 + lane;
-        if (j0 + lane < gnb) {
-          const int lc = B.bgc[j] - c0;  // beads of the group's other cells: another warp's
-          if (CPW == 32 || (unsigned)lc < (unsigned)CPW) f(j, lc);
-        }
+        if (j0 + lane < gnb) f(j, B.bgc[j] - c0);
       }
     };
     if (BEADS && MODE != MODE_P) {
@@ -1046,9 +1028,5 @@ __global__ void __launch_bounds__(BLOCK, (AT || ANG) ? 2 : 4) k_cells_warp(const
     }
   }
 }
-
-// The F-mode instance of the SRD variant (thermo, force, beads) with cpw = 8 or
-// 16 cells per warp and pass-2 chunks of 3 windows (k_cells_warp_narrow.cu).
-void* cells_warp_narrow_fn(bool thermo, bool force, bool beads, int cpw);
 
 }  // namespace mpcd

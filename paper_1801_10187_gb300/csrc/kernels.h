@@ -26,18 +26,22 @@ void launch_cells(bool mixed, int variant, int mode, const BoxDev* boxes, const 
 // beads: the box has solute beads; at: Andersen-thermostat rule (Eq. at)
 // instead of the rotation (thermo is then false).
 constexpr int WARP_MAX_K = 448;
+// Members that a warp of k_srd stages at a time, and the longest row it takes.
+constexpr int SRD_SLOTS = 192;
 // ang (mixed model, SRD without beads): the angular-momentum correction.
-// chunk: windows of 32 members whose loads and slot requests pass 2 keeps in
-// flight together (2, 3 or 4; used by the F mode of the SRD variants, 3
-// elsewhere); cpw: cells per warp (8, 16 or 32; 8 and 16 only in the F mode
-// of the SRD variants, with chunks of 3, 32 elsewhere).  Both are launch-tuner
-// choices.  With cpw < 32 a 256-cell span is taken in 32 / cpw parts, each by
-// one block: grid sizes count parts.
-int cells_warp_blocks_per_sm(bool thermo, bool force, bool beads, bool at, bool ang, int mode,
-                             int chunk, int cpw);
+int cells_warp_blocks_per_sm(bool thermo, bool force, bool beads, bool at, bool ang, int mode);
 void launch_cells_warp(bool thermo, bool force, bool beads, bool at, bool ang, int mode,
-                       const BoxDev* boxes, const int2* spans, int nspans, int grid, int chunk,
-                       int cpw, int* err, cudaStream_t s);
+                       const BoxDev* boxes, const int2* spans, int nspans, int grid, int* err,
+                       cudaStream_t s);
+// The same step for periodic mixed SRD boxes with rows of at most SRD_SLOTS
+// records, members held in registers (k_srd.cu).  cpw: cells per warp (32, 16,
+// 8 or 4); a 256-cell span is then taken in srd_parts(cpw) parts, one block
+// each: grid sizes count parts.  SRD_MIN_WARPS: see srd_cpw() in capi.cu.
+constexpr int SRD_MIN_WARPS = 16;
+int srd_blocks_per_sm(bool thermo, bool force, bool beads, int mode);
+int srd_parts(int cpw);
+void launch_srd(bool thermo, bool force, bool beads, int mode, const BoxDev* boxes,
+                const int2* spans, int nspans, int grid, int cpw, int* err, cudaStream_t s);
 // The FP64 model's counterpart (k_cells_warp_d.cu), same conditions.
 int cells_warpd_blocks_per_sm(bool thermo, bool force, bool beads, bool at, int mode);
 void launch_cells_warpd(bool thermo, bool force, bool beads, bool at, int mode, const BoxDev* boxes,

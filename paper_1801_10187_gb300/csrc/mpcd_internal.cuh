@@ -119,7 +119,7 @@ struct BoxDev {
   // WCA: epsilon, sigma^2, cutoff^2, list radius^2 (cutoff + buffer), (buffer/2)^2
   double lj_eps, lj_sig2, wca_rc2, wca_rl2, wca_half_skin2;
   int32_t nl_hsize;     // hash buckets of the bead grid (2 per bead, tile-rounded)
-  int32_t pad_w;
+  int32_t subc;         // k_srd: most cells per sub-tile (a power of two)
   int32_t* nl_head;     // bucket -> first bead (-1 empty)
   int32_t* nl_next;     // bead -> next bead in its bucket
   int32_t* nl_key;      // bead -> its cell (edge 1, unshifted) at the build
