@@ -78,6 +78,7 @@ size_t footprint_bytes(const mpcd_params& p, int64_t nsol, int64_t nbead) {
   b += 2 * (size_t)C * sizeof(uint32_t);                                  // counts
   b += 2 * (size_t)std::max<int64_t>(nsol, 1) * (rec_size(mixed) + 4);     // overflow lists
   b += (size_t)nsol * 6 * elem_size(mixed);                               // staging (r, v)
+  b += XBUCKETS * sizeof(uint32_t);                                       // read-out buckets
   if (nbead > 0) {
     b += (size_t)nbead * (9 * sizeof(double) + 2 * sizeof(int32_t) + sizeof(uint64_t) +
                           sizeof(uint32_t));
@@ -870,6 +871,7 @@ struct Engine {
     }
     if ((rc = alloc(b, d.ovf_n, 2))) return rc;
     CUDA_TRY(cudaMemsetAsync(d.ovf_n, 0, sizeof(uint32_t) * 2, stream));
+    if ((rc = alloc(b, d.xcnt, (size_t)XBUCKETS))) return rc;
     if ((rc = alloc_bytes(b, b->stage_r, (size_t)nsol * 3 * es))) return rc;
     if ((rc = alloc_bytes(b, b->stage_v, (size_t)nsol * 3 * es))) return rc;
     if (nbead > 0) {
@@ -960,23 +962,32 @@ struct Engine {
     return place(b, b->stage_r, b->stage_v, nullptr, nullptr, step);
   }
 
-  // The completed state into the box's staging arrays (input order).
-  int extract(Box* b, int32_t* cell_out) {
+  // The last step completed and reported on, the host's record current.
+  int settle() {
     int rc = complete();
     if (rc) return rc;
     if ((rc = pull_records())) return rc;
-    if ((rc = check_err())) return rc;
-    launch_extract(mixed, d_boxes + b->dev_index, b->stage_r, b->stage_v, cell_out,
-                   (int)b->d.ncells, stream);
+    return check_err();
+  }
+
+  // The completed state in input order, into the given device arrays or (NULL)
+  // the box's staging arrays.
+  int extract(Box* b, int32_t* cell_out, void* pos = nullptr, void* vel = nullptr) {
+    const int rc = settle();
+    if (rc) return rc;
+    launch_extract(mixed, d_boxes + b->dev_index, pos ? pos : b->stage_r, vel ? vel : b->stage_v,
+                   cell_out, (int)b->d.ncells, (int)b->nsol, b->d.xcnt, stream);
     CUDA_TRY(cudaGetLastError());
     return MPCD_OK;
   }
 
   int download_state(Box* b, double* pos, double* vel, double* spos, double* svel, uint64_t* step) {
-    int rc = extract(b, nullptr);
+    // a caller that wants only the beads does not pay for the solvent
+    const bool solvent = b->nsol > 0 && (pos || vel);
+    int rc = solvent ? extract(b, nullptr) : settle();
     if (rc) return rc;
     const size_t n3 = (size_t)b->nsol * 3;
-    if (b->nsol > 0 && (pos || vel)) {
+    if (solvent) {
       XferSeg seg[2];
       int nseg = 0;
       if (pos) seg[nseg++] = {pos, b->stage_r, n3};
@@ -1173,13 +1184,9 @@ int mpcd_get_state_device(mpcd_ctx* ctx, void* pos, void* vel) {
   if (!ctx->box->has_state) return fail(MPCD_ESTATE, "no state set");
   Engine& E = ctx->eng;
   Box* b = ctx->box;
-  int rc = E.extract(b, nullptr);
+  // straight into the caller's arrays
+  int rc = E.extract(b, nullptr, pos, vel);
   if (rc) return rc;
-  const size_t bytes = (size_t)b->nsol * 3 * elem_size(E.mixed);
-  if (bytes) {
-    if (pos) CUDA_TRY(cudaMemcpyAsync(pos, b->stage_r, bytes, cudaMemcpyDeviceToDevice, E.stream));
-    if (vel) CUDA_TRY(cudaMemcpyAsync(vel, b->stage_v, bytes, cudaMemcpyDeviceToDevice, E.stream));
-  }
   CUDA_TRY(cudaStreamSynchronize(E.stream));
   CUDA_TRY(cudaGetLastError());
   return MPCD_OK;
@@ -1533,7 +1540,7 @@ extern "C" int mpcd_profile_noalloc(mpcd_ctx* ctx, int32_t nbins, double* out) {
   }
   const int n = (int)b->nsol;
   launch_extract(E.mixed, E.d_boxes + b->dev_index, b->stage_r, b->stage_v, nullptr,
-                 (int)cells_of(b->p), E.stream);
+                 (int)cells_of(b->p), n, b->d.xcnt, E.stream);
   int grid = (n + 255) / 256;
   if (grid < 1) grid = 1;
   if (grid > 4096) grid = 4096;

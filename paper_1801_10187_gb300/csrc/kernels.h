@@ -50,9 +50,13 @@ void launch_cells_warpd(bool thermo, bool force, bool beads, bool at, int mode, 
 // current rows of a box whose counts are zero.
 void launch_load(bool mixed, const BoxDev* box, const void* pos, const void* vel, int n, int* err,
                  cudaStream_t s);
-// Current state into device arrays in input order (cell_out optional).
+// Current state (of a box at rest between steps) into device arrays in input
+// order (cell_out optional); large outputs go through the row set not in use and
+// the box's xcnt.  Outputs up to EXTRACT_DIRECT bytes are scattered directly.
+constexpr size_t EXTRACT_DIRECT = size_t(48) << 20;
+constexpr int XBUCKETS = 1024;
 void launch_extract(bool mixed, const BoxDev* box, void* pos, void* vel, int32_t* cell_out,
-                    int ncells, cudaStream_t s);
+                    int ncells, int nsol, uint32_t* xcnt, cudaStream_t s);
 
 // Thermal initial state drawn on the device into pos/vel (n x 3 of the storage
 // type); sums: 3 device words of scratch.

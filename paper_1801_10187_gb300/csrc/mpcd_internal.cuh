@@ -96,6 +96,7 @@ struct BoxDev {
   void* ovf_rec[2];     // overflow records
   uint32_t* ovf_cell[2];
   uint32_t* ovf_n;      // two counters
+  uint32_t* xcnt;       // records per tag bucket of a state read-out (XBUCKETS)
   // solute
   double* spos;
   double* svel;
