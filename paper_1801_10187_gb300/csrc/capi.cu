@@ -79,6 +79,7 @@ size_t footprint_bytes(const mpcd_params& p, int64_t nsol, int64_t nbead) {
   b += 2 * (size_t)std::max<int64_t>(nsol, 1) * (rec_size(mixed) + 4);     // overflow lists
   b += (size_t)nsol * 6 * elem_size(mixed);                               // staging (r, v)
   b += XBUCKETS * sizeof(uint32_t);                                       // read-out buckets
+  if (mixed && p.walls_z) b += 2 * (size_t)p.n[0] * p.n[1] * (4 * sizeof(long long) + 4);
   if (nbead > 0) {
     b += (size_t)nbead * (9 * sizeof(double) + 2 * sizeof(int32_t) + sizeof(uint64_t) +
                           sizeof(uint32_t));
@@ -286,8 +287,7 @@ struct Engine {
   // for the warp-spread kernel bit 2 means a nonzero body force, bit 8 beads
   // and bit 16 the Andersen rule
   // per-cell kernel: bit 16 the Andersen rule, bit 32 the angular correction;
-  // bit 64: the register kernel of periodic mixed SRD boxes (bits 1, 2 and 8
-  // as for the warp-spread kernel)
+  // bit 64: k_srd (bits 1, 2 and 8 as for the warp-spread kernel; bit 4 walls)
   static constexpr int NVAR = 128;
   int2* d_spans[NVAR] = {};
   int n_spans[NVAR] = {};
@@ -298,6 +298,8 @@ struct Engine {
   int n_btiles = 0;
   int2* d_mdtiles = nullptr;
   int n_mdtiles = 0;
+  int2* d_vtiles = nullptr;  // wall-cut layers of the boxes with virtual particles
+  int n_vtiles = 0;
   int md_chains_per_block = 1, md_threads = 32;
   uint32_t* d_tsum = nullptr;
   unsigned long long* d_gscan = nullptr;
@@ -307,6 +309,7 @@ struct Engine {
   bool any_beads = false;
   int wca_substeps = 0;  // most MD substeps of a box with the WCA repulsion (0: none)
   int cells_bps[3][NVAR] = {};
+  int srd_bead_bps[3][8] = {};  // k_srd's launch over the groups with beads
   // k_srd: cells per warp chosen by the launch tuner (0: by size)
   int tuned_cpw = 0;
 
@@ -331,8 +334,11 @@ struct Engine {
         const bool at = (v & 16) != 0, ang = (v & 32) != 0;
         cells_bps[m][v] = 1;
         if (v & 64) {
-          if (mixed && !(v & (4 | 16 | 32)))
-            cells_bps[m][v] = srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, m);
+          if (mixed && !(v & (16 | 32)) && !((v & 4) && (v & (2 | 8))))
+            if (v & 8)
+              srd_bead_bps[m][v & 7] = std::max(
+                  1, srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, true, (v & 4) != 0, m));
+            cells_bps[m][v] = srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, m);
         } else if ((v & 4) && ang) {  // warp-spread angular correction: mixed SRD without beads
           if (mixed && !(v & (8 | 16)))
             cells_bps[m][v] = cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, false, true, m);
@@ -359,7 +365,7 @@ struct Engine {
   }
 
   void free_tables() {
-    void* ptrs[] = {d_boxes, d_bsegs, d_bstiles, d_btiles, d_mdtiles, d_tsum, d_gscan, d_toff};
+    void* ptrs[] = {d_boxes, d_bsegs, d_bstiles, d_btiles, d_mdtiles, d_vtiles, d_tsum, d_gscan, d_toff};
     for (void* q : ptrs)
       if (q) cudaFree(q);
     for (int v = 0; v < NVAR; ++v) {
@@ -368,8 +374,9 @@ struct Engine {
       n_spans[v] = 0;
     }
     d_boxes = nullptr; d_bsegs = nullptr; d_bstiles = nullptr; d_btiles = nullptr;
-    d_mdtiles = nullptr; d_tsum = nullptr; d_gscan = nullptr; d_toff = nullptr;
+    d_mdtiles = nullptr; d_vtiles = nullptr; d_tsum = nullptr; d_gscan = nullptr; d_toff = nullptr;
     n_records = 0;
+    n_vtiles = 0;
   }
 
   void drop_graphs() {
@@ -459,7 +466,7 @@ struct Engine {
     tables_ok = true;
     if (live.empty()) return MPCD_OK;
     std::vector<BoxDev> rec;
-    std::vector<int2> sp[NVAR], bst, bt, mt;
+    std::vector<int2> sp[NVAR], bst, bt, mt, vt;
     std::vector<ScanSeg> bseg;
     any_beads = false;
     wca_substeps = 0;
@@ -483,13 +490,15 @@ struct Engine {
       int variant = (d.thermostat ? 1 : 0) | ((d.walls || d.nbead > 0) ? 2 : 0) | (at ? 16 : 0) |
                     (d.angular ? 32 : 0);
       const bool warp_ang = mixed && !at && d.nbead == 0;
+      if (on_srd(d) && d.walls) variant = 64 | 4 | (d.thermostat ? 1 : 0);
       if ((!d.angular || warp_ang) && !d.walls && d.K <= WARP_MAX_K &&
           std::max(d.n[0], std::max(d.n[1], d.n[2])) < (1 << 22)) {
         const bool force = d.g[0] != 0.0 || d.g[1] != 0.0 || d.g[2] != 0.0;
-        const bool reg = mixed && !at && !d.angular && d.K <= SRD_SLOTS;
-        variant = (reg ? 64 : 4) | (d.thermostat ? 1 : 0) | (force ? 2 : 0) |
+        variant = (on_srd(d) ? 64 : 4) | (d.thermostat ? 1 : 0) | (force ? 2 : 0) |
                   (d.nbead > 0 ? 8 : 0) | (at ? 16 : 0) | (d.angular ? 32 : 0);
       }
+      if (on_srd(d) && d.walls)
+        for (int i0 = 0; i0 < 2 * d.n[0] * d.n[1]; i0 += VIRT_CELLS) vt.push_back(make_int2((int)i, i0));
       for (int c0 = 0; c0 < d.ncells; c0 += BLOCK) sp[variant].push_back(make_int2((int)i, c0));
       if (d.nbead > 0) {
         any_beads = true;
@@ -518,6 +527,7 @@ struct Engine {
     if ((rc = up(bst, d_bstiles, &n_bstiles))) return rc;
     if ((rc = up(bt, d_btiles, &n_btiles))) return rc;
     if ((rc = up(mt, d_mdtiles, &n_mdtiles))) return rc;
+    if ((rc = up(vt, d_vtiles, &n_vtiles))) return rc;
     if (n_bstiles > 0) {
       CUDA_TRY(cudaMalloc(&d_tsum, sizeof(uint32_t) * n_bstiles));
       CUDA_TRY(cudaMalloc(&d_gscan, sizeof(unsigned long long) * n_bstiles));
@@ -532,7 +542,13 @@ struct Engine {
     return n < g ? std::max(n, 1) : g;
   }
 
-  // Cells per warp of the register kernel: as chosen by the tuner, else the
+  // Boxes that k_srd steps.
+  bool on_srd(const BoxDev& d) const {
+    return mixed && d.collision != RULE_AT && !d.angular && d.K <= SRD_SLOTS &&
+           std::max(d.n[0], std::max(d.n[1], d.n[2])) < (1 << 22);
+  }
+
+  // Cells per warp of k_srd: as chosen by the tuner, else the
   // most of 32, 16, 8 and 4 that still gives every SM SRD_MIN_WARPS warps.
   int srd_cpw() const {
     if (tuned_cpw) return tuned_cpw;
@@ -545,7 +561,7 @@ struct Engine {
 
   // Grid of the fused pass: tuned_grid 0 = the occupancy limit (blocks per
   // SM that fit), k > 0 = at most k blocks per SM, -1 = one block per span
-  // part (the register kernel takes a 256-cell span in parts).
+  // part (the k_srd takes a 256-cell span in parts).
   int tuned_grid = 0;
   int grid_of(int v, int mode) const {
     const int items = n_spans[v] * ((v & 64) ? srd_parts(srd_cpw()) : 1);
@@ -559,10 +575,14 @@ struct Engine {
       if (n_spans[v] == 0) continue;
       const int grid = grid_of(v, mode);
       const bool at = (v & 16) != 0;
-      if (v & 64)
-        launch_srd((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, mode, d_boxes, d_spans[v], n_spans[v],
+      if (v & 64) {
+        launch_srd((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, mode, d_boxes, d_spans[v], n_spans[v],
                    grid, srd_cpw(), d_err, stream);
-      else if ((v & 4) && mixed)
+        if ((v & 8) && mode != MODE_P)
+          launch_srd((v & 1) != 0, (v & 2) != 0, true, (v & 4) != 0, mode, d_boxes, d_spans[v],
+                     n_spans[v], grid_for(srd_bead_items(n_spans[v]), srd_bead_bps[mode][v & 7]), 32,
+                     d_err, stream);
+      } else if ((v & 4) && mixed)
         launch_cells_warp((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, (v & 32) != 0, mode,
                           d_boxes, d_spans[v], n_spans[v], grid, d_err, stream);
       else if (v & 4)
@@ -573,8 +593,10 @@ struct Engine {
     }
   }
 
-  // Solute: MD substeps and bead grouping for the step in the records.
+  // What the collision of the step in the records needs beside the solvent:
+  // virtual wall particles; solute MD substeps and bead grouping.
   void launch_beads() {
+    launch_virtual(d_boxes, d_vtiles, n_vtiles, stream);
     if (!any_beads) return;
     if (wca_substeps > 0)
       launch_wca_md(d_boxes, d_btiles, n_btiles, wca_substeps, d_err, stream);
@@ -872,6 +894,11 @@ struct Engine {
     if ((rc = alloc(b, d.ovf_n, 2))) return rc;
     CUDA_TRY(cudaMemsetAsync(d.ovf_n, 0, sizeof(uint32_t) * 2, stream));
     if ((rc = alloc(b, d.xcnt, (size_t)XBUCKETS))) return rc;
+    if (d.walls && on_srd(d)) {
+      const size_t cut = 2 * (size_t)d.n[0] * d.n[1];
+      if ((rc = alloc(b, d.virt_n, cut))) return rc;
+      if ((rc = alloc(b, d.virt_sum, 4 * cut))) return rc;
+    }
     if ((rc = alloc_bytes(b, b->stage_r, (size_t)nsol * 3 * es))) return rc;
     if ((rc = alloc_bytes(b, b->stage_v, (size_t)nsol * 3 * es))) return rc;
     if (nbead > 0) {

@@ -466,14 +466,16 @@ __device__ __forceinline__ int virtual_count(const BoxDev& B, unsigned long long
   return nv;
 }
 
+__device__ __forceinline__ double virtual_component(const BoxDev& B, unsigned long long t,
+                                                    uint32_t cell, int q, int k) {
+  const uint4 w = draw(B, PURPOSE_VIRT, cell, 1u + 3u * (uint32_t)q + (uint32_t)k, t);
+  const double U = unit53(w.x, w.y), U2 = unit53(w.z, w.w);
+  return B.sigma_virt * (sqrt(-2.0 * log(1.0 - U)) * cospi(2.0 * U2));
+}
 __device__ __forceinline__ void virtual_velocity(const BoxDev& B, unsigned long long t,
                                                  uint32_t cell, int q, double vv[3]) {
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const uint4 w = draw(B, PURPOSE_VIRT, cell, 1u + 3u * (uint32_t)q + (uint32_t)k, t);
-    const double U = unit53(w.x, w.y), U2 = unit53(w.z, w.w);
-    vv[k] = B.sigma_virt * (sqrt(-2.0 * log(1.0 - U)) * cospi(2.0 * U2));
-  }
+  for (int k = 0; k < 3; ++k) vv[k] = virtual_component(B, t, cell, q, k);
 }
 
 // ---------------------------------------------------------------------------

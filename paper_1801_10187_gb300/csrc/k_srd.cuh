@@ -2,8 +2,8 @@
 // Eqs. stream, srd and thermo; Sec. 3.4 cell list; Sec. 3.5 cell properties;
 // Sec. 3.6 rotation and thermostat, algorithm "SRD collision rule").
 //
-// For periodic SRD boxes (body force, thermostat and solute beads allowed)
-// whose rows hold at most SRD_SLOTS records; modes, records and results are
+// For SRD boxes (body force, thermostat, and solute beads or channel walls
+// allowed) whose rows hold at most SRD_SLOTS records; modes, records and results are
 // those of k_cells_warp.  A warp owns cpw consecutive cells (32, or 16, 8 or 4
 // on small boxes) and takes them in sub-tiles of at most subc cells with at
 // most SRD_SLOTS members between them.  A map in shared memory gives each
@@ -18,6 +18,16 @@
 //            registers and written straight to their rows with one 32-byte store;
 //            a chunk's slot requests (one atomic for the lanes of a window bound
 //            for one cell) are all out before its first record is stored
+//
+// Channel walls (WALLS): the virtual particles that fill up the cells a wall cuts
+// enter a cell's sums as their number and exact totals, which k_virtual
+// (k_step.cu) has left in the box for the pending step; a particle that would
+// cross a wall bounces back.  k_cells draws them inside the cell's one thread.
+//
+// Solute boxes take two launches in modes F and C: one over the bead groups
+// without beads, one (BEADS) over those with.  In one launch the bead code's
+// registers cost every cell: 2.69 ms a step at 7.8 10^7 particles with 2000 chains
+// and the thermostat, against 2.14 ms for the same box without beads.
 //
 // What bounds it: neither DRAM (44 % of its peak at 10^7 particles) nor the
 // issue slots (53 %) nor the L1 pipe (63 %), but the chain count -> stage ->
@@ -62,7 +72,7 @@ constexpr int SWARPS = SB / 32;
 // Parameters of the box, shared by the block.
 struct SrdBox {
   float dt, ca, sa, omc, m;
-  float L[3], hg[3], gdt[3];
+  float L[3], hg[3], gdt[3], g[2];
   // binning under the next grid shift s: floor(x - s) = floor(x) + bias +
   // [frac(x) >= thr], and the one index outside the grid is out, for in
   float thr[3];
@@ -74,7 +84,8 @@ struct SrdBox {
   RecF* ovf_out;
   uint32_t* ovf_cell_out;
   uint32_t* ovf_n_out;
-  int ovf_cap, pad;
+  int ovf_cap;
+  int zb;  // walls: the bottom layer that the wall can cut in the collision step, -1: none
 };
 
 // Shared memory of a warp: sv[SRD_SLOTS], sr[SRD_SLOTS], map[SRD_SLOTS], then this.
@@ -113,8 +124,8 @@ __device__ __forceinline__ void split_bits(float x, unsigned& th, unsigned& tl) 
 
 }  // namespace
 
-template <bool THERMO, int MODE, bool FORCE, bool BEADS>
-__global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
+template <bool THERMO, int MODE, bool FORCE, bool BEADS, bool WALLS>
+__global__ void __launch_bounds__(SB, BEADS ? 6 : 7) k_srd(const BoxDev* __restrict__ boxes,
                                                const int2* __restrict__ spans, int nspans,
                                                int cpw, int* err) {
   constexpr int SW = THERMO ? 1 : 2;  // windows of 32 members per chunk
@@ -128,12 +139,16 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
   SrdWarp& W = *reinterpret_cast<SrdWarp*>(wp + (size_t)SRD_SLOTS * 34);
   SrdThermo& TS = *reinterpret_cast<SrdThermo*>(&W + 1);
   SrdBeads& BS = *reinterpret_cast<SrdBeads*>(wp + (size_t)SRD_SLOTS * 34 + sizeof(SrdWarp) + (THERMO ? sizeof(SrdThermo) : 0));
-  const int parts = BLOCK / (SWARPS * cpw);  // blocks' work per 256-cell span
+  // a block's work: a part of a 256-cell span (its warps next to each other), or,
+  // with beads, SWARPS spans, one to a warp
+  const int parts = BEADS ? 1 : BLOCK / (SWARPS * cpw);
+  const int items = BEADS ? (nspans + SWARPS - 1) / SWARPS : nspans * parts;
   int box_of_params = -1;
   const unsigned lt = (1u << lane) - 1u;
-  for (int it = blockIdx.x; it < nspans * parts; it += gridDim.x) {
+  for (int it = blockIdx.x; it < items; it += gridDim.x) {
     const int sp = it / parts, part = it - sp * parts;
-    const int2 tt = spans[sp];
+    // (with beads there is one box: a warp without a span takes the last's box)
+    const int2 tt = spans[BEADS ? min(it * SWARPS + wid, nspans - 1) : sp];
     const BoxDev& B = boxes[tt.x];
     if (tt.x != box_of_params) {  // block-uniform
       __syncthreads();
@@ -151,10 +166,18 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
           H.bias[q] = (s < 0 ? 0 : -1) - 0x4B000000;
           H.out[q] = s < 0 ? B.n[q] : -1;
           H.in[q] = s < 0 ? 0 : B.n[q] - 1;
+          if (WALLS && q == 2) H.bias[q] += 1;  // layers 0 .. n_z + 1, no wrap
         }
       } else if (threadIdx.x == 32) {
         H.dt = B.dt_f; H.ca = B.ca_f; H.sa = B.sa_f; H.omc = B.omc_f; H.m = B.m_f;
         H.K = B.K;
+        if (WALLS) {
+          H.g[0] = B.g_f[0];
+          H.g[1] = B.g_f[1];
+          long long S[3];
+          shift_units(B, B.step, S);
+          H.zb = S[2] > 0 ? 0 : S[2] < 0 ? 1 : -1;
+        }
         const int out = B.cur ^ 1;
         H.rows_cur = (RecF*)B.rows[B.cur];
         H.rows_out = (RecF*)B.rows[out];
@@ -167,8 +190,22 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
       __syncthreads();
       box_of_params = tt.x;
     }
-    const int c0 = tt.y + (part * SWARPS + wid) * cpw;
-    if (c0 >= B.ncells) continue;  // warp-uniform
+    // Solute boxes: the groups of 32 cells that hold beads are left to a second
+    // launch (BEADS), which takes only them; so the bead code and its registers
+    // weigh on no other cell.
+    unsigned groups = 1u;
+    if (BEADS) {
+      const int g = tt.y / BEAD_TILE + lane;
+      groups = __ballot_sync(FULL, it * SWARPS + wid < nspans && lane < BLOCK / BEAD_TILE &&
+                                       g < B.nctiles && B.bstart[g + 1] != B.bstart[g]);
+    }
+    for (; groups; groups &= groups - 1) {
+    const int c0 = BEADS ? tt.y + BEAD_TILE * (__ffs(groups) - 1) : tt.y + (part * SWARPS + wid) * cpw;
+    if (c0 >= B.ncells) break;  // warp-uniform
+    if (!BEADS && MODE != MODE_P && B.nbead > 0) {
+      const int g = c0 / BEAD_TILE;
+      if (B.bstart[g + 1] != B.bstart[g]) break;
+    }
     const int K = H.K;
     uint32_t n = 0u;
     if (lane < cpw && c0 + lane < B.ncells) {
@@ -176,11 +213,10 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
       n = *cn;
       if (MODE != MODE_C && n) *cn = 0u;  // this set is written two steps on
     }
-    int gb0 = 0, gnb = 0;  // the beads of the 32-cell bead group, loaded with the counts
-    if (BEADS && MODE != MODE_P) {
-      const int g = c0 / B.tc;
-      gb0 = (int)B.bstart[g];
-      gnb = (int)B.bstart[g + 1] - gb0;
+    int gb0 = 0, gnb = 0;  // the beads of the group
+    if (BEADS) {
+      gb0 = (int)B.bstart[c0 / BEAD_TILE];
+      gnb = (int)B.bstart[c0 / BEAD_TILE + 1] - gb0;
     }
     const int nrow = (int)n < K ? (int)n : K;
     int incl = nrow;
@@ -190,7 +226,7 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
       if (lane >= d) incl += y;
     }
     const int N = __shfl_sync(FULL, incl, 31);
-    if (N == 0 && gnb == 0) continue;
+    if (N == 0 && gnb == 0) continue;  // (the next group)
     RecF* rows = H.rows_cur + (size_t)c0 * K;
     // f(record) for the members of cell c in the overflow list (rare)
     auto for_overflow = [&](int c, auto&& f) {
@@ -210,7 +246,8 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
         }
       }
     };
-    int nb = 0;
+    int nb = 0;     // beads of this lane's cell; with walls its virtual particles
+    int virt = -1;  // with walls: their place in the box's sums
     const int subc = min(B.subc, cpw);  // most cells per sub-tile, a power of two
     const int plog = __clz(subc) - 26;  // 2^plog = 32 / subc lanes add up a cell
 
@@ -258,6 +295,15 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
           __syncwarp();
           nb = BS.nb[lane];
         }
+        if (WALLS && n > 0 && H.zb >= 0) {  // virtual particles of this lane's cell
+          const int nxy = B.n[0] * B.n[1];
+          const int cz = (c0 + lane) / nxy;
+          const int side = cz == H.zb ? 0 : cz == H.zb + B.n[2] ? 1 : -1;
+          if (side >= 0) {
+            virt = side * nxy + (c0 + lane - cz * nxy);
+            nb = B.virt_n[virt];  // (walls exclude beads)
+          }
+        }
         // the per-cell draws need only the member count: the axis (Sec. 3.6)
         // and, with the thermostat, the accepted Gamma pair (d, v), E^ = d v kT
         if (n > 0 || nb > 0) {
@@ -281,7 +327,8 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
         const int cc = a + (lane >> plog), part = lane & ((1 << plog) - 1);
         const int src = cc < b ? cc : a;
         const int nC = __shfl_sync(FULL, (int)n, src), s0C = __shfl_sync(FULL, s0, src);
-        const int nbC = BEADS ? __shfl_sync(FULL, nb, src) : 0;
+        const int nbC = (BEADS || WALLS) ? __shfl_sync(FULL, nb, src) : 0;
+        const int virtC = WALLS ? __shfl_sync(FULL, virt, src) : -1;
         const int nrowC = cc < b ? min(nC, K) : 0;
         int slow = 0;  // beyond |v| < 2^10 (or NaN) the split fails: exact sums below
         unsigned hs[3] = {0u, 0u, 0u}, ls[3] = {0u, 0u, 0u};
@@ -368,13 +415,16 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
               else u[2] = c;
             }
           }
-          const bool bd = BEADS && gnb > 0;
+          const bool bd = BEADS && gnb > 0, vp = WALLS && nbC > 0;
+          const long long* vs = vp ? B.virt_sum + 4 * (size_t)virtC : nullptr;
           float M = H.m * small_to_float(nC);
           if (BEADS) M = M + (small_to_float(nbC) * B.Mb_f + 0.0f * H.m);
+          if (WALLS) M = M + (0.0f * B.Mb_f + small_to_float(nbC) * H.m);
 #pragma unroll
           for (int q = 0; q < 3; ++q) {
             float P = H.m * u[q];
             if (BEADS) P = P + (bd ? i64_to_float((long long)BS.X[q][cc]) : 0.0f);
+            if (WALLS) P = P + (vp ? i64_to_float(vs[q]) : 0.0f);
             u[q] = (P * 0x1p-32f) / M;
           }
           float xi = 1.0f;
@@ -385,8 +435,13 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
 #pragma unroll
               for (int q = 0; q < 3; ++q) X[q] = (long long)BS.X[q][cc];
             }
+            if (vp) {
+#pragma unroll
+              for (int q = 0; q < 3; ++q) X[q] = vs[q];
+            }
             double Mt;
-            const double Ep = mixed_ek_mt(B, nC, nbC, 0, Qt, S2, X, bd ? (long long)BS.E[cc] : 0ll, Mt);
+            const double Ep = mixed_ek_mt(B, nC, WALLS ? 0 : nbC, WALLS ? nbC : 0, Qt, S2, X,
+                                          bd ? (long long)BS.E[cc] : vp ? vs[3] : 0ll, Mt);
             const float2 dv = TS.gdv[cc];
             if (!thermo_xi_from_draw(B, dv.x, dv.y, Ep, Mt, xi)) atomicOr(err, ERR_GAMMA_CAP);
           }
@@ -429,6 +484,31 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
         if constexpr (MODE == MODE_C) {
           return 0u;
         } else {
+        bool hit = false;
+        if (WALLS) {  // no-slip bounce-back at z = 0 and z = n_z (stream_one)
+          const float Lz = H.L[2], zn = fmaf(w[2], H.dt, x[2]);
+          hit = !(zn >= 0.0f && zn < Lz);
+          if (hit) {
+            const float wall = (zn < 0.0f) ? 0.0f : Lz;
+            float tau = (wall - x[2]) / w[2];
+            if (!(tau >= 0.0f)) tau = 0.0f;
+            if (tau > H.dt) tau = H.dt;
+            const float rem = H.dt - tau;
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+              x[k] = fmaf(w[k], tau, x[k]) + ((0.5f * H.g[k]) * tau) * tau;
+              w[k] = -(w[k] + H.g[k] * tau);
+              x[k] = fmaf(w[k], rem, x[k]) + ((0.5f * H.g[k]) * rem) * rem;
+              w[k] = w[k] + H.g[k] * rem;
+            }
+            w[2] = -w[2];
+            float z = fmaf(w[2], rem, wall);
+            if (z < 0.0f) z = 0.0f;
+            if (z >= Lz) z = nextafterf(Lz, 0.0f);
+            x[2] = z;
+          }
+        }
+        if (!hit)
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
           x[q] = fmaf(w[q], H.dt, x[q]);
@@ -441,16 +521,16 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
         // is outside do not
         if (!(__float_as_uint(x[0]) < __float_as_uint(H.L[0]) &&
               __float_as_uint(x[1]) < __float_as_uint(H.L[1]) &&
-              __float_as_uint(x[2]) < __float_as_uint(H.L[2]))) {
+              (WALLS || __float_as_uint(x[2]) < __float_as_uint(H.L[2])))) {
           bool far = false;
 #pragma unroll
-          for (int q = 0; q < 3; ++q) {
+          for (int q = 0; q < (WALLS ? 2 : 3); ++q) {
             x[q] = wrap_fast(x[q] + 0.0f, H.L[q]);
             far |= !(x[q] >= 0.0f && x[q] < H.L[q]);
           }
           if (far) {  // more than one box length out, or non-finite (one copy: it is cold)
 #pragma unroll 1
-            for (int q = 0; q < 3; ++q) {
+            for (int q = 0; q < (WALLS ? 2 : 3); ++q) {
               float y = q == 0 ? x[0] : q == 1 ? x[1] : x[2];
               y = wrap(y, H.L[q]);
               if (q == 0) x[0] = y;
@@ -465,7 +545,7 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
           const float tf = __fadd_rd(x[q], 8388608.0f);  // 2^23 + floor(x)
           const float f = __fsub_rn(x[q], __fsub_rn(tf, 8388608.0f));
           const int i = __float_as_int(tf) + H.bias[q] + (f >= H.thr[q] ? 1 : 0);
-          c[q] = i == H.out[q] ? H.in[q] : i;
+          c[q] = (WALLS && q == 2) ? min(max(i, 0), H.n[2] + 1) : i == H.out[q] ? H.in[q] : i;
         }
         return (uint32_t)(c[0] + H.n[0] * (c[1] + H.n[1] * c[2]));
         }
@@ -542,6 +622,7 @@ __global__ void __launch_bounds__(SB, 7) k_srd(const BoxDev* __restrict__ boxes,
           else emit(x, w, tg, c, atomicAdd(&H.cnt_out[c], 1u));
         });
       a = b;
+    }
     }
   }
 }

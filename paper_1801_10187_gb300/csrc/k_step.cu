@@ -6,6 +6,7 @@
 // (box, first index) tiles, so one launch serves every box of a batch.
 #include <type_traits>
 
+#include "dev_collide.cuh"
 #include "dev_stream.cuh"
 #include "kernels.h"
 #include "mpcd_internal.cuh"
@@ -267,6 +268,82 @@ __global__ void k_bead_scatter(const BoxDev* __restrict__ boxes, const int2* __r
       B.bgv[3 * slot + 2] = B.svel[3 * b + 2];
     }
   }
+}
+
+// ---------------------------------------------------------------------------
+// Virtual wall particles of the pending step (mixed model): for every cell of
+// the two layers a wall can cut, their number and the exact sums of their
+// momenta and kinetic terms, as the cell's own thread adds them in k_cells.
+// A velocity component costs a double log, square root and cospi: a hundred
+// dependent instructions on the FP64 pipe, a few microseconds however few are
+// drawn.  So a block takes only VIRT_CELLS cells and gives every component a
+// thread of its own (about 120 components at density 10): one such chain per
+// block, and blocks on every SM.  (One thread a particle, 256 cells a block:
+// 150 us a step for 50 x 50 cells.)
+// ---------------------------------------------------------------------------
+namespace {
+constexpr int VT = 128;           // threads per block
+constexpr int VPART = VT / 3;     // particles per round
+}  // namespace
+
+__global__ void __launch_bounds__(VT) k_virtual(const BoxDev* __restrict__ boxes,
+                                                const int2* __restrict__ tiles) {
+  __shared__ int first[VIRT_CELLS + 1];  // first particle of each cell; the last: all
+  __shared__ double v[3][VPART];
+  const int2 tt = tiles[blockIdx.x];
+  const BoxDev& B = boxes[tt.x];
+  const int t = threadIdx.x;
+  const int nxy = B.n[0] * B.n[1], items = min(VIRT_CELLS, 2 * nxy - tt.y);
+  long long S[3];
+  shift_units(B, B.step, S);
+  const int zb = S[2] > 0 ? 0 : 1;  // (S = 0: no cell is cut)
+  auto cell_of_item = [&](int i) {
+    const int side = tt.y + i >= nxy ? 1 : 0;
+    return (uint32_t)((zb + side * B.n[2]) * nxy + (tt.y + i - side * nxy));
+  };
+  if (t < 32) {
+    int nv = 0;
+    if (t < items && S[2] != 0)
+      nv = virtual_count(B, B.step, cell_of_item(t), (double)S[2] * 0x1p-32);
+    int incl = nv;
+#pragma unroll
+    for (int d = 1; d < VIRT_CELLS; d <<= 1) {
+      const int y = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+      if (t >= d) incl += y;
+    }
+    if (t < VIRT_CELLS) first[t + 1] = incl;
+    if (t == 0) first[0] = 0;
+    if (t < items) B.virt_n[tt.y + t] = nv;
+  }
+  __syncthreads();
+  const int total = first[VIRT_CELLS];
+  long long sum = 0;  // thread 4 i + k: word k of cell i
+  for (int p0 = 0; p0 < total; p0 += VPART) {
+    const int np = min(VPART, total - p0);
+    if (t < 3 * np) {
+      const int j = p0 + t / 3;
+      int i = 0;
+#pragma unroll
+      for (int k = 1; k < VIRT_CELLS; ++k)
+        if (j >= first[k]) i = k;
+      v[t % 3][t / 3] = virtual_component(B, B.step, cell_of_item(i), j - first[i], t % 3);
+    }
+    __syncthreads();
+    if (t < 4 * items) {
+      const int i = t >> 2, k = t & 3;
+      for (int j = max(first[i] - p0, 0); j < min(first[i + 1] - p0, np); ++j)
+        sum += k < 3 ? __double2ll_rn((B.m * v[k][j]) * 4294967296.0)
+                     : __double2ll_rn((B.m * (v[0][j] * v[0][j] + v[1][j] * v[1][j] +
+                                              v[2][j] * v[2][j])) * 4294967296.0);
+    }
+    __syncthreads();
+  }
+  if (t < 4 * items) B.virt_sum[4 * (size_t)tt.y + t] = sum;
+}
+
+void launch_virtual(const BoxDev* boxes, const int2* tiles, int ntiles, cudaStream_t s) {
+  if (ntiles <= 0) return;
+  k_virtual<<<ntiles, VT, 0, s>>>(boxes, tiles);
 }
 
 // ---------------------------------------------------------------------------

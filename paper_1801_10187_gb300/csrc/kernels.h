@@ -33,14 +33,17 @@ int cells_warp_blocks_per_sm(bool thermo, bool force, bool beads, bool at, bool 
 void launch_cells_warp(bool thermo, bool force, bool beads, bool at, bool ang, int mode,
                        const BoxDev* boxes, const int2* spans, int nspans, int grid, int* err,
                        cudaStream_t s);
-// The same step for periodic mixed SRD boxes with rows of at most SRD_SLOTS
-// records, members held in registers (k_srd.cu).  cpw: cells per warp (32, 16,
+// The same step for mixed SRD boxes (walls: with channel walls, then without
+// beads) with rows of at most SRD_SLOTS records (k_srd.cu).  cpw: cells per warp (32, 16,
 // 8 or 4); a 256-cell span is then taken in srd_parts(cpw) parts, one block
-// each: grid sizes count parts.  SRD_MIN_WARPS: see srd_cpw() in capi.cu.
+// each: grid sizes count parts.  A solute box takes a launch without beads, over
+// the bead groups that hold none, and one with (cpw 32), over the others; mode P
+// only the first.  SRD_MIN_WARPS: see srd_cpw() in capi.cu.
 constexpr int SRD_MIN_WARPS = 16;
-int srd_blocks_per_sm(bool thermo, bool force, bool beads, int mode);
+int srd_blocks_per_sm(bool thermo, bool force, bool beads, bool walls, int mode);
 int srd_parts(int cpw);
-void launch_srd(bool thermo, bool force, bool beads, int mode, const BoxDev* boxes,
+int srd_bead_items(int nspans);  // blocks' work of the bead launch
+void launch_srd(bool thermo, bool force, bool beads, bool walls, int mode, const BoxDev* boxes,
                 const int2* spans, int nspans, int grid, int cpw, int* err, cudaStream_t s);
 // The FP64 model's counterpart (k_cells_warp_d.cu), same conditions.
 int cells_warpd_blocks_per_sm(bool thermo, bool force, bool beads, bool at, int mode);
@@ -74,6 +77,11 @@ void launch_bead_scatter(const BoxDev* boxes, const int2* tiles, int ntiles, cud
 // flip: the output set becomes current (after modes P and F); advance: step += 1
 // (after modes F and C).
 void launch_after_pass(BoxDev* boxes, int nboxes, bool flip, bool advance, cudaStream_t s);
+
+// Virtual wall particles of the pending step, for the boxes of the tiles (box,
+// first of VIRT_CELLS cells of its two wall-cut layers); mixed boxes on k_srd.
+constexpr int VIRT_CELLS = 8;
+void launch_virtual(const BoxDev* boxes, const int2* tiles, int ntiles, cudaStream_t s);
 
 // ---- observables (k_obs.cu) ----
 struct ObsCells {

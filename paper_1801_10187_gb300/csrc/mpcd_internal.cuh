@@ -96,6 +96,11 @@ struct BoxDev {
   void* ovf_rec[2];     // overflow records
   uint32_t* ovf_cell[2];
   uint32_t* ovf_n;      // two counters
+  // channel walls, mixed model: virtual particles of the pending step in the
+  // two layers a wall can cut, n_x n_y cells each: their number, exact sums of
+  // rne(m v 2^32) and of rne(m v^2 2^32) (four words a cell)
+  int32_t* virt_n;
+  long long* virt_sum;
   uint32_t* xcnt;       // records per tag bucket of a state read-out (XBUCKETS)
   // solute
   double* spos;
