@@ -78,7 +78,7 @@ size_t footprint_bytes(const mpcd_params& p, int64_t nsol, int64_t nbead) {
   b += 2 * (size_t)C * sizeof(uint32_t);                                  // counts
   b += 2 * (size_t)std::max<int64_t>(nsol, 1) * (rec_size(mixed) + 4);     // overflow lists
   b += (size_t)nsol * 6 * elem_size(mixed);                               // staging (r, v)
-  b += XBUCKETS * sizeof(uint32_t);                                       // read-out buckets
+  b += (size_t)xbuckets(mixed, nsol) * XCNT_STRIDE * sizeof(uint32_t);    // read-out buckets
   if (mixed && p.walls_z) b += 2 * (size_t)p.n[0] * p.n[1] * (4 * sizeof(long long) + 4);
   if (nbead > 0) {
     b += (size_t)nbead * (9 * sizeof(double) + 2 * sizeof(int32_t) + sizeof(uint64_t) +
@@ -352,6 +352,7 @@ struct Engine {
         if (cells_bps[m][v] < 1) cells_bps[m][v] = 1;
       }
     CUDA_TRY((cudaError_t)md_bin_prepare());
+    CUDA_TRY((cudaError_t)extract_prepare());
     CUDA_TRY(cudaMalloc(&d_err, sizeof(int)));
     CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), stream));
     CUDA_TRY(cudaMalloc(&d_partials, sizeof(double) * 4 * 4096));
@@ -893,7 +894,7 @@ struct Engine {
     }
     if ((rc = alloc(b, d.ovf_n, 2))) return rc;
     CUDA_TRY(cudaMemsetAsync(d.ovf_n, 0, sizeof(uint32_t) * 2, stream));
-    if ((rc = alloc(b, d.xcnt, (size_t)XBUCKETS))) return rc;
+    if ((rc = alloc(b, d.xcnt, (size_t)xbuckets(mixed, nsol) * XCNT_STRIDE))) return rc;
     if (d.walls && on_srd(d)) {
       const size_t cut = 2 * (size_t)d.n[0] * d.n[1];
       if ((rc = alloc(b, d.virt_n, cut))) return rc;

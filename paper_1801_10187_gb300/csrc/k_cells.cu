@@ -21,6 +21,8 @@
 // at): a second pass over the cell's members forms dL = sum m r_c x (v - v')
 // and the inertia tensor about the cell's centre of mass, and every member
 // then receives omega x r_c with Pi omega = dL.
+#include <algorithm>
+
 #include "dev_angular.cuh"
 #include "dev_collide.cuh"
 #include "dev_rows.cuh"
@@ -357,26 +359,25 @@ __global__ void k_load(const BoxDev* __restrict__ box, const real_t<MIXED>* __re
 // receives each particle's cell.  The outputs are a scatter by tag: 12-byte
 // (FP64: 24-byte) writes all over two arrays.
 //
-// Outputs that fit L2 (EXTRACT_DIRECT bytes) are scattered straight from the
-// rows.  Larger ones would leave L2 as partial sectors, each merged in DRAM
-// (10^7 mixed particles: 0.74 ms for 240 MB), so the records first go, whole
-// sectors at a time, to buckets of consecutive tags, and then bucket by bucket
-// to the outputs, whose sectors fill up in L2.  The bucket of a tag is tag >>
-// shift, it holds exactly the records of its tags, and so buckets lie end to end
-// in [0, nsol) of the row set that is not in use between steps.
+// Small outputs (EXTRACT_DIRECT bytes) are scattered straight from the rows.
+// From larger ones that costs six scattered 4-byte stores a particle, and beyond
+// L2 partial sectors merged in DRAM as well (10^7 mixed particles: 0.74 ms).
+// There the records first move, whole, to buckets of XBUCKET consecutive tags,
+// and then a block gathers each bucket's outputs in shared memory and writes
+// them out in order.  A bucket holds exactly the records of its tags, so the
+// buckets lie end to end in [0, nsol) of the row set that is not in use between
+// steps.  (10^7 particles: 0.30 ms; buckets of 2^17 tags scattered
+// within L2 instead: 0.68 ms.)
 //
-// f(record, cell) for every record of 32 consecutive cells of the warp: eight
-// lanes a cell, four cells at a time.
+// f(act, record, cell) with every record of four consecutive cells, eight lanes a
+// cell; called by the whole warp together, act marking the lanes with a record.
 template <class R, class F>
 __device__ __forceinline__ void for_rows(const BoxDev& B, int cur, int c0, F&& f) {
-  const int lane = threadIdx.x & 31, K = B.K;
-  const int nmine = c0 + lane < B.ncells ? min((int)B.cnt[cur][c0 + lane], K) : 0;
-  for (int q = 0; q < 32; q += 4) {
-    const int c = q + (lane >> 3);
-    const int n = __shfl_sync(0xFFFFFFFFu, nmine, c);
-    const R* row = ((const R*)B.rows[cur]) + (size_t)(c0 + c) * K;
-    for (int k = lane & 7; k < n; k += 8) f(row + k, c0 + c);
-  }
+  const int lane = threadIdx.x & 31, c = c0 + (lane >> 3), K = B.K;
+  const int n = c < B.ncells ? min((int)B.cnt[cur][c], K) : 0;
+  const R* row = ((const R*)B.rows[cur]) + (size_t)c * K;
+  const int most = __reduce_max_sync(0xFFFFFFFFu, n);
+  for (int k = lane & 7; k - (lane & 7) < most; k += 8) f(k < n, row + k, c);
 }
 
 template <bool MIXED>
@@ -402,9 +403,10 @@ __global__ void __launch_bounds__(BLOCK) k_extract(const BoxDev* __restrict__ bo
   using R = rec_t<MIXED>;
   const BoxDev& B = *box;
   const int cur = B.cur;
-  for (int c0 = (blockIdx.x * BLOCK + threadIdx.x) & ~31; c0 < B.ncells; c0 += gridDim.x * BLOCK)
-    for_rows<R>(B, cur, c0, [&](const R* p, int cell) {
-      put_particle<MIXED>(p, pos, vel, cell_out, cell);
+  for (int c0 = (blockIdx.x * BLOCK + threadIdx.x) / 32 * 4; c0 < B.ncells;
+       c0 += gridDim.x * (BLOCK / 8))
+    for_rows<R>(B, cur, c0, [&](bool act, const R* p, int cell) {
+      if (act) put_particle<MIXED>(p, pos, vel, cell_out, cell);
     });
   const uint32_t novf = min(B.ovf_n[cur], (uint32_t)B.ovf_cap);
   for (uint32_t j = blockIdx.x * BLOCK + threadIdx.x; j < novf; j += gridDim.x * BLOCK)
@@ -432,56 +434,71 @@ __device__ __forceinline__ void move_rec(RecD* d, const RecD* p, int cell) {
 __device__ __forceinline__ int noted_cell(const RecF* p) { return (int)p->pad; }
 __device__ __forceinline__ int noted_cell(const RecD* p) { return (int)p->pad; }
 
-// Records into buckets of tags: a block takes 256 cells (then 2048 overflow
-// records at a time), counts its records per bucket in shared memory, reserves
-// their places with one global atomic a bucket, and moves them.
+// Records into buckets of tags; the lanes of a warp bound for one bucket share an
+// atomic and take consecutive places.
 template <bool MIXED>
-__global__ void __launch_bounds__(BLOCK) k_bucket(const BoxDev* __restrict__ box, int shift, int nb) {
+__global__ void __launch_bounds__(BLOCK) k_bucket(const BoxDev* __restrict__ box) {
   using R = rec_t<MIXED>;
-  extern __shared__ uint32_t hist[];  // nb counts, then nb first places
-  uint32_t* first = hist + nb;
+  constexpr int SHIFT = xbucket_shift(MIXED);
   const BoxDev& B = *box;
-  const int cur = B.cur;
+  const int cur = B.cur, lane = threadIdx.x & 31;
   R* out = (R*)B.rows[cur ^ 1];
+  auto place = [&](bool act, const R* p, int cell) {
+    const uint32_t bucket = act ? tag_of(p) >> SHIFT : 0xFFFFFFFFu;
+    const unsigned peers = __match_any_sync(0xFFFFFFFFu, bucket);
+    const int leader = __ffs(peers) - 1;
+    uint32_t at = 0u;
+    if (act && lane == leader) at = atomicAdd(&B.xcnt[(size_t)bucket * XCNT_STRIDE], (uint32_t)__popc(peers));
+    at = __shfl_sync(0xFFFFFFFFu, at, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+    if (act) move_rec(out + (((size_t)bucket << SHIFT) + at), p, cell);
+  };
+  for (int c0 = (blockIdx.x * BLOCK + threadIdx.x) / 32 * 4; c0 < B.ncells;
+       c0 += gridDim.x * (BLOCK / 8))
+    for_rows<R>(B, cur, c0, place);
   const uint32_t novf = min(B.ovf_n[cur], (uint32_t)B.ovf_cap);
-  const int cell_blocks = (B.ncells + BLOCK - 1) / BLOCK;
-  const int blocks = cell_blocks + (int)((novf + 8 * BLOCK - 1) / (8 * BLOCK));
-  for (int it = blockIdx.x; it < blocks; it += gridDim.x) {
-    auto each = [&](auto&& f) {
-      if (it < cell_blocks) {
-        for_rows<R>(B, cur, it * BLOCK + (int)(threadIdx.x & ~31u), f);
-      } else {
-        const uint32_t j0 = (uint32_t)(it - cell_blocks) * 8 * BLOCK;
-        for (uint32_t j = j0 + threadIdx.x; j < min(j0 + 8 * BLOCK, novf); j += BLOCK)
-          f(((const R*)B.ovf_rec[cur]) + j, (int)B.ovf_cell[cur][j]);
-      }
-    };
-    for (int b = threadIdx.x; b < nb; b += BLOCK) hist[b] = 0u;
-    __syncthreads();
-    each([&](const R* p, int) { atomicAdd(&hist[tag_of(p) >> shift], 1u); });
-    __syncthreads();
-    for (int b = threadIdx.x; b < nb; b += BLOCK) {
-      const uint32_t n = hist[b];
-      first[b] = ((uint32_t)b << shift) + (n ? atomicAdd(&B.xcnt[b], n) : 0u);
-    }
-    __syncthreads();
-    each([&](const R* p, int cell) {
-      move_rec(out + atomicAdd(&first[tag_of(p) >> shift], 1u), p, cell);
-    });
-    __syncthreads();  // before the counts are cleared
+  for (uint32_t j0 = blockIdx.x * BLOCK + (threadIdx.x & ~31u); j0 < novf; j0 += gridDim.x * BLOCK) {
+    const uint32_t j = j0 + lane;
+    place(j < novf, ((const R*)B.ovf_rec[cur]) + j, j < novf ? (int)B.ovf_cell[cur][j] : 0);
   }
 }
 
+// A bucket's outputs gathered in shared memory and written in order.
+constexpr int UT = 512;  // threads per block
 template <bool MIXED>
-__global__ void __launch_bounds__(BLOCK) k_unbucket(const BoxDev* __restrict__ box,
-                                                    real_t<MIXED>* __restrict__ pos,
-                                                    real_t<MIXED>* __restrict__ vel,
-                                                    int32_t* __restrict__ cell_out) {
+__global__ void __launch_bounds__(UT) k_unbucket(const BoxDev* __restrict__ box,
+                                                 real_t<MIXED>* __restrict__ pos,
+                                                 real_t<MIXED>* __restrict__ vel,
+                                                 int32_t* __restrict__ cell_out) {
+  using T = real_t<MIXED>;
   using R = rec_t<MIXED>;
+  constexpr int N = 1 << xbucket_shift(MIXED);
+  extern __shared__ __align__(16) unsigned char xs_[];
+  T* sr = reinterpret_cast<T*>(xs_);
+  T* sv = sr + 3 * N;
+  int32_t* sc = reinterpret_cast<int32_t*>(sv + 3 * N);
   const BoxDev& B = *box;
-  const R* in = (const R*)B.rows[B.cur ^ 1];
-  for (int i = blockIdx.x * BLOCK + threadIdx.x; i < B.nsol; i += gridDim.x * BLOCK)
-    put_particle<MIXED>(in + i, pos, vel, cell_out, noted_cell(in + i));
+  const size_t i0 = (size_t)blockIdx.x * N;
+  const int n = (int)min((size_t)N, (size_t)B.nsol - i0);
+  const R* in = (const R*)B.rows[B.cur ^ 1] + i0;
+  for (int i = threadIdx.x; i < n; i += UT) {
+    T r[3], v[3];
+    uint32_t tag;
+    load_rec(in + i, r, v, tag);
+    const int j = (int)(tag & (N - 1));
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      sr[3 * j + q] = r[q];
+      sv[3 * j + q] = v[q];
+    }
+    if (cell_out) sc[j] = noted_cell(in + i);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < 3 * n; i += UT) {
+    pos[3 * i0 + i] = sr[i];
+    vel[3 * i0 + i] = sv[i];
+  }
+  if (cell_out)
+    for (int i = threadIdx.x; i < n; i += UT) cell_out[i0 + i] = sc[i];
 }
 
 // ---------------------------------------------------------------------------
@@ -552,17 +569,26 @@ void launch_load(bool mixed, const BoxDev* box, const void* pos, const void* vel
 template <bool MIXED>
 static void extract(const BoxDev* box, real_t<MIXED>* pos, real_t<MIXED>* vel, int32_t* cell_out,
                     int ncells, int nsol, uint32_t* xcnt, cudaStream_t s) {
+  const int warps = (ncells + 3) / 4;  // four cells each
+  const int g = std::min(std::max((warps + BLOCK / 32 - 1) / (BLOCK / 32), 1), 65536);
   if ((size_t)nsol * 6 * sizeof(real_t<MIXED>) <= EXTRACT_DIRECT) {
-    k_extract<MIXED><<<grid_for_n(ncells), BLOCK, 0, s>>>(box, pos, vel, cell_out);
+    k_extract<MIXED><<<g, BLOCK, 0, s>>>(box, pos, vel, cell_out);
     return;
   }
-  // buckets of 2^17 tags (3.1 MB of outputs, 6.3 in FP64), at most XBUCKETS
-  int shift = 17;
-  while ((((int64_t)nsol - 1) >> shift) + 1 > XBUCKETS) ++shift;
-  const int nb = (int)((((int64_t)nsol - 1) >> shift) + 1);
-  cudaMemsetAsync(xcnt, 0, sizeof(uint32_t) * XBUCKETS, s);
-  k_bucket<MIXED><<<grid_for_n(ncells), BLOCK, 2 * sizeof(uint32_t) * nb, s>>>(box, shift, nb);
-  k_unbucket<MIXED><<<grid_for_n(nsol), BLOCK, 0, s>>>(box, pos, vel, cell_out);
+  constexpr int N = 1 << xbucket_shift(MIXED);
+  const int nb = xbuckets(MIXED, nsol);
+  const size_t smem = (size_t)N * (6 * sizeof(real_t<MIXED>) + (cell_out ? sizeof(int32_t) : 0));
+  cudaMemsetAsync(xcnt, 0, sizeof(uint32_t) * XCNT_STRIDE * nb, s);
+  k_bucket<MIXED><<<g, BLOCK, 0, s>>>(box);
+  k_unbucket<MIXED><<<nb, UT, smem, s>>>(box, pos, vel, cell_out);
+}
+
+int extract_prepare() {
+  const int most = (1 << xbucket_shift(true)) * (6 * (int)sizeof(float) + (int)sizeof(int32_t));
+  const int mostd = (1 << xbucket_shift(false)) * (6 * (int)sizeof(double) + (int)sizeof(int32_t));
+  const cudaError_t e = cudaFuncSetAttribute(k_unbucket<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+  if (e != cudaSuccess) return (int)e;
+  return (int)cudaFuncSetAttribute(k_unbucket<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mostd);
 }
 
 void launch_extract(bool mixed, const BoxDev* box, void* pos, void* vel, int32_t* cell_out,

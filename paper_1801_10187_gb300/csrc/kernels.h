@@ -56,8 +56,16 @@ void launch_load(bool mixed, const BoxDev* box, const void* pos, const void* vel
 // Current state (of a box at rest between steps) into device arrays in input
 // order (cell_out optional); large outputs go through the row set not in use and
 // the box's xcnt.  Outputs up to EXTRACT_DIRECT bytes are scattered directly.
-constexpr size_t EXTRACT_DIRECT = size_t(48) << 20;
-constexpr int XBUCKETS = 1024;
+constexpr size_t EXTRACT_DIRECT = size_t(16) << 20;
+// Tags per bucket, as a power of two: 96 KB of outputs.
+__host__ __device__ constexpr int xbucket_shift(bool mixed) { return mixed ? 12 : 11; }
+// Counters 64 bytes apart: 10^7 atomics on 2442 neighbouring words took 0.42 ms.
+constexpr int XCNT_STRIDE = 16;
+inline int xbuckets(bool mixed, int64_t nsol) {
+  return (int)((nsol + (1 << xbucket_shift(mixed)) - 1) >> xbucket_shift(mixed));
+}
+// Allows k_unbucket its shared memory; returns a cudaError_t.
+int extract_prepare();
 void launch_extract(bool mixed, const BoxDev* box, void* pos, void* vel, int32_t* cell_out,
                     int ncells, int nsol, uint32_t* xcnt, cudaStream_t s);
 

@@ -101,7 +101,7 @@ struct BoxDev {
   // rne(m v 2^32) and of rne(m v^2 2^32) (four words a cell)
   int32_t* virt_n;
   long long* virt_sum;
-  uint32_t* xcnt;       // records per tag bucket of a state read-out (XBUCKETS)
+  uint32_t* xcnt;       // records per tag bucket of a state read-out
   // solute
   double* spos;
   double* svel;
