@@ -287,7 +287,7 @@ struct Engine {
   // for the warp-spread kernel bit 2 means a nonzero body force, bit 8 beads
   // and bit 16 the Andersen rule
   // per-cell kernel: bit 16 the Andersen rule, bit 32 the angular correction;
-  // bit 64: k_srd (bits 1, 2 and 8 as for the warp-spread kernel; bit 4 walls)
+  // bit 64: k_srd or k_srd_d (bits 1, 2 and 8 as for the warp-spread kernel; bit 4 walls)
   static constexpr int NVAR = 128;
   int2* d_spans[NVAR] = {};
   int n_spans[NVAR] = {};
@@ -334,6 +334,8 @@ struct Engine {
         const bool at = (v & 16) != 0, ang = (v & 32) != 0;
         cells_bps[m][v] = 1;
         if (v & 64) {
+          if (!mixed && !(v & (4 | 8 | 16 | 32)))
+            cells_bps[m][v] = srdd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, m);
           if (mixed && !(v & (16 | 32)) && !((v & 4) && (v & (2 | 8))))
             if (v & 8)
               srd_bead_bps[m][v & 7] = std::max(
@@ -543,20 +545,22 @@ struct Engine {
     return n < g ? std::max(n, 1) : g;
   }
 
-  // Boxes that k_srd steps.
+  // Boxes that k_srd (mixed) or k_srd_d (FP64) steps.
   bool on_srd(const BoxDev& d) const {
-    return mixed && d.collision != RULE_AT && !d.angular && d.K <= SRD_SLOTS &&
+    if (!mixed && (d.walls || d.nbead > 0 || d.K > SRDD_SLOTS || d.ncells > SRDD_MAX_CELLS)) return false;
+    return d.collision != RULE_AT && !d.angular && d.K <= SRD_SLOTS &&
            std::max(d.n[0], std::max(d.n[1], d.n[2])) < (1 << 22);
   }
 
-  // Cells per warp of k_srd: as chosen by the tuner, else the
-  // most of 32, 16, 8 and 4 that still gives every SM SRD_MIN_WARPS warps.
+  // Cells per warp of k_srd and k_srd_d: as chosen by the tuner, else the
+  // most of 32, 16, 8 and 4 that still gives every SM SRD_MIN_WARPS (FP64:
+  // SRDD_MIN_WARPS) warps, that is between half and all of what fits on it.
   int srd_cpw() const {
     if (tuned_cpw) return tuned_cpw;
     int64_t cells = 0;
     for (int v = 64; v < NVAR; ++v) cells += (int64_t)n_spans[v] * BLOCK;
     int cpw = 32;
-    while (cpw > 4 && cells < (int64_t)cpw * SRD_MIN_WARPS * nsm) cpw >>= 1;
+    while (cpw > 4 && cells < (int64_t)cpw * (mixed ? SRD_MIN_WARPS : SRDD_MIN_WARPS) * nsm) cpw >>= 1;
     return cpw;
   }
 
@@ -576,7 +580,10 @@ struct Engine {
       if (n_spans[v] == 0) continue;
       const int grid = grid_of(v, mode);
       const bool at = (v & 16) != 0;
-      if (v & 64) {
+      if ((v & 64) && !mixed) {
+        launch_srdd((v & 1) != 0, (v & 2) != 0, mode, d_boxes, d_spans[v], n_spans[v], grid,
+                    srd_cpw(), d_err, stream);
+      } else if (v & 64) {
         launch_srd((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, mode, d_boxes, d_spans[v], n_spans[v],
                    grid, srd_cpw(), d_err, stream);
         if ((v & 8) && mode != MODE_P)
@@ -828,12 +835,12 @@ struct Engine {
     d.collision = p.collision;
     d.K = row_capacity(p, nsol);
     d.angular = p.angular ? 1 : 0;
-    // k_srd: cells per sub-tile, as many as rarely have more members than the
+    // k_srd, k_srd_d: cells per sub-tile, as many as rarely have more members than the
     // staging area holds
     d.subc = 32;
     while (d.subc > 1) {
       const double mean = (double)nsol / (double)C * d.subc;
-      if (mean + 2.5 * std::sqrt(mean) <= SRD_SLOTS) break;
+      if (mean + 2.5 * std::sqrt(mean) <= (mixed ? SRD_SLOTS : SRDD_SLOTS)) break;
       d.subc >>= 1;
     }
     if (d.collision == RULE_AT && nbead > 0 &&

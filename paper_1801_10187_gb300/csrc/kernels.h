@@ -39,13 +39,22 @@ void launch_cells_warp(bool thermo, bool force, bool beads, bool at, bool ang, i
 // each: grid sizes count parts.  A solute box takes a launch without beads, over
 // the bead groups that hold none, and one with (cpw 32), over the others; mode P
 // only the first.  SRD_MIN_WARPS: see srd_cpw() in capi.cu.
-constexpr int SRD_MIN_WARPS = 16;
+constexpr int SRD_MIN_WARPS = 16, SRDD_MIN_WARPS = 6;
 int srd_blocks_per_sm(bool thermo, bool force, bool beads, bool walls, int mode);
 int srd_parts(int cpw);
 int srd_bead_items(int nspans);  // blocks' work of the bead launch
 void launch_srd(bool thermo, bool force, bool beads, bool walls, int mode, const BoxDev* boxes,
                 const int2* spans, int nspans, int grid, int cpw, int* err, cudaStream_t s);
-// The FP64 model's counterpart (k_cells_warp_d.cu), same conditions.
+// The FP64 model's counterpart of k_srd (k_srd_d.cu), for periodic SRD boxes
+// without solute and rows of at most SRDD_SLOTS records.
+// It pays where the latency of a tile counts and not the FP64 pipe's rate:
+// against k_cells_warp_d (us a step, density 10) 16^3 cells 19 to 51, 24^3 29 to
+// 52, 40^3 71 to 75, 50^3 121 to 142, 64^3 229 to 229, 100^3 823 to 760.
+constexpr int SRDD_SLOTS = 112, SRDD_MAX_CELLS = 200000;
+int srdd_blocks_per_sm(bool thermo, bool force, int mode);
+void launch_srdd(bool thermo, bool force, int mode, const BoxDev* boxes, const int2* spans,
+                 int nspans, int grid, int cpw, int* err, cudaStream_t s);
+// The FP64 model's counterpart of k_cells_warp (k_cells_warp_d.cu), same conditions.
 int cells_warpd_blocks_per_sm(bool thermo, bool force, bool beads, bool at, int mode);
 void launch_cells_warpd(bool thermo, bool force, bool beads, bool at, int mode, const BoxDev* boxes,
                         const int2* spans, int nspans, int grid, int* err, cudaStream_t s);
