@@ -86,7 +86,8 @@ size_t footprint_bytes(const mpcd_params& p, int64_t nsol, int64_t nbead) {
     b += (size_t)ng * sizeof(uint32_t) + (size_t)(ng + 1) * sizeof(uint32_t);
     if (p.lj_epsilon > 0.0)  // neighbour list: buckets, next, key, count, list, build r, forces
       b += (size_t)(2 * ((nbead + PTILE - 1) / PTILE) * PTILE) * sizeof(int32_t) +
-           (size_t)nbead * (3 * sizeof(int32_t) + NL_MAX * sizeof(int32_t) + 6 * sizeof(double));
+           (size_t)nbead * (3 * sizeof(int32_t) + NL_MAX * sizeof(int32_t) + 12 * sizeof(double) +
+                            2 * sizeof(int4));
   }
   return b;
 }
@@ -300,6 +301,10 @@ struct Engine {
   int n_mdtiles = 0;
   int2* d_vtiles = nullptr;  // wall-cut layers of the boxes with virtual particles
   int n_vtiles = 0;
+  int2* d_wtiles = nullptr;  // beads of the boxes with the repulsion
+  int n_wtiles = 0;
+  unsigned* d_wsync = nullptr;  // their MD's barrier count and flags
+  int wca_bps = 1;
   int md_chains_per_block = 1, md_threads = 32;
   uint32_t* d_tsum = nullptr;
   unsigned long long* d_gscan = nullptr;
@@ -358,6 +363,8 @@ struct Engine {
     CUDA_TRY(cudaMalloc(&d_err, sizeof(int)));
     CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), stream));
     CUDA_TRY(cudaMalloc(&d_partials, sizeof(double) * 4 * 4096));
+    CUDA_TRY(cudaMalloc(&d_wsync, sizeof(unsigned) * 4));
+    wca_bps = std::max(1, wca_blocks_per_sm());
     // keep freed box memory cached in the pool for quick re-admission
     cudaMemPool_t pool;
     if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess) {
@@ -368,7 +375,7 @@ struct Engine {
   }
 
   void free_tables() {
-    void* ptrs[] = {d_boxes, d_bsegs, d_bstiles, d_btiles, d_mdtiles, d_vtiles, d_tsum, d_gscan, d_toff};
+    void* ptrs[] = {d_boxes, d_bsegs, d_bstiles, d_btiles, d_mdtiles, d_vtiles, d_wtiles, d_tsum, d_gscan, d_toff};
     for (void* q : ptrs)
       if (q) cudaFree(q);
     for (int v = 0; v < NVAR; ++v) {
@@ -377,9 +384,10 @@ struct Engine {
       n_spans[v] = 0;
     }
     d_boxes = nullptr; d_bsegs = nullptr; d_bstiles = nullptr; d_btiles = nullptr;
-    d_mdtiles = nullptr; d_vtiles = nullptr; d_tsum = nullptr; d_gscan = nullptr; d_toff = nullptr;
+    d_mdtiles = nullptr; d_vtiles = nullptr; d_wtiles = nullptr; d_tsum = nullptr; d_gscan = nullptr; d_toff = nullptr;
     n_records = 0;
     n_vtiles = 0;
+    n_wtiles = 0;
   }
 
   void drop_graphs() {
@@ -396,6 +404,7 @@ struct Engine {
     free_tables();
     if (d_err) cudaFree(d_err);
     if (d_partials) cudaFree(d_partials);
+    if (d_wsync) cudaFree(d_wsync);
     if (own_stream && stream) cudaStreamDestroy(stream);
   }
 
@@ -450,6 +459,7 @@ struct Engine {
       if (h & ERR_GAMMA_CAP) m += "thermostat Gamma sampler rejected 64 draws; ";
       if (h & ERR_CELL_RANGE) m += "a position was not finite (cell id clamped); ";
       if (h & ERR_OVERFLOW_CAP) m += "cell overflow list full; ";
+      if (h & ERR_BARRIER) m += "solute MD: the blocks of a launch did not meet; ";
       if (h & ERR_NLIST) m += "solute neighbour list: a bead had more than 64 neighbours; ";
       return fail(MPCD_EDEVICE, m);
     }
@@ -469,7 +479,7 @@ struct Engine {
     tables_ok = true;
     if (live.empty()) return MPCD_OK;
     std::vector<BoxDev> rec;
-    std::vector<int2> sp[NVAR], bst, bt, mt, vt;
+    std::vector<int2> sp[NVAR], bst, bt, mt, vt, wt;
     std::vector<ScanSeg> bseg;
     any_beads = false;
     wca_substeps = 0;
@@ -505,7 +515,10 @@ struct Engine {
       for (int c0 = 0; c0 < d.ncells; c0 += BLOCK) sp[variant].push_back(make_int2((int)i, c0));
       if (d.nbead > 0) {
         any_beads = true;
-        if (d.wca) wca_substeps = std::max(wca_substeps, (int)d.md_substeps);
+        if (d.wca) {
+          wca_substeps = std::max(wca_substeps, (int)d.md_substeps);
+          for (int b0 = 0; b0 < d.nbead; b0 += WCA_BEADS) wt.push_back(make_int2((int)i, b0));
+        }
         bseg.push_back(ScanSeg{d.bcount, d.bstart, d.nctiles, 0});
         for (int c0 = 0; c0 < d.nctiles; c0 += STILE)
           bst.push_back(make_int2((int)bseg.size() - 1, c0));
@@ -531,6 +544,7 @@ struct Engine {
     if ((rc = up(bt, d_btiles, &n_btiles))) return rc;
     if ((rc = up(mt, d_mdtiles, &n_mdtiles))) return rc;
     if ((rc = up(vt, d_vtiles, &n_vtiles))) return rc;
+    if ((rc = up(wt, d_wtiles, &n_wtiles))) return rc;
     if (n_bstiles > 0) {
       CUDA_TRY(cudaMalloc(&d_tsum, sizeof(uint32_t) * n_bstiles));
       CUDA_TRY(cudaMalloc(&d_gscan, sizeof(unsigned long long) * n_bstiles));
@@ -607,7 +621,7 @@ struct Engine {
     launch_virtual(d_boxes, d_vtiles, n_vtiles, stream);
     if (!any_beads) return;
     if (wca_substeps > 0)
-      launch_wca_md(d_boxes, d_btiles, n_btiles, wca_substeps, d_err, stream);
+      launch_wca_md(d_boxes, d_wtiles, n_wtiles, wca_substeps, wca_bps * nsm, d_wsync, d_err, stream);
     launch_md_bin(d_boxes, d_mdtiles, n_mdtiles, md_chains_per_block, md_threads, d_err, stream);
     launch_scan(d_bsegs, d_bstiles, n_bstiles, d_tsum, d_gscan, d_toff, grid_for(n_bstiles, 8),
                 stream);
@@ -938,8 +952,18 @@ struct Engine {
         if ((rc = alloc(b, d.nl_nbr, (size_t)nbead * NL_MAX))) return rc;
         if ((rc = alloc(b, d.nl_rb, (size_t)nbead * 3))) return rc;
         if ((rc = alloc(b, d.bF, (size_t)nbead * 3))) return rc;
-        if ((rc = alloc(b, d.nl_stale, 1))) return rc;
-        CUDA_TRY(cudaMemsetAsync(d.nl_stale, 0, sizeof(int32_t), stream));
+        double lmax = 0.0;
+        for (int k = 0; k < 3; ++k) {
+          d.wfrac[k] = 4294967296.0 / d.L[k];
+          lmax = std::max(lmax, d.L[k]);
+        }
+        // float distances of the fractions: a few units of 2^-24, and at most
+        // two fractions' 2^-32 L an axis
+        d.wca_rc2f = (float)(d.wca_rc2 * (1.0 + 1e-5) + 16.0 * lmax * 0x1p-32 * rcut);
+        for (int k = 0; k < 2; ++k) {
+          if ((rc = alloc(b, d.wpos[k], (size_t)nbead * 3))) return rc;
+          if ((rc = alloc(b, d.wfix[k], (size_t)nbead))) return rc;
+        }
       }
     }
     d.cur = 0;

@@ -4,22 +4,31 @@
 // potential is only cited, and the Weeks-Chandler-Andersen repulsion is the
 // reading taken here).
 //
-// Per collision step, for the boxes with the repulsion on:
-//   clear, insert   a hash grid of the beads: cells of edge 1 (unshifted),
-//                   two buckets per bead, each bucket a linked list built by
-//                   atomic exchange of its head
-//   list            each bead lists the beads of the 27 surrounding cells
-//                   that lie within cutoff + buffer (minimum image)
-//   force           bonds (its chain neighbours) plus WCA over the list
-//   kick-drift, [clear, insert, list,] force, kick    one velocity-Verlet
-//                   substep, md_substeps times
-// The list holds every pair within the cutoff while no bead has moved more
-// than half the buffer from where it was at the build.  The drift marks the
-// box stale when one has, and the list kernels of that substep then rebuild
-// it (they return at once for a box that is not stale), so every force uses
-// a complete list.  More than NL_MAX listed neighbours raises ERR_NLIST.  The
-// later binning of the beads for the collision (k_md_bin) skips its own MD
-// for these boxes.
+// One cooperative launch runs the whole solute MD of a collision step for the
+// boxes with the repulsion.  Its blocks walk tiles of WCA_BEADS beads and meet
+// at a grid barrier:
+//   rebuild  clear, insert: a hash grid of the beads (cells of edge 1, unshifted,
+//            two buckets per bead, each a linked list built by atomic exchange of
+//            its head); list: each bead's neighbours among the 27 cells around it
+//            within cutoff + buffer (minimum image)
+//   force    bonds, each computed once, plus WCA over the list
+//   drift    closing half kick of the last substep, half kick, drift into the
+//            other of two position buffers (so that slower blocks may still read
+//            the last positions: one barrier a substep)
+// The list holds every pair within the cutoff while no bead has moved more than
+// half the buffer since the build; a drift that finds one raises a flag, and the
+// list is rebuilt before the forces.  More than NL_MAX listed neighbours raises
+// ERR_NLIST.  The later binning of the beads for the collision (k_md_bin) skips
+// its own MD for these boxes.
+//
+// What bounds it: the FP64 pipe (a warp instruction every 16 cycles of an SM) and
+// the launches.  The first form took five launches a substep, of which three
+// returned at once in nearly every one, and 45 us of force kernel: distances of
+// all listed pairs in double, each bond from both its sides with a square root
+// and a division.  Here pairs are sorted out by their distance in float from
+// 32-bit fixed-point positions (whose differences wrap to the minimum image by
+// themselves), only those within the cutoff cost FP64, and a bond costs one
+// reciprocal square root.
 #include "dev_stream.cuh"
 #include "kernels.h"
 #include "mpcd_internal.cuh"
@@ -27,6 +36,12 @@
 namespace mpcd {
 
 namespace {
+
+constexpr unsigned FULL = 0xFFFFFFFFu;
+constexpr int WT = WCA_BEADS + 1;  // threads per block: one bond more than beads
+constexpr int FW = WT / 32;
+constexpr int QCAP = 64;           // queue: fewer than 32 waiting plus one round of 32
+constexpr unsigned SPIN_LIMIT = 1u << 22;
 
 __device__ __forceinline__ uint32_t bucket_of(int key, int hsize) {
   return ((uint32_t)key * 2654435761u) % (uint32_t)hsize;
@@ -39,158 +54,77 @@ __device__ __forceinline__ int grid_coord(double x, int n) {
   return c;
 }
 
-// minimum-image difference along one axis for |d| < L (both points in the
-// box): the same result as d - L rint(d / L), without the division
+// minimum-image difference along one axis for |d| < L (both points in the box):
+// the same as d - L rint(d / L).  L / 2 has no low word, so its high word
+// settles the comparison off the FP64 pipe.
 __device__ __forceinline__ double min_image(double d, double L) {
-  if (fabs(d) > 0.5 * L) d -= copysign(L, d);
+  const int h = __double2hiint(0.5 * L);
+  if ((__double2hiint(d) & 0x7FFFFFFF) >= h) d -= copysign(L, d);
   return d;
 }
 
-// Harmonic bond forces on global bead b from its chain neighbours.
-__device__ __forceinline__ void bonds_on(const BoxDev& B, int b, double F[3]) {
-  F[0] = F[1] = F[2] = 0.0;
-  const int pos = b % B.chain_len;
-#pragma unroll
-  for (int side = 0; side < 2; ++side) {
-    int o;
-    if (side == 0) {
-      if (pos == 0) continue;
-      o = b - 1;
-    } else {
-      if (pos == B.chain_len - 1) continue;
-      o = b + 1;
-    }
-    double d[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) d[k] = min_image(B.spos[3 * o + k] - B.spos[3 * b + k], B.L[k]);
-    const double dist = sqrt(d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
-    if (!(dist > 0.0)) continue;
-    const double f = (B.bond_k * (dist - B.bond_r0)) / dist;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) F[k] += f * d[k];
-  }
+// Position x in [0, L) as a fraction of the box in 32 bits (f = 2^32 / L).
+__device__ __forceinline__ int fraction(double x, double f) {
+  return (int)(unsigned)__double2ull_rd(x * f);
 }
 
-// A tile of PTILE beads is split over WCA_SPLIT blocks of WCA_THREADS
-// threads, one bead per thread, so that even 5 * 10^4 beads fill every SM.
-constexpr int WCA_SPLIT = 8;
-constexpr int WCA_THREADS = PTILE / WCA_SPLIT;
-
-// f(B, b) for the bead of this thread, in a box with the repulsion on.
-template <class F>
-__device__ __forceinline__ void for_tile_beads(const BoxDev* boxes, const int2* tiles, F&& f) {
-  const int2 tt = tiles[blockIdx.x / WCA_SPLIT];
-  const BoxDev& B = boxes[tt.x];
-  if (!B.wca) return;
-  const int b = tt.y + (int)(blockIdx.x % WCA_SPLIT) * WCA_THREADS + (int)threadIdx.x;
-  if (b < B.nbead) f(B, b);
-}
-
-}  // namespace
-
-__global__ void __launch_bounds__(WCA_THREADS) k_wca_clear(const BoxDev* __restrict__ boxes, const int2* __restrict__ tiles,
-                            int always) {
-  const int2 tt = tiles[blockIdx.x / WCA_SPLIT];
-  const BoxDev& B = boxes[tt.x];
-  if (!B.wca || !(always || *B.nl_stale)) return;
-  const int h0 = 2 * tt.y + (int)(blockIdx.x % WCA_SPLIT) * 2 * WCA_THREADS;
-  const int h1 = min(h0 + 2 * WCA_THREADS, B.nl_hsize);
-  for (int h = h0 + (int)threadIdx.x; h < h1; h += blockDim.x) B.nl_head[h] = -1;
-}
-
-__global__ void __launch_bounds__(WCA_THREADS) k_wca_insert(const BoxDev* __restrict__ boxes, const int2* __restrict__ tiles,
-                             int always) {
-  for_tile_beads(boxes, tiles, [&](const BoxDev& B, int b) {
-    if (!(always || *B.nl_stale)) return;
-    int c[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const double x = B.spos[3 * b + k];
-      B.nl_rb[3 * b + k] = x;
-      c[k] = grid_coord(x, B.n[k]);
-    }
-    const int key = c[0] + B.n[0] * (c[1] + B.n[1] * c[2]);
-    B.nl_key[b] = key;
-    B.nl_next[b] = atomicExch(&B.nl_head[bucket_of(key, B.nl_hsize)], b);
-  });
-}
-
-__global__ void __launch_bounds__(WCA_THREADS) k_wca_list(const BoxDev* __restrict__ boxes, const int2* __restrict__ tiles,
-                           int always, int* err) {
-  for_tile_beads(boxes, tiles, [&](const BoxDev& B, int b) {
-    if (!(always || *B.nl_stale)) return;
-    const int key = B.nl_key[b];
-    const int c[3] = {key % B.n[0], (key / B.n[0]) % B.n[1], key / (B.n[0] * B.n[1])};
-    const double rb[3] = {B.nl_rb[3 * b], B.nl_rb[3 * b + 1], B.nl_rb[3 * b + 2]};
-    int cnt = 0;
-    bool over = false;
-    // n_k >= 3 on every axis, so the 27 cells are distinct
-    for (int dz = -1; dz <= 1; ++dz)
-      for (int dy = -1; dy <= 1; ++dy)
-        for (int dx = -1; dx <= 1; ++dx) {
-          const int x = (c[0] + dx + B.n[0]) % B.n[0], y = (c[1] + dy + B.n[1]) % B.n[1],
-                    z = (c[2] + dz + B.n[2]) % B.n[2];
-          const int k2 = x + B.n[0] * (y + B.n[1] * z);
-          int j = B.nl_head[bucket_of(k2, B.nl_hsize)];
-          // a bucket's list is acyclic and holds at most every bead once
-          for (int guard = 0; j >= 0 && guard < B.nbead; ++guard, j = B.nl_next[j]) {
-            if (j == b || B.nl_key[j] != k2) continue;
-            double r2 = 0.0;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-              const double d = min_image(B.nl_rb[3 * j + q] - rb[q], B.L[q]);
-              r2 += d * d;
-            }
-            if (!(r2 < B.wca_rl2)) continue;
-            if (cnt < NL_MAX) B.nl_nbr[(size_t)b * NL_MAX + cnt] = j;
-            else over = true;
-            ++cnt;
-          }
-        }
-    B.nl_cnt[b] = min(cnt, NL_MAX);
-    if (over) atomicOr(err, ERR_NLIST);
-  });
-}
-
-// Bond forces plus the WCA repulsion over the bead's list (Sec. 4.3 reading).
-//
-// The arithmetic is FP64, and the FP64 pipe issues a warp instruction only
-// every many cycles on this GPU, so what counts is how many lanes of each
-// instruction do useful work.  A warp owns 32 consecutive beads.  Each lane
-// takes its own bead's two bonds.  The warp's listed pairs are then taken as
-// one flat sequence (bead by bead, in list order), 32 at a time: each lane
-// forms the distance of one pair, and the pairs within the cutoff go, in
-// order, to a queue in shared memory.  Whenever the queue holds 32 pairs,
-// every lane takes one and computes its force; the forces of each bead's run
-// in the queue are added in queue order by the run's first lane (no
-// atomics).  So the divisions run on full warps however the list lengths and
-// hits are spread over the beads.  The list order follows the hash grid's
-// insertion order, which may differ between runs, and so may the last bits
-// of a sum.
-namespace {
-constexpr int FW = WCA_THREADS / 32;  // warps per block
-constexpr int QCAP = 64;              // queue: fewer than 32 waiting plus one round of 32
-
-struct ForceWarp {
+struct MdWarp {
   int off[33];          // first flat pair index of each bead; off[32] = all pairs
   int qown[QCAP];       // queued pair: the warp-local bead it acts on
-  double qd[4][QCAP];   // queued pair: d (3) and r^2
+  int qj[QCAP];         // and the other bead
   double c[3][32];      // forces of one flush, one per lane
   double F[3][32];      // sum of each bead's pair forces
-  double rb[3][32];     // bead positions
+};
+struct MdShared {
+  MdWarp w[FW];
+  double r[3][WT];      // positions of beads b0 - 1 ... b0 + WCA_BEADS - 1
+  double g[3][WT];      // force of the bond from bead b0 - 1 + t to the next, on the former
+  int X[3][WT];         // fixed-point positions, as r
 };
 
-// Forces of queue entries [0, nq): lane l takes entry l; each run of
-// entries of one bead is summed, in order, by its first lane.
-__device__ __forceinline__ void wca_flush(const BoxDev& B, ForceWarp& W, int nq, int lane) {
+// Grid barrier of a cooperative launch: *bar counts arrivals.  The wait is
+// bounded; a block that gives up raises ERR_BARRIER and waits at no barrier again.
+__device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned& target, bool& dead, int* err) {
+  __syncthreads();
+  target += gridDim.x;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(bar, 1u);
+    if (!dead) {
+      unsigned spins = 0, seen = 0;
+      do {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
+      } while ((int)(seen - target) < 0 && ++spins < SPIN_LIMIT);
+      if ((int)(seen - target) < 0) {
+        dead = true;
+        atomicOr(err, ERR_BARRIER);
+      }
+    }
+    __threadfence();
+  }
+  __syncthreads();
+}
+
+// Forces of queue entries [0, nq): lane l takes entry l; each run of entries of
+// one bead is summed, in order, by its first lane.
+__device__ __forceinline__ void wca_flush(const BoxDev& B, MdShared& S, MdWarp& W, int wbase,
+                                          const double* pos, int nq, int lane) {
   if (lane < nq) {
-    const double r2 = W.qd[3][lane];
-    const double inv = 1.0 / r2;
-    const double x = B.lj_sig2 * inv;
-    const double x6 = x * x * x;
-    const double g = 24.0 * B.lj_eps * x6 * (2.0 * x6 - 1.0) * inv;
+    const int own = W.qown[lane], j = W.qj[lane];
+    double d[3];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) W.c[q][lane] = -(g * W.qd[q][lane]);
+    for (int q = 0; q < 3; ++q)
+      d[q] = min_image(__ldcg(&pos[3 * (size_t)j + q]) - S.r[q][wbase + own], B.L[q]);
+    const double r2 = fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0]));
+    double g = 0.0;
+    if (r2 < B.wca_rc2) {
+      const double inv = 1.0 / r2;
+      const double x = B.lj_sig2 * inv;
+      const double x6 = x * x * x;
+      g = 24.0 * B.lj_eps * x6 * (2.0 * x6 - 1.0) * inv;
+    }
+#pragma unroll
+    for (int q = 0; q < 3; ++q) W.c[q][lane] = -(g * d[q]);
   }
   __syncwarp();
   if (lane < nq) {
@@ -207,147 +141,270 @@ __device__ __forceinline__ void wca_flush(const BoxDev& B, ForceWarp& W, int nq,
   }
   __syncwarp();
 }
+
 }  // namespace
 
-__global__ void __launch_bounds__(WCA_THREADS) k_wca_force(const BoxDev* __restrict__ boxes, const int2* __restrict__ tiles,
-                            int substep) {
-  __shared__ ForceWarp fw[FW];
-  const int2 tt = tiles[blockIdx.x / WCA_SPLIT];
-  const BoxDev& B = boxes[tt.x];
-  if (!B.wca || substep > B.md_substeps) return;  // the same for the whole block
-  const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
-  ForceWarp& W = fw[warp];
-  const int b0 = tt.y + (int)(blockIdx.x % WCA_SPLIT) * WCA_THREADS + warp * 32;
-  const int b = b0 + lane;
-  const bool valid = b < B.nbead;
-  double F[3] = {0.0, 0.0, 0.0};
-  int cnt = 0;
-  if (valid) {
-    if (b == 0) *B.nl_stale = 0;  // this substep's list kernels have all run
-    bonds_on(B, b, F);
-    cnt = B.nl_cnt[b];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) W.rb[q][lane] = B.spos[3 * b + q];
-  }
-#pragma unroll
-  for (int q = 0; q < 3; ++q) W.F[q][lane] = 0.0;
-  // flat pair offsets: exclusive scan of the list lengths over the warp
-  int incl = cnt;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  W.off[lane] = incl - cnt;
-  if (lane == 31) W.off[32] = incl;
-  __syncwarp();
-  const int total = W.off[32];  // at most 32 NL_MAX
-  int nq = 0;                   // queued pairs (the same in every lane)
-  for (int base = 0; base < total; base += 32) {
-    const int k = base + lane;
-    bool hit = false;
-    int own = 0;
-    double d[3] = {0.0, 0.0, 0.0}, r2 = 0.0;
-    if (k < total) {
-      // the bead of pair k: the last with off <= k (offsets do not decrease)
-#pragma unroll
-      for (int step = 16; step > 0; step >>= 1)
-        if (W.off[own + step] <= k) own += step;
-      const int j = B.nl_nbr[(size_t)(b0 + own) * NL_MAX + (k - W.off[own])];
-#pragma unroll
-      for (int q = 0; q < 3; ++q) d[q] = min_image(B.spos[3 * j + q] - W.rb[q][own], B.L[q]);
-      r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-      hit = r2 < B.wca_rc2;
-    }
-    const unsigned m = __ballot_sync(0xFFFFFFFFu, hit);
-    if (hit) {
-      const int pos = nq + __popc(m & ((1u << lane) - 1u));  // < nq + 32 <= QCAP
-      W.qown[pos] = own;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) W.qd[q][pos] = d[q];
-      W.qd[3][pos] = r2;
-    }
-    nq += __popc(m);
-    __syncwarp();
-    if (nq >= 32) {
-      wca_flush(B, W, 32, lane);
-      nq -= 32;
-      // move the rest (fewer than 32) to the front
-      int own2 = 0;
-      double e[4] = {0.0, 0.0, 0.0, 0.0};
-      if (lane < nq) {
-        own2 = W.qown[32 + lane];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) e[q] = W.qd[q][32 + lane];
-      }
-      __syncwarp();
-      if (lane < nq) {
-        W.qown[lane] = own2;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) W.qd[q][lane] = e[q];
-      }
-      __syncwarp();
-    }
-  }
-  if (nq > 0) wca_flush(B, W, nq, lane);
-  if (valid) {
-#pragma unroll
-    for (int q = 0; q < 3; ++q) B.bF[3 * b + q] = F[q] + W.F[q][lane];
-  }
-}
+__global__ void __launch_bounds__(WT, 4) k_wca_md(const BoxDev* __restrict__ boxes,
+                                               const int2* __restrict__ tiles, int ntiles,
+                                               int max_substeps, unsigned* bar, int* stale, int* err) {
+  __shared__ MdShared S;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  MdWarp& W = S.w[warp];
+  unsigned target = 0u;
+  bool dead = false;
 
-// First half of a velocity-Verlet substep: half kick, drift (periodic), and
-// the check whether the list still covers every pair within the cutoff.
-// With close_prev, the closing half kick of the previous substep comes first
-// (the same force, added as a separate step, as the substeps are written).
-__global__ void __launch_bounds__(WCA_THREADS) k_wca_kick_drift(const BoxDev* __restrict__ boxes, const int2* __restrict__ tiles,
-                                 int substep, int close_prev) {
-  for_tile_beads(boxes, tiles, [&](const BoxDev& B, int b) {
-    if (substep >= B.md_substeps) return;
-    double m2 = 0.0;
+  // f(box, bead, first bead of the tile) for every bead of this block's tiles
+  auto for_beads = [&](auto&& f) {
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+      const int2 tt = tiles[tile];
+      const BoxDev& B = boxes[tt.x];
+      if (t < WCA_BEADS && tt.y + t < B.nbead) f(B, tt.y + t);
+    }
+  };
+  // rebuild the lists of the boxes with substeps left, at positions buf
+  auto rebuild = [&](int sub, int buf) {
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+      const int2 tt = tiles[tile];
+      const BoxDev& B = boxes[tt.x];
+      if (sub >= B.md_substeps) continue;
+      const int h1 = tt.y + WCA_BEADS >= B.nbead ? B.nl_hsize : 2 * (tt.y + WCA_BEADS);
+      for (int h = 2 * tt.y + t; h < h1; h += WT) B.nl_head[h] = -1;
+    }
+    grid_barrier(bar, target, dead, err);
+    for_beads([&](const BoxDev& B, int b) {
+      if (sub >= B.md_substeps) return;
+      int c[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const double x = B.wpos[buf][3 * (size_t)b + k];
+        B.nl_rb[3 * (size_t)b + k] = x;
+        c[k] = grid_coord(x, B.n[k]);
+      }
+      const int key = c[0] + B.n[0] * (c[1] + B.n[1] * c[2]);
+      B.nl_key[b] = key;
+      B.nl_next[b] = atomicExch(&B.nl_head[bucket_of(key, B.nl_hsize)], b);
+    });
+    grid_barrier(bar, target, dead, err);
+    for_beads([&](const BoxDev& B, int b) {
+      if (sub >= B.md_substeps) return;
+      const int key = B.nl_key[b];
+      const int c[3] = {key % B.n[0], (key / B.n[0]) % B.n[1], key / (B.n[0] * B.n[1])};
+      const double rb[3] = {B.nl_rb[3 * (size_t)b], B.nl_rb[3 * (size_t)b + 1],
+                            B.nl_rb[3 * (size_t)b + 2]};
+      int cnt = 0;
+      bool over = false;
+      // n_k >= 3 on every axis, so the 27 cells are distinct
+      for (int dz = -1; dz <= 1; ++dz)
+        for (int dy = -1; dy <= 1; ++dy)
+          for (int dx = -1; dx <= 1; ++dx) {
+            int x = c[0] + dx, y = c[1] + dy, z = c[2] + dz;
+            x += x < 0 ? B.n[0] : x >= B.n[0] ? -B.n[0] : 0;
+            y += y < 0 ? B.n[1] : y >= B.n[1] ? -B.n[1] : 0;
+            z += z < 0 ? B.n[2] : z >= B.n[2] ? -B.n[2] : 0;
+            const int k2 = x + B.n[0] * (y + B.n[1] * z);
+            // other blocks' heads and links of this very launch: past L1
+            int j = __ldcg(&B.nl_head[bucket_of(k2, B.nl_hsize)]);
+            // a bucket's list is acyclic and holds at most every bead once
+            for (int guard = 0; j >= 0 && guard < B.nbead; ++guard, j = __ldcg(&B.nl_next[j])) {
+              if (j == b || __ldcg(&B.nl_key[j]) != k2) continue;
+              double r2 = 0.0;
+#pragma unroll
+              for (int q = 0; q < 3; ++q) {
+                const double d = min_image(__ldcg(&B.nl_rb[3 * (size_t)j + q]) - rb[q], B.L[q]);
+                r2 = fma(d, d, r2);
+              }
+              if (!(r2 < B.wca_rl2)) continue;
+              if (cnt < NL_MAX) B.nl_nbr[(size_t)b * NL_MAX + cnt] = j;
+              else over = true;
+              ++cnt;
+            }
+          }
+      B.nl_cnt[b] = min(cnt, NL_MAX);
+      if (over) atomicOr(err, ERR_NLIST);
+    });
+    __syncthreads();  // a bead's list is read by its whole warp
+  };
+  // bond and WCA forces of this block's beads at positions buf
+  auto forces = [&](int sub, int buf) {
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+      const int2 tt = tiles[tile];
+      const BoxDev& B = boxes[tt.x];
+      if (sub > B.md_substeps) continue;  // the same for the whole block
+      const double* pos = B.wpos[buf];
+      const int4* fix = B.wfix[buf];
+      const int b0 = tt.y, cl = B.chain_len;
+      __syncthreads();  // the last tile is done with S
+      // thread t: bead b0 - 1 + t and its bond to the next bead of its chain
+      const int jb = b0 - 1 + t;
+      double rj[3] = {0.0, 0.0, 0.0};
+      if (jb >= 0 && jb < B.nbead) {
+        const int4 f = __ldcg(&fix[jb]);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          rj[q] = __ldcg(&pos[3 * (size_t)jb + q]);
+          S.r[q][t] = rj[q];
+        }
+        S.X[0][t] = f.x;
+        S.X[1][t] = f.y;
+        S.X[2][t] = f.z;
+      }
+      __syncthreads();
+      double g[3] = {0.0, 0.0, 0.0};
+      if (jb >= 0 && jb + 1 < B.nbead && jb % cl != cl - 1) {
+        double d[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          const double rn = t + 1 < WT ? S.r[q][t + 1] : __ldcg(&pos[3 * (size_t)(jb + 1) + q]);
+          d[q] = min_image(rn - rj[q], B.L[q]);
+        }
+        const double r2 = fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0]));
+        if (r2 > 0.0) {  // k (1 - r0 / |d|) d; coincident beads: no force
+          const double f = fma(-(B.bond_k * B.bond_r0), rsqrt(r2), B.bond_k);
+#pragma unroll
+          for (int q = 0; q < 3; ++q) g[q] = f * d[q];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) S.g[q][t] = g[q];
+      const int b = b0 + t;
+      const bool valid = t < WCA_BEADS && b < B.nbead;
+      const int cnt = valid ? B.nl_cnt[b] : 0;
+      // flat pair offsets: exclusive scan of the list lengths over the warp
+      int incl = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += y;
+      }
+      W.off[lane] = incl - cnt;
+      if (lane == 31) W.off[32] = incl;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) W.F[q][lane] = 0.0;
+      __syncthreads();
+      const float sc[3] = {(float)(B.L[0] * 0x1p-32), (float)(B.L[1] * 0x1p-32),
+                           (float)(B.L[2] * 0x1p-32)};
+      const int wbase = warp * 32 + 1;  // place of the warp's first bead in S.r and S.X
+      const int total = W.off[32];      // at most 32 NL_MAX
+      int nq = 0;                       // queued pairs (the same in every lane)
+      for (int base = 0; base < total; base += 32) {
+        const int k = base + lane;
+        bool hit = false;
+        int own = 0, j = 0;
+        if (k < total) {
+          // the bead of pair k: the last with off <= k (offsets do not decrease)
+#pragma unroll
+          for (int step = 16; step > 0; step >>= 1)
+            if (W.off[own + step] <= k) own += step;
+          j = B.nl_nbr[(size_t)(b0 + warp * 32 + own) * NL_MAX + (k - W.off[own])];
+          const int4 f = __ldcg(&fix[j]);
+          const float dx = (float)(int)((unsigned)f.x - (unsigned)S.X[0][wbase + own]) * sc[0];
+          const float dy = (float)(int)((unsigned)f.y - (unsigned)S.X[1][wbase + own]) * sc[1];
+          const float dz = (float)(int)((unsigned)f.z - (unsigned)S.X[2][wbase + own]) * sc[2];
+          hit = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < B.wca_rc2f;
+        }
+        const unsigned m = __ballot_sync(FULL, hit);
+        if (hit) {
+          const int at = nq + __popc(m & ((1u << lane) - 1u));  // < nq + 32 <= QCAP
+          W.qown[at] = own;
+          W.qj[at] = j;
+        }
+        nq += __popc(m);
+        __syncwarp();
+        if (nq >= 32) {
+          wca_flush(B, S, W, wbase, pos, 32, lane);
+          nq -= 32;
+          // move the rest (fewer than 32) to the front
+          int e0 = 0, e1 = 0;
+          if (lane < nq) {
+            e0 = W.qown[32 + lane];
+            e1 = W.qj[32 + lane];
+          }
+          __syncwarp();
+          if (lane < nq) {
+            W.qown[lane] = e0;
+            W.qj[lane] = e1;
+          }
+          __syncwarp();
+        }
+      }
+      if (nq > 0) wca_flush(B, S, W, wbase, pos, nq, lane);
+      if (valid) {
+        // bond to the left (index t) and to the right (t + 1; b0 + t is bead t + 1 of S)
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          B.bF[3 * (size_t)b + q] = (S.g[q][t + 1] - S.g[q][t]) + W.F[q][lane];
+      }
+    }
+  };
+  auto put = [&](const BoxDev& B, int buf, int b, const double r[3]) {
+    int x[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      double v = B.svel[3 * b + k];
-      if (close_prev) v = v + B.md_hh * B.bF[3 * b + k];
-      v = v + B.md_hh * B.bF[3 * b + k];
-      const double r = wrap(B.spos[3 * b + k] + B.md_h * v, B.L[k]);
-      B.svel[3 * b + k] = v;
-      B.spos[3 * b + k] = r;
-      const double d = min_image(r - B.nl_rb[3 * b + k], B.L[k]);
-      m2 += d * d;
+      B.wpos[buf][3 * (size_t)b + k] = r[k];
+      x[k] = fraction(r[k], B.wfrac[k]);
     }
-    if (m2 > B.wca_half_skin2) *B.nl_stale = 1;
-  });
-}
+    B.wfix[buf][b] = make_int4(x[0], x[1], x[2], 0);
+  };
 
-// Closing half kick of a box's last substep (its force is the last one computed).
-__global__ void __launch_bounds__(WCA_THREADS) k_wca_kick(const BoxDev* __restrict__ boxes, const int2* __restrict__ tiles) {
-  for_tile_beads(boxes, tiles, [&](const BoxDev& B, int b) {
+  for_beads([&](const BoxDev& B, int b) {
+    const double r[3] = {B.spos[3 * (size_t)b], B.spos[3 * (size_t)b + 1], B.spos[3 * (size_t)b + 2]};
+    put(B, 0, b, r);
+  });
+  rebuild(0, 0);
+  forces(0, 0);
+  for (int sub = 0; sub < max_substeps; ++sub) {
+    const int nxt = (sub + 1) & 1;
+    for_beads([&](const BoxDev& B, int b) {
+      if (sub >= B.md_substeps) return;
+      double r[3], m2 = 0.0;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const double F = B.bF[3 * (size_t)b + k];
+        double v = B.svel[3 * (size_t)b + k];
+        if (sub > 0) v = fma(B.md_hh, F, v);  // closes the last substep
+        v = fma(B.md_hh, F, v);
+        r[k] = wrap_bits(fma(B.md_h, v, B.wpos[nxt ^ 1][3 * (size_t)b + k]), B.L[k]);
+        B.svel[3 * (size_t)b + k] = v;
+        const double d = min_image(r[k] - B.nl_rb[3 * (size_t)b + k], B.L[k]);
+        m2 = fma(d, d, m2);
+      }
+      put(B, nxt, b, r);
+      if (m2 > B.wca_half_skin2) stale[sub % 3] = 1;
+    });
+    grid_barrier(bar, target, dead, err);
+    // the flag of two substeps on: read by all before this barrier, set after the next
+    if (blockIdx.x == 0 && t == 0) stale[(sub + 2) % 3] = 0;
+    int again;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(again) : "l"(stale + sub % 3) : "memory");
+    if (again) rebuild(sub, nxt);
+    forces(sub + 1, nxt);
+  }
+  for_beads([&](const BoxDev& B, int b) {
     if (B.md_substeps <= 0) return;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) B.svel[3 * b + k] = B.svel[3 * b + k] + B.md_hh * B.bF[3 * b + k];
+    for (int k = 0; k < 3; ++k) {
+      B.svel[3 * (size_t)b + k] = fma(B.md_hh, B.bF[3 * (size_t)b + k], B.svel[3 * (size_t)b + k]);
+      B.spos[3 * (size_t)b + k] = B.wpos[B.md_substeps & 1][3 * (size_t)b + k];
+    }
   });
 }
 
-// The whole solute MD of one collision step for the boxes with the repulsion.
-void launch_wca_md(const BoxDev* boxes, const int2* tiles, int ntiles, int max_substeps, int* err,
-                   cudaStream_t s) {
-  if (ntiles <= 0) return;
-  k_wca_clear<<<ntiles * WCA_SPLIT, WCA_THREADS, 0, s>>>(boxes, tiles, 1);
-  k_wca_insert<<<ntiles * WCA_SPLIT, WCA_THREADS, 0, s>>>(boxes, tiles, 1);
-  k_wca_list<<<ntiles * WCA_SPLIT, WCA_THREADS, 0, s>>>(boxes, tiles, 1, err);
-  k_wca_force<<<ntiles * WCA_SPLIT, WCA_THREADS, 0, s>>>(boxes, tiles, 0);
-  // substep sub: kick-drift (closing substep sub - 1 first), rebuild where
-  // stale, force; the last substep's closing kick is a launch of its own, and
-  // so is that of a box whose md_substeps is below the largest
-  for (int sub = 0; sub < max_substeps; ++sub) {
-    k_wca_kick_drift<<<ntiles * WCA_SPLIT, WCA_THREADS, 0, s>>>(boxes, tiles, sub, sub > 0);
-    k_wca_clear<<<ntiles * WCA_SPLIT, WCA_THREADS, 0, s>>>(boxes, tiles, 0);  // rebuild where stale
-    k_wca_insert<<<ntiles * WCA_SPLIT, WCA_THREADS, 0, s>>>(boxes, tiles, 0);
-    k_wca_list<<<ntiles * WCA_SPLIT, WCA_THREADS, 0, s>>>(boxes, tiles, 0, err);
-    k_wca_force<<<ntiles * WCA_SPLIT, WCA_THREADS, 0, s>>>(boxes, tiles, sub + 1);
-  }
-  k_wca_kick<<<ntiles * WCA_SPLIT, WCA_THREADS, 0, s>>>(boxes, tiles);
+int wca_blocks_per_sm() {
+  int nb = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_wca_md, WT, 0);
+  return nb;
+}
+
+// sync: four words (the barrier's count and the flags), zeroed here.
+int launch_wca_md(const BoxDev* boxes, const int2* tiles, int ntiles, int max_substeps, int max_blocks,
+                  unsigned* sync, int* err, cudaStream_t s) {
+  if (ntiles <= 0) return 0;
+  cudaMemsetAsync(sync, 0, 4 * sizeof(unsigned), s);
+  int* stale = (int*)(sync + 1);
+  void* args[] = {(void*)&boxes, (void*)&tiles, (void*)&ntiles, (void*)&max_substeps,
+                  (void*)&sync, (void*)&stale, (void*)&err};
+  return (int)cudaLaunchCooperativeKernel((void*)k_wca_md, dim3(ntiles < max_blocks ? ntiles : max_blocks),
+                                          dim3(WT), args, 0, s);
 }
 
 }  // namespace mpcd

@@ -15,8 +15,13 @@ namespace mpcd {
 // Solute MD of one collision step for the boxes with the non-bonded WCA
 // repulsion (k_wca.cu): neighbour-list build, then max_substeps velocity-
 // Verlet substeps (each box takes its own md_substeps).
-void launch_wca_md(const BoxDev* boxes, const int2* tiles, int ntiles, int max_substeps, int* err,
-                   cudaStream_t s);
+// tiles: (box, first of WCA_BEADS beads); sync: four device words, zeroed here;
+// max_blocks: blocks that fit on the device together (wca_blocks_per_sm per
+// SM; the launch is cooperative).  Returns a cudaError_t.
+constexpr int WCA_BEADS = 127;
+int wca_blocks_per_sm();
+int launch_wca_md(const BoxDev* boxes, const int2* tiles, int ntiles, int max_substeps, int max_blocks,
+                  unsigned* sync, int* err, cudaStream_t s);
 int cells_blocks_per_sm(bool mixed, int variant, int mode);
 void launch_cells(bool mixed, int variant, int mode, const BoxDev* boxes, const int2* spans,
                   int nspans, int grid, int* err, cudaStream_t s);

@@ -42,6 +42,7 @@ constexpr int STILE = 2048;    // entries per scan tile
 constexpr int BLOCK = 256;     // threads per block; the fused step has one thread per cell
 constexpr int BEAD_TILE = 32;  // cells per bead group
 constexpr int ERR_OVERFLOW_CAP = 4;  // overflow list full (cannot happen: it holds N records)
+constexpr int ERR_BARRIER = 16;  // the solute MD's grid barrier gave up
 constexpr int ERR_NLIST = 8;   // solute neighbour list: more than NL_MAX pairs for a bead
 constexpr int NL_MAX = 64;     // neighbours per bead in the solute pair list
 constexpr double NL_SKIN = 0.4;  // neighbour-list buffer (the paper's 0.4 a)
@@ -133,7 +134,11 @@ struct BoxDev {
   int32_t* nl_nbr;      // bead -> neighbours (NL_MAX each)
   double* nl_rb;        // positions at the build (3 per bead)
   double* bF;           // forces on the beads (3 per bead)
-  int32_t* nl_stale;    // 1: a bead moved more than half the buffer since the build
+  double* wpos[2];      // positions during the MD of a step (3 per bead, by turns)
+  int4* wfix[2];        // the same as 32-bit fractions of the box (x, y, z, 0)
+  double wfrac[3];      // 2^32 / L
+  float wca_rc2f;       // cutoff^2 with a margin for float distances of wfix
+  int32_t pad_x;
 };
 
 // Segments for the segmented exclusive scan (cells of each box, and bead
