@@ -40,7 +40,8 @@ namespace {
 constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int WT = WCA_BEADS + 1;  // threads per block: one bond more than beads
 constexpr int FW = WT / 32;
-constexpr int QCAP = 64;           // queue: fewer than 32 waiting plus one round of 32
+constexpr int ROUNDS = 4;          // rounds of 32 pairs whose loads are in flight together
+constexpr int QCAP = 32 * (ROUNDS + 1);  // queue: fewer than 32 waiting plus those
 constexpr unsigned SPIN_LIMIT = 1u << 22;
 
 __device__ __forceinline__ uint32_t bucket_of(int key, int hsize) {
@@ -58,7 +59,7 @@ __device__ __forceinline__ int grid_coord(double x, int n) {
 // the same as d - L rint(d / L).  L / 2 has no low word, so its high word
 // settles the comparison off the FP64 pipe.
 __device__ __forceinline__ double min_image(double d, double L) {
-  const int h = __double2hiint(0.5 * L);
+  const int h = __double2hiint(L) - 0x00100000;  // of L / 2
   if ((__double2hiint(d) & 0x7FFFFFFF) >= h) d -= copysign(L, d);
   return d;
 }
@@ -105,12 +106,13 @@ __device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned& target, bo
   __syncthreads();
 }
 
-// Forces of queue entries [0, nq): lane l takes entry l; each run of entries of
+// Forces of queue entries [q0, q0 + nq), nq <= 32: lane l takes entry q0 + l; each run of entries of
 // one bead is summed, in order, by its first lane.
 __device__ __forceinline__ void wca_flush(const BoxDev& B, MdShared& S, MdWarp& W, int wbase,
-                                          const double* pos, int nq, int lane) {
+                                          const double* pos, int q0, int nq, int lane) {
+  const int* qown = W.qown + q0;
   if (lane < nq) {
-    const int own = W.qown[lane], j = W.qj[lane];
+    const int own = qown[lane], j = W.qj[q0 + lane];
     double d[3];
 #pragma unroll
     for (int q = 0; q < 3; ++q)
@@ -128,10 +130,10 @@ __device__ __forceinline__ void wca_flush(const BoxDev& B, MdShared& S, MdWarp& 
   }
   __syncwarp();
   if (lane < nq) {
-    const int own = W.qown[lane];
-    if (lane == 0 || W.qown[lane - 1] != own) {
+    const int own = qown[lane];
+    if (lane == 0 || qown[lane - 1] != own) {
       double acc[3] = {W.c[0][lane], W.c[1][lane], W.c[2][lane]};
-      for (int l = lane + 1; l < nq && W.qown[l] == own; ++l) {
+      for (int l = lane + 1; l < nq && qown[l] == own; ++l) {
 #pragma unroll
         for (int q = 0; q < 3; ++q) acc[q] += W.c[q][l];
       }
@@ -259,7 +261,9 @@ __global__ void __launch_bounds__(WT, 4) k_wca_md(const BoxDev* __restrict__ box
         }
         const double r2 = fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0]));
         if (r2 > 0.0) {  // k (1 - r0 / |d|) d; coincident beads: no force
-          const double f = fma(-(B.bond_k * B.bond_r0), rsqrt(r2), B.bond_k);
+          double y = rsqrt(r2);
+          y = fma(0.5 * y, fma(-(r2 * y), y, 1.0), y);  // to half a unit in the last place
+          const double f = fma(-(B.bond_k * B.bond_r0), y, B.bond_k);
 #pragma unroll
           for (int q = 0; q < 3; ++q) g[q] = f * d[q];
         }
@@ -286,38 +290,51 @@ __global__ void __launch_bounds__(WT, 4) k_wca_md(const BoxDev* __restrict__ box
       const int wbase = warp * 32 + 1;  // place of the warp's first bead in S.r and S.X
       const int total = W.off[32];      // at most 32 NL_MAX
       int nq = 0;                       // queued pairs (the same in every lane)
-      for (int base = 0; base < total; base += 32) {
-        const int k = base + lane;
-        bool hit = false;
-        int own = 0, j = 0;
-        if (k < total) {
-          // the bead of pair k: the last with off <= k (offsets do not decrease)
+      for (int base = 0; base < total; base += 32 * ROUNDS) {
+        int own[ROUNDS], j[ROUNDS];
+        int4 f[ROUNDS];
 #pragma unroll
-          for (int step = 16; step > 0; step >>= 1)
-            if (W.off[own + step] <= k) own += step;
-          j = B.nl_nbr[(size_t)(b0 + warp * 32 + own) * NL_MAX + (k - W.off[own])];
-          const int4 f = __ldcg(&fix[j]);
-          const float dx = (float)(int)((unsigned)f.x - (unsigned)S.X[0][wbase + own]) * sc[0];
-          const float dy = (float)(int)((unsigned)f.y - (unsigned)S.X[1][wbase + own]) * sc[1];
-          const float dz = (float)(int)((unsigned)f.z - (unsigned)S.X[2][wbase + own]) * sc[2];
-          hit = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < B.wca_rc2f;
+        for (int u = 0; u < ROUNDS; ++u) {
+          const int k = base + 32 * u + lane;
+          own[u] = 0;
+          j[u] = -1;
+          if (k < total) {
+            // the bead of pair k: the last with off <= k (offsets do not decrease)
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1)
+              if (W.off[own[u] + step] <= k) own[u] += step;
+            j[u] = B.nl_nbr[(size_t)(b0 + warp * 32 + own[u]) * NL_MAX + (k - W.off[own[u]])];
+          }
         }
-        const unsigned m = __ballot_sync(FULL, hit);
-        if (hit) {
-          const int at = nq + __popc(m & ((1u << lane) - 1u));  // < nq + 32 <= QCAP
-          W.qown[at] = own;
-          W.qj[at] = j;
+#pragma unroll
+        for (int u = 0; u < ROUNDS; ++u)
+          if (j[u] >= 0) f[u] = __ldcg(&fix[j[u]]);
+#pragma unroll
+        for (int u = 0; u < ROUNDS; ++u) {
+          bool hit = false;
+          if (j[u] >= 0) {
+            const float dx = (float)(int)((unsigned)f[u].x - (unsigned)S.X[0][wbase + own[u]]) * sc[0];
+            const float dy = (float)(int)((unsigned)f[u].y - (unsigned)S.X[1][wbase + own[u]]) * sc[1];
+            const float dz = (float)(int)((unsigned)f[u].z - (unsigned)S.X[2][wbase + own[u]]) * sc[2];
+            hit = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < B.wca_rc2f;
+          }
+          const unsigned m = __ballot_sync(FULL, hit);
+          if (hit) {
+            const int at = nq + __popc(m & ((1u << lane) - 1u));  // < QCAP
+            W.qown[at] = own[u];
+            W.qj[at] = j[u];
+          }
+          nq += __popc(m);
         }
-        nq += __popc(m);
         __syncwarp();
-        if (nq >= 32) {
-          wca_flush(B, S, W, wbase, pos, 32, lane);
-          nq -= 32;
-          // move the rest (fewer than 32) to the front
+        int q0 = 0;
+        for (; nq - q0 >= 32; q0 += 32) wca_flush(B, S, W, wbase, pos, q0, 32, lane);
+        if (q0 > 0) {  // the rest (fewer than 32) to the front
+          nq -= q0;
           int e0 = 0, e1 = 0;
           if (lane < nq) {
-            e0 = W.qown[32 + lane];
-            e1 = W.qj[32 + lane];
+            e0 = W.qown[q0 + lane];
+            e1 = W.qj[q0 + lane];
           }
           __syncwarp();
           if (lane < nq) {
@@ -327,7 +344,7 @@ __global__ void __launch_bounds__(WT, 4) k_wca_md(const BoxDev* __restrict__ box
           __syncwarp();
         }
       }
-      if (nq > 0) wca_flush(B, S, W, wbase, pos, nq, lane);
+      if (nq > 0) wca_flush(B, S, W, wbase, pos, 0, nq, lane);
       if (valid) {
         // bond to the left (index t) and to the right (t + 1; b0 + t is bead t + 1 of S)
 #pragma unroll
