@@ -310,6 +310,7 @@ struct Engine {
   unsigned long long* d_gscan = nullptr;
   uint32_t* d_toff = nullptr;
   int* d_err = nullptr;
+  unsigned* d_done = nullptr;  // finished blocks of the launch that ends a pass
   double* d_partials = nullptr;
   bool any_beads = false;
   int wca_substeps = 0;  // most MD substeps of a box with the WCA repulsion (0: none)
@@ -318,7 +319,11 @@ struct Engine {
   // k_srd: cells per warp chosen by the launch tuner (0: by size)
   int tuned_cpw = 0;
 
-  cudaGraphExec_t gexec[3] = {nullptr, nullptr, nullptr};  // MODE_P, MODE_F, MODE_C
+  // MODE_P, MODE_F, MODE_C, and GRAPH_STEPS passes of mode F: a graph takes about
+  // 10 us to launch, which is longer than a step of a small box (16^3 cells at
+  // density 10: 10.3 us a step with a launch each).
+  cudaGraphExec_t gexec[4] = {nullptr, nullptr, nullptr, nullptr};
+  static constexpr int GRAPH_MANY = 3, GRAPH_STEPS = 16;
   bool tables_ok = false;
   bool pending = false;  // the last collision of every live box is still to do
 
@@ -334,35 +339,13 @@ struct Engine {
       CUDA_TRY(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
       own_stream = true;
     }
-    for (int m = 0; m < 3; ++m)
-      for (int v = 0; v < NVAR; ++v) {
-        const bool at = (v & 16) != 0, ang = (v & 32) != 0;
-        cells_bps[m][v] = 1;
-        if (v & 64) {
-          if (!mixed && !(v & (4 | 8 | 16 | 32)))
-            cells_bps[m][v] = srdd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, m);
-          if (mixed && !(v & (16 | 32)) && !((v & 4) && (v & (2 | 8))))
-            if (v & 8)
-              srd_bead_bps[m][v & 7] = std::max(
-                  1, srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, true, (v & 4) != 0, m));
-            cells_bps[m][v] = srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, m);
-        } else if ((v & 4) && ang) {  // warp-spread angular correction: mixed SRD without beads
-          if (mixed && !(v & (8 | 16)))
-            cells_bps[m][v] = cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, false, true, m);
-        } else if ((v & 4) && !(at && (v & 1))) {
-          cells_bps[m][v] =
-              mixed ? cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, false, m)
-                    : cells_warpd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, m);
-        } else if (!(v & 4)) {
-          cells_bps[m][v] = cells_blocks_per_sm(mixed, v, m);
-        }
-        if (cells_bps[m][v] < 1) cells_bps[m][v] = 1;
-      }
     CUDA_TRY((cudaError_t)md_bin_prepare());
     CUDA_TRY((cudaError_t)extract_prepare());
     CUDA_TRY(cudaMalloc(&d_err, sizeof(int)));
     CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), stream));
     CUDA_TRY(cudaMalloc(&d_partials, sizeof(double) * 4 * 4096));
+    CUDA_TRY(cudaMalloc(&d_done, sizeof(unsigned)));
+    CUDA_TRY(cudaMemsetAsync(d_done, 0, sizeof(unsigned), stream));
     CUDA_TRY(cudaMalloc(&d_wsync, sizeof(unsigned) * 4));
     wca_bps = std::max(1, wca_blocks_per_sm());
     // keep freed box memory cached in the pool for quick re-admission
@@ -372,6 +355,34 @@ struct Engine {
       cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
     }
     return MPCD_OK;
+  }
+
+  // Blocks per SM of a kernel variant in every mode (asked for when a box first
+  // needs the variant: there are too many to ask for all when an engine starts).
+  void prepare_variant(int v) {
+    for (int m = 0; m < 3 && cells_bps[2][v] == 0; ++m) {
+      const bool at = (v & 16) != 0, ang = (v & 32) != 0;
+      cells_bps[m][v] = 1;
+      if (v & 64) {
+        if (!mixed && !(v & (4 | 8 | 16 | 32)))
+          cells_bps[m][v] = srdd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, m);
+        if (mixed && !(v & (16 | 32)) && !((v & 4) && (v & (2 | 8))))
+          if (v & 8)
+            srd_bead_bps[m][v & 7] = std::max(
+                1, srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, true, (v & 4) != 0, m));
+          cells_bps[m][v] = srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, m);
+      } else if ((v & 4) && ang) {  // warp-spread angular correction: mixed SRD without beads
+        if (mixed && !(v & (8 | 16)))
+          cells_bps[m][v] = cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, false, true, m);
+      } else if ((v & 4) && !(at && (v & 1))) {
+        cells_bps[m][v] =
+            mixed ? cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, false, m)
+                  : cells_warpd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, m);
+      } else if (!(v & 4)) {
+        cells_bps[m][v] = cells_blocks_per_sm(mixed, v, m);
+      }
+      cells_bps[m][v] = std::max(1, cells_bps[m][v]);
+    }
   }
 
   void free_tables() {
@@ -405,6 +416,7 @@ struct Engine {
     if (d_err) cudaFree(d_err);
     if (d_partials) cudaFree(d_partials);
     if (d_wsync) cudaFree(d_wsync);
+    if (d_done) cudaFree(d_done);
     if (own_stream && stream) cudaStreamDestroy(stream);
   }
 
@@ -537,8 +549,10 @@ struct Engine {
       return MPCD_OK;
     };
     if ((rc = up(rec, d_boxes, &n_records))) return rc;
-    for (int v = 0; v < NVAR; ++v)
+    for (int v = 0; v < NVAR; ++v) {
       if ((rc = up(sp[v], d_spans[v], &n_spans[v]))) return rc;
+      if (n_spans[v] > 0) prepare_variant(v);
+    }
     if ((rc = up(bseg, d_bsegs, nullptr))) return rc;
     if ((rc = up(bst, d_bstiles, &n_bstiles))) return rc;
     if ((rc = up(bt, d_btiles, &n_btiles))) return rc;
@@ -589,30 +603,43 @@ struct Engine {
     return grid_for(items, (mode == MODE_F && tuned_grid > 0) ? std::min(tuned_grid, limit) : limit);
   }
 
+  // One pass over every box, with the record updates that end it: by the last
+  // launch itself where that is k_srd or k_srd_d (they come last), else by a
+  // kernel of their own.
   void launch_cells_all(int mode) {
+    const AfterPass none{};
+    AfterPass end{d_boxes, (int)live.size(), mode != MODE_C, mode != MODE_P, d_done};
+    int last = -1;
+    for (int v = 0; v < NVAR; ++v)
+      if (n_spans[v] > 0) last = v;
     for (int v = 0; v < NVAR; ++v) {
       if (n_spans[v] == 0) continue;
       const int grid = grid_of(v, mode);
       const bool at = (v & 16) != 0;
+      const AfterPass after = v == last ? end : none;
       if ((v & 64) && !mixed) {
         launch_srdd((v & 1) != 0, (v & 2) != 0, mode, d_boxes, d_spans[v], n_spans[v], grid,
-                    srd_cpw(), d_err, stream);
+                    srd_cpw(), after, d_err, stream);
       } else if (v & 64) {
-        launch_srd((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, mode, d_boxes, d_spans[v], n_spans[v],
-                   grid, srd_cpw(), d_err, stream);
-        if ((v & 8) && mode != MODE_P)
+        const bool beads = (v & 8) && mode != MODE_P;  // then a second launch, over their groups
+        launch_srd((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, mode, d_boxes, d_spans[v],
+                   n_spans[v], grid, srd_cpw(), beads ? none : after, d_err, stream);
+        if (beads)
           launch_srd((v & 1) != 0, (v & 2) != 0, true, (v & 4) != 0, mode, d_boxes, d_spans[v],
                      n_spans[v], grid_for(srd_bead_items(n_spans[v]), srd_bead_bps[mode][v & 7]), 32,
-                     d_err, stream);
-      } else if ((v & 4) && mixed)
+                     after, d_err, stream);
+      } else if ((v & 4) && mixed) {
         launch_cells_warp((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, (v & 32) != 0, mode,
                           d_boxes, d_spans[v], n_spans[v], grid, d_err, stream);
-      else if (v & 4)
+      } else if (v & 4) {
         launch_cells_warpd((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, mode, d_boxes,
                            d_spans[v], n_spans[v], grid, d_err, stream);
-      else
+      } else {
         launch_cells(mixed, v, mode, d_boxes, d_spans[v], n_spans[v], grid, d_err, stream);
+      }
     }
+    if (last < 64)
+      launch_after_pass(d_boxes, (int)live.size(), mode != MODE_C, mode != MODE_P, stream);
   }
 
   // What the collision of the step in the records needs beside the solvent:
@@ -630,18 +657,9 @@ struct Engine {
 
   // One pass over every live box (plain launches; captured into the graphs).
   void enqueue_pass(int mode) {
-    const int nb = (int)live.size();
-    if (nb == 0) return;
+    if (live.empty()) return;
     launch_cells_all(mode);
-    if (mode == MODE_P) {
-      launch_after_pass(d_boxes, nb, true, false, stream);
-      launch_beads();
-    } else if (mode == MODE_F) {
-      launch_after_pass(d_boxes, nb, true, true, stream);
-      launch_beads();
-    } else {
-      launch_after_pass(d_boxes, nb, false, true, stream);
-    }
+    if (mode != MODE_C) launch_beads();
   }
 
   int ensure_tables() {
@@ -655,7 +673,10 @@ struct Engine {
     if (gexec[mode]) return MPCD_OK;
     cudaGraph_t g = nullptr;
     CUDA_TRY(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
-    enqueue_pass(mode);
+    if (mode == GRAPH_MANY)
+      for (int i = 0; i < GRAPH_STEPS; ++i) enqueue_pass(MODE_F);
+    else
+      enqueue_pass(mode);
     cudaError_t e = cudaStreamEndCapture(stream, &g);
     if (e != cudaSuccess) return fail(MPCD_ECUDA, std::string("capture: ") + cudaGetErrorString(e));
     e = cudaGraphInstantiate(&gexec[mode], g, 0);
@@ -681,6 +702,10 @@ struct Engine {
       if ((rc = run_pass(MODE_P))) return rc;
       pending = true;
       n -= 1;
+    }
+    if (n >= 2 * GRAPH_STEPS) {
+      if ((rc = ensure_graph(GRAPH_MANY))) return rc;
+      for (; n >= GRAPH_STEPS; n -= GRAPH_STEPS) CUDA_TRY(cudaGraphLaunch(gexec[GRAPH_MANY], stream));
     }
     if (n > 0) {
       if ((rc = ensure_graph(MODE_F))) return rc;
@@ -784,13 +809,11 @@ struct Engine {
     pending = true;
     cudaEvent_t ev[kPhases + 1];
     for (auto& e : ev) CUDA_TRY(cudaEventCreate(&e));
-    const int nb = (int)live.size();
     for (int64_t s = 0; s < n; ++s) {
       CUDA_TRY(cudaEventRecord(ev[0], stream));
       launch_cells_all(MODE_F);
       CUDA_TRY(cudaEventRecord(ev[1], stream));
-      launch_after_pass(d_boxes, nb, true, true, stream);
-      CUDA_TRY(cudaEventRecord(ev[2], stream));
+      CUDA_TRY(cudaEventRecord(ev[2], stream));  // (the record updates are part of the pass)
       launch_beads();
       CUDA_TRY(cudaEventRecord(ev[3], stream));
       CUDA_TRY(cudaEventSynchronize(ev[3]));
@@ -1021,29 +1044,24 @@ struct Engine {
     return place(b, b->stage_r, b->stage_v, nullptr, nullptr, step);
   }
 
-  // The last step completed and reported on, the host's record current.
-  int settle() {
-    int rc = complete();
-    if (rc) return rc;
-    if ((rc = pull_records())) return rc;
-    return check_err();
-  }
-
-  // The completed state in input order, into the given device arrays or (NULL)
-  // the box's staging arrays.
+  // The last step completed, and the state in input order into the given device
+  // arrays or (NULL) the box's staging arrays; waits for them and reports device
+  // errors.
   int extract(Box* b, int32_t* cell_out, void* pos = nullptr, void* vel = nullptr) {
-    const int rc = settle();
+    const int rc = complete();
     if (rc) return rc;
     launch_extract(mixed, d_boxes + b->dev_index, pos ? pos : b->stage_r, vel ? vel : b->stage_v,
                    cell_out, (int)b->d.ncells, (int)b->nsol, b->d.xcnt, stream);
     CUDA_TRY(cudaGetLastError());
-    return MPCD_OK;
+    return check_err();
   }
 
   int download_state(Box* b, double* pos, double* vel, double* spos, double* svel, uint64_t* step) {
     // a caller that wants only the beads does not pay for the solvent
     const bool solvent = b->nsol > 0 && (pos || vel);
-    int rc = solvent ? extract(b, nullptr) : settle();
+    int rc = solvent ? extract(b, nullptr) : complete();
+    if (!rc && !solvent) rc = check_err();
+    if (!rc && step) rc = pull_records();
     if (rc) return rc;
     const size_t n3 = (size_t)b->nsol * 3;
     if (solvent) {
@@ -1067,6 +1085,7 @@ struct Engine {
   int observables(Box* b, mpcd_obs* out) {
     if (!out) return fail(MPCD_EINVAL, "out is NULL");
     int rc = extract(b, nullptr);
+    if (!rc) rc = pull_records();  // the step counter
     if (rc) return rc;
     const mpcd_params& p = b->p;
     const int nc = p.n[0] * p.n[1] * p.n[2];
@@ -1243,12 +1262,7 @@ int mpcd_get_state_device(mpcd_ctx* ctx, void* pos, void* vel) {
   if (!ctx->box->has_state) return fail(MPCD_ESTATE, "no state set");
   Engine& E = ctx->eng;
   Box* b = ctx->box;
-  // straight into the caller's arrays
-  int rc = E.extract(b, nullptr, pos, vel);
-  if (rc) return rc;
-  CUDA_TRY(cudaStreamSynchronize(E.stream));
-  CUDA_TRY(cudaGetLastError());
-  return MPCD_OK;
+  return E.extract(b, nullptr, pos, vel);  // straight into the caller's arrays
 }
 
 int mpcd_observables(mpcd_ctx* ctx, mpcd_obs* out) {

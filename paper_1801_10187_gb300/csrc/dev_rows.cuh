@@ -53,6 +53,34 @@ __device__ __forceinline__ void load_v(const RecD* p, double v[3]) {
   v[0] = b.y; v[1] = c.x; v[2] = c.y;
 }
 
+// Record updates after a pass: the output set becomes current and the consumed
+// overflow list is emptied (flip), a collision completes the step (advance).
+__device__ __forceinline__ void after_pass(BoxDev& B, int flip, int advance) {
+  if (flip) {
+    B.ovf_n[B.cur] = 0u;
+    B.cur ^= 1;
+  }
+  if (advance) B.step += 1ull;
+}
+
+// At the end of a launch: the block that finishes last does the updates of the
+// pass (the others have read the records for the last time), which saves the
+// launch of a kernel for them: 3 of 10 us a step on a box of 16^3 cells.
+__device__ __forceinline__ void finish_pass(const AfterPass& A) {
+  if (!A.boxes) return;
+  __shared__ int last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(A.done, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int b = threadIdx.x; b < A.nboxes; b += blockDim.x) after_pass(A.boxes[b], A.flip, A.advance);
+  if (threadIdx.x == 0) *A.done = 0u;
+}
+
 // Append a record to the row of cell c in the output set (or to the output
 // overflow list when the row is full).
 template <bool MIXED>

@@ -42,9 +42,9 @@ int srd_parts(int cpw) { return BLOCK / (SWARPS * cpw); }
 int srd_bead_items(int nspans) { return (nspans + SWARPS - 1) / SWARPS; }
 
 void launch_srd(bool thermo, bool force, bool beads, bool walls, int mode, const BoxDev* boxes,
-                const int2* spans, int nspans, int grid, int cpw, int* err, cudaStream_t s) {
+                const int2* spans, int nspans, int grid, int cpw, AfterPass after, int* err, cudaStream_t s) {
   if (nspans <= 0) return;
-  void* args[] = {(void*)&boxes, (void*)&spans, (void*)&nspans, (void*)&cpw, (void*)&err};
+  void* args[] = {(void*)&boxes, (void*)&spans, (void*)&nspans, (void*)&cpw, (void*)&after, (void*)&err};
   cudaLaunchKernel(srd_variant(thermo, force, beads, walls, mode), dim3(grid), dim3(SB), args,
                    srd_variant_smem(thermo, beads, mode), s);
 }

@@ -127,7 +127,7 @@ __device__ __forceinline__ void split_bits(float x, unsigned& th, unsigned& tl) 
 template <bool THERMO, int MODE, bool FORCE, bool BEADS, bool WALLS>
 __global__ void __launch_bounds__(SB, BEADS ? 6 : 7) k_srd(const BoxDev* __restrict__ boxes,
                                                const int2* __restrict__ spans, int nspans,
-                                               int cpw, int* err) {
+                                               int cpw, AfterPass after, int* err) {
   constexpr int SW = THERMO ? 1 : 2;  // windows of 32 members per chunk
   extern __shared__ __align__(16) unsigned char smem_[];
   SrdBox& H = *reinterpret_cast<SrdBox*>(smem_);
@@ -625,6 +625,7 @@ __global__ void __launch_bounds__(SB, BEADS ? 6 : 7) k_srd(const BoxDev* __restr
     }
     }
   }
+  finish_pass(after);
 }
 
 }  // namespace mpcd

@@ -121,7 +121,7 @@ __device__ __forceinline__ int2 halves(long long x) {
 template <bool THERMO, int MODE, bool FORCE>
 __global__ void __launch_bounds__(DB, 4) k_srd_d(const BoxDev* __restrict__ boxes,
                                                  const int2* __restrict__ spans, int nspans, int cpw,
-                                                 int* err) {
+                                                 AfterPass after, int* err) {
   extern __shared__ __align__(16) unsigned char smem_[];
   DBox& H = *reinterpret_cast<DBox*>(smem_);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -481,6 +481,7 @@ __global__ void __launch_bounds__(DB, 4) k_srd_d(const BoxDev* __restrict__ boxe
       a = b;
     }
   }
+  finish_pass(after);
 }
 
 template <int MODE>
@@ -505,9 +506,9 @@ int srdd_blocks_per_sm(bool thermo, bool force, int mode) {
 }
 
 void launch_srdd(bool thermo, bool force, int mode, const BoxDev* boxes, const int2* spans,
-                 int nspans, int grid, int cpw, int* err, cudaStream_t s) {
+                 int nspans, int grid, int cpw, AfterPass after, int* err, cudaStream_t s) {
   if (nspans <= 0) return;
-  void* args[] = {(void*)&boxes, (void*)&spans, (void*)&nspans, (void*)&cpw, (void*)&err};
+  void* args[] = {(void*)&boxes, (void*)&spans, (void*)&nspans, (void*)&cpw, (void*)&after, (void*)&err};
   cudaLaunchKernel(srdd_variant(thermo, force, mode), dim3(grid), dim3(DB), args, DSMEM, s);
 }
 

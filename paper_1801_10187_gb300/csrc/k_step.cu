@@ -7,6 +7,7 @@
 #include <type_traits>
 
 #include "dev_collide.cuh"
+#include "dev_rows.cuh"
 #include "dev_stream.cuh"
 #include "kernels.h"
 #include "mpcd_internal.cuh"
@@ -354,12 +355,7 @@ void launch_virtual(const BoxDev* boxes, const int2* tiles, int ntiles, cudaStre
 __global__ void k_after_pass(BoxDev* boxes, int nboxes, int flip, int advance) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= nboxes) return;
-  BoxDev& B = boxes[b];
-  if (flip) {
-    B.ovf_n[B.cur] = 0u;
-    B.cur ^= 1;
-  }
-  if (advance) B.step += 1ull;
+  after_pass(boxes[b], flip, advance);
 }
 
 // ---------------------------------------------------------------------------

@@ -49,7 +49,8 @@ int srd_blocks_per_sm(bool thermo, bool force, bool beads, bool walls, int mode)
 int srd_parts(int cpw);
 int srd_bead_items(int nspans);  // blocks' work of the bead launch
 void launch_srd(bool thermo, bool force, bool beads, bool walls, int mode, const BoxDev* boxes,
-                const int2* spans, int nspans, int grid, int cpw, int* err, cudaStream_t s);
+                const int2* spans, int nspans, int grid, int cpw, AfterPass after, int* err,
+                cudaStream_t s);
 // The FP64 model's counterpart of k_srd (k_srd_d.cu), for periodic SRD boxes
 // without solute and rows of at most SRDD_SLOTS records.
 // It pays where the latency of a tile counts and not the FP64 pipe's rate:
@@ -58,7 +59,7 @@ void launch_srd(bool thermo, bool force, bool beads, bool walls, int mode, const
 constexpr int SRDD_SLOTS = 112, SRDD_MAX_CELLS = 200000;
 int srdd_blocks_per_sm(bool thermo, bool force, int mode);
 void launch_srdd(bool thermo, bool force, int mode, const BoxDev* boxes, const int2* spans,
-                 int nspans, int grid, int cpw, int* err, cudaStream_t s);
+                 int nspans, int grid, int cpw, AfterPass after, int* err, cudaStream_t s);
 // The FP64 model's counterpart of k_cells_warp (k_cells_warp_d.cu), same conditions.
 int cells_warpd_blocks_per_sm(bool thermo, bool force, bool beads, bool at, int mode);
 void launch_cells_warpd(bool thermo, bool force, bool beads, bool at, int mode, const BoxDev* boxes,

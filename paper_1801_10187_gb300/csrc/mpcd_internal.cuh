@@ -141,6 +141,14 @@ struct BoxDev {
   int32_t pad_x;
 };
 
+// What a pass leaves to do once all its blocks are done (see finish_pass), passed
+// to its last launch; done counts finished blocks and is left at zero.
+struct AfterPass {
+  BoxDev* boxes;  // NULL: nothing
+  int nboxes, flip, advance;
+  unsigned* done;
+};
+
 // Segments for the segmented exclusive scan (cells of each box, and bead
 // counts per collision tile of each box).
 struct ScanSeg {
