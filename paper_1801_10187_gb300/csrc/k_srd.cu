@@ -6,12 +6,16 @@ namespace mpcd {
 
 template <int MODE, bool TH, bool FO>
 static void* srd_fn(bool beads, bool walls) {
-  if (walls) return (void*)k_srd<TH, MODE, true, false, true>;  // always with the force terms
-  return beads ? (void*)k_srd<TH, MODE, FO, true, false> : (void*)k_srd<TH, MODE, FO, false, false>;
+  if (walls) return (void*)k_srd<TH, MODE, true, false, true, false>;  // always with the force terms
+  return beads ? (void*)k_srd<TH, MODE, FO, true, false, false>
+               : (void*)k_srd<TH, MODE, FO, false, false, false>;
 }
 
 template <int MODE>
-static void* srd_mode(bool thermo, bool force, bool beads, bool walls) {
+static void* srd_mode(bool thermo, bool force, bool beads, bool walls, bool at) {
+  if (at && MODE != MODE_P)
+    return force ? (void*)k_srd<false, MODE, true, false, false, true>
+                 : (void*)k_srd<false, MODE, false, false, false, true>;
   // mode P only streams and bins: nothing in it depends on thermostat or beads
   if (MODE == MODE_P) return force ? srd_fn<MODE, false, true>(false, walls)
                                       : srd_fn<MODE, false, false>(false, walls);
@@ -19,18 +23,18 @@ static void* srd_mode(bool thermo, bool force, bool beads, bool walls) {
   return force ? srd_fn<MODE, false, true>(beads, walls) : srd_fn<MODE, false, false>(beads, walls);
 }
 
-static void* srd_variant(bool thermo, bool force, bool beads, bool walls, int mode) {
-  if (mode == MODE_P) return srd_mode<MODE_P>(thermo, force, beads, walls);
-  if (mode == MODE_F) return srd_mode<MODE_F>(thermo, force, beads, walls);
-  return srd_mode<MODE_C>(thermo, force, beads, walls);
+static void* srd_variant(bool thermo, bool force, bool beads, bool walls, bool at, int mode) {
+  if (mode == MODE_P) return srd_mode<MODE_P>(thermo, force, beads, walls, at);
+  if (mode == MODE_F) return srd_mode<MODE_F>(thermo, force, beads, walls, at);
+  return srd_mode<MODE_C>(thermo, force, beads, walls, at);
 }
 
 static size_t srd_variant_smem(bool thermo, bool beads, int mode) {
   return mode == MODE_P ? srd_smem(false, false) : srd_smem(thermo, beads);
 }
 
-int srd_blocks_per_sm(bool thermo, bool force, bool beads, bool walls, int mode) {
-  const void* fn = srd_variant(thermo, force, beads, walls, mode);
+int srd_blocks_per_sm(bool thermo, bool force, bool beads, bool walls, bool at, int mode) {
+  const void* fn = srd_variant(thermo, force, beads, walls, at, mode);
   const size_t smem = srd_variant_smem(thermo, beads, mode);
   cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   int nb = 0;
@@ -41,11 +45,11 @@ int srd_blocks_per_sm(bool thermo, bool force, bool beads, bool walls, int mode)
 int srd_parts(int cpw) { return BLOCK / (SWARPS * cpw); }
 int srd_bead_items(int nspans) { return (nspans + SWARPS - 1) / SWARPS; }
 
-void launch_srd(bool thermo, bool force, bool beads, bool walls, int mode, const BoxDev* boxes,
+void launch_srd(bool thermo, bool force, bool beads, bool walls, bool at, int mode, const BoxDev* boxes,
                 const int2* spans, int nspans, int grid, int cpw, AfterPass after, int* err, cudaStream_t s) {
   if (nspans <= 0) return;
   void* args[] = {(void*)&boxes, (void*)&spans, (void*)&nspans, (void*)&cpw, (void*)&after, (void*)&err};
-  cudaLaunchKernel(srd_variant(thermo, force, beads, walls, mode), dim3(grid), dim3(SB), args,
+  cudaLaunchKernel(srd_variant(thermo, force, beads, walls, at, mode), dim3(grid), dim3(SB), args,
                    srd_variant_smem(thermo, beads, mode), s);
 }
 

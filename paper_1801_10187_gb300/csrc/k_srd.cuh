@@ -3,7 +3,8 @@
 // Sec. 3.6 rotation and thermostat, algorithm "SRD collision rule").
 //
 // For SRD boxes (body force, thermostat, and solute beads or channel walls
-// allowed) whose rows hold at most SRD_SLOTS records; modes, records and results are
+// allowed), and boxes with the Andersen rule (Eq. at, Sec. 3.7; without solute),
+// whose rows hold at most SRD_SLOTS records; modes, records and results are
 // those of k_cells_warp.  A warp owns cpw consecutive cells (32, or 16, 8 or 4
 // on small boxes) and takes them in sub-tiles of at most subc cells with at
 // most SRD_SLOTS members between them.  A map in shared memory gives each
@@ -124,11 +125,11 @@ __device__ __forceinline__ void split_bits(float x, unsigned& th, unsigned& tl) 
 
 }  // namespace
 
-template <bool THERMO, int MODE, bool FORCE, bool BEADS, bool WALLS>
-__global__ void __launch_bounds__(SB, BEADS ? 6 : 7) k_srd(const BoxDev* __restrict__ boxes,
+template <bool THERMO, int MODE, bool FORCE, bool BEADS, bool WALLS, bool AT>
+__global__ void __launch_bounds__(SB, AT ? 5 : BEADS ? 6 : 7) k_srd(const BoxDev* __restrict__ boxes,
                                                const int2* __restrict__ spans, int nspans,
                                                int cpw, AfterPass after, int* err) {
-  constexpr int SW = THERMO ? 1 : 2;  // windows of 32 members per chunk
+  constexpr int SW = THERMO || AT ? 1 : 2;  // windows of 32 members per chunk
   extern __shared__ __align__(16) unsigned char smem_[];
   SrdBox& H = *reinterpret_cast<SrdBox*>(smem_);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(SB, BEADS ? 6 : 7) k_srd(const BoxDev* __restr
         }
         // the per-cell draws need only the member count: the axis (Sec. 3.6)
         // and, with the thermostat, the accepted Gamma pair (d, v), E^ = d v kT
-        if (n > 0 || nb > 0) {
+        if (!AT && (n > 0 || nb > 0)) {
           float ax[3];
           axis_of(B, B.step, (uint32_t)(c0 + lane), ax);
           W.prm[1][lane] = make_float4(ax[0], ax[1], ax[2], 0.0f);
@@ -333,38 +334,41 @@ __global__ void __launch_bounds__(SB, BEADS ? 6 : 7) k_srd(const BoxDev* __restr
         int slow = 0;  // beyond |v| < 2^10 (or NaN) the split fails: exact sums below
         unsigned hs[3] = {0u, 0u, 0u}, ls[3] = {0u, 0u, 0u};
         long long Shh = 0, Shl = 0, Sll = 0;  // thermostat: sums of H^2, H L and L^2
+        auto sum_cells = [&] {
 #pragma unroll (THERMO ? 1 : 2)
-        for (int k = part; k < nrowC; k += 1 << plog) {
-          const float4 x = sv[s0C + k];
-          const float xv[3] = {x.x, x.y, x.z};
-          slow |= !(fabsf(x.x) < 1024.0f && fabsf(x.y) < 1024.0f && fabsf(x.z) < 1024.0f);
+          for (int k = part; k < nrowC; k += 1 << plog) {
+            const float4 x = sv[s0C + k];
+            const float xv[3] = {x.x, x.y, x.z};
+            slow |= !(fabsf(x.x) < 1024.0f && fabsf(x.y) < 1024.0f && fabsf(x.z) < 1024.0f);
 #pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            unsigned th, tl;
-            split_bits(xv[q], th, tl);
-            hs[q] += th;
-            ls[q] += tl;
-            if (THERMO) {  // Sec. 3.5: the kinetic energy in the same pass, exactly
-              const int h = (int)(th - MAGIC_BITS), l = (int)(tl - MAGIC_BITS);
-              Shh += (long long)h * h;
-              Shl += (long long)h * l;
-              Sll += (long long)l * l;
+            for (int q = 0; q < 3; ++q) {
+              unsigned th, tl;
+              split_bits(xv[q], th, tl);
+              hs[q] += th;
+              ls[q] += tl;
+              if (THERMO) {  // Sec. 3.5: the kinetic energy in the same pass, exactly
+                const int h = (int)(th - MAGIC_BITS), l = (int)(tl - MAGIC_BITS);
+                Shh += (long long)h * h;
+                Shl += (long long)h * l;
+                Sll += (long long)l * l;
+              }
             }
           }
-        }
-        for (int d = 1; d < (1 << plog); d <<= 1) {
-          slow |= __shfl_xor_sync(FULL, slow, d);
+          for (int d = 1; d < (1 << plog); d <<= 1) {
+            slow |= __shfl_xor_sync(FULL, slow, d);
 #pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            hs[q] += __shfl_xor_sync(FULL, hs[q], d);
-            ls[q] += __shfl_xor_sync(FULL, ls[q], d);
+            for (int q = 0; q < 3; ++q) {
+              hs[q] += __shfl_xor_sync(FULL, hs[q], d);
+              ls[q] += __shfl_xor_sync(FULL, ls[q], d);
+            }
+            if (THERMO) {
+              Shh += __shfl_xor_sync(FULL, Shh, d);
+              Shl += __shfl_xor_sync(FULL, Shl, d);
+              Sll += __shfl_xor_sync(FULL, Sll, d);
+            }
           }
-          if (THERMO) {
-            Shh += __shfl_xor_sync(FULL, Shh, d);
-            Shl += __shfl_xor_sync(FULL, Shl, d);
-            Sll += __shfl_xor_sync(FULL, Sll, d);
-          }
-        }
+        };
+        sum_cells();
 
         // ---- per cell: u (Sec. 3.5), then E_k and xi ----
         if (part == 0 && cc < b && (nC > 0 || nbC > 0)) {
@@ -447,6 +451,52 @@ __global__ void __launch_bounds__(SB, BEADS ? 6 : 7) k_srd(const BoxDev* __restr
           }
           W.prm[0][cc] = make_float4(u[0], u[1], u[2], xi);
         }
+        if (AT) {
+          // Eq. at: every member's random velocity takes the place of its own,
+          // which only the sums needed; dbar = sum dv / n the same way
+          __syncwarp();
+          for (int m = lane; m < cnt; m += 32) {
+            const float tg = sv[m].w;
+            float dv[3];
+            at_draw(B, B.step, __float_as_uint(tg), 0u, B.sig_f, dv);
+            sv[m] = make_float4(dv[0], dv[1], dv[2], tg);
+          }
+          __syncwarp();
+          slow = 0;
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            hs[q] = 0u;
+            ls[q] = 0u;
+          }
+          sum_cells();
+          if (cc < b && part == 0 && nC > 0) {
+            const unsigned magic = (unsigned)nrowC * MAGIC_BITS;
+            const float M = H.m * small_to_float(nC);
+            long long Qd[3] = {0, 0, 0};
+            auto add_dv = [&](float x, float y, float z) {
+              Qd[0] += fix32_rne(x);
+              Qd[1] += fix32_rne(y);
+              Qd[2] += fix32_rne(z);
+            };
+            if (slow)
+              for (int k = 0; k < nrowC; ++k) add_dv(sv[s0C + k].x, sv[s0C + k].y, sv[s0C + k].z);
+            if (nC > K)
+              for_overflow(c0 + cc, [&](const RecF* p) {
+                float dv[3];
+                at_draw(B, B.step, p->tag, 0u, B.sig_f, dv);
+                add_dv(dv[0], dv[1], dv[2]);
+              });
+            float dbar[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+              const float D = H.m * (slow ? i64_to_float(Qd[q])
+                                          : split_sum_to_float((int)(hs[q] - magic),
+                                                               (int)(ls[q] - magic), Qd[q]));
+              dbar[q] = (D * 0x1p-32f) / M;
+            }
+            W.prm[1][cc] = make_float4(dbar[0], dbar[1], dbar[2], 0.0f);
+          }
+        }
         __syncwarp();
         if (BEADS && gnb > 0) {  // collide the beads with their cell's parameters
           for_beads(a, b, [&](int j, int lc) {
@@ -472,14 +522,20 @@ __global__ void __launch_bounds__(SB, BEADS ? 6 : 7) k_srd(const BoxDev* __restr
       auto advance = [&](float x[3], float w[3], int o) -> uint32_t {
         if (MODE != MODE_P) {
           const float4 pa = W.prm[0][o], pb = W.prm[1][o];
-          const float nn[3] = {pb.x, pb.y, pb.z};
-          const float uu[3] = {pa.x, pa.y, pa.z};
-          float d[3], rr[3];
+          if constexpr (AT) {  // Eq. at; w is the random velocity
+            w[0] = (pa.x + w[0]) - pb.x;
+            w[1] = (pa.y + w[1]) - pb.y;
+            w[2] = (pa.z + w[2]) - pb.z;
+          } else {
+            const float nn[3] = {pb.x, pb.y, pb.z};
+            const float uu[3] = {pa.x, pa.y, pa.z};
+            float d[3], rr[3];
 #pragma unroll
-          for (int q = 0; q < 3; ++q) d[q] = w[q] - uu[q];
-          rotate(nn, H.ca, H.sa, H.omc, d, rr);
+            for (int q = 0; q < 3; ++q) d[q] = w[q] - uu[q];
+            rotate(nn, H.ca, H.sa, H.omc, d, rr);
 #pragma unroll
-          for (int q = 0; q < 3; ++q) w[q] = uu[q] + (THERMO ? pa.w * rr[q] : rr[q]);
+            for (int q = 0; q < 3; ++q) w[q] = uu[q] + (THERMO ? pa.w * rr[q] : rr[q]);
+          }
         }
         if constexpr (MODE == MODE_C) {
           return 0u;
@@ -617,6 +673,7 @@ __global__ void __launch_bounds__(SB, BEADS ? 6 : 7) k_srd(const BoxDev* __restr
           float x[3], w[3];
           uint32_t tg;
           load_rec(p, x, w, tg);
+          if (AT && MODE != MODE_P) at_draw(B, B.step, tg, 0u, B.sig_f, w);
           const uint32_t c = advance(x, w, lane);
           if constexpr (MODE == MODE_C) store_rec(p, x, w, tg);
           else emit(x, w, tg, c, atomicAdd(&H.cnt_out[c], 1u));
