@@ -1099,8 +1099,9 @@ struct Engine {
     }
     ObsCells oc;
     char* base = (char*)b->obs;
-    oc.mass = (long long*)base;
-    oc.p = oc.mass + nc;
+    oc.mass = b->nbead > 0 ? (long long*)base : nullptr;
+    oc.mass_fix = std::llrint(p.mass * 4294967296.0);
+    oc.p = (long long*)base + nc;
     oc.k = oc.p + 3 * (size_t)nc;
     oc.cnt = (uint32_t*)(oc.k + nc);
     oc.ncells = nc;

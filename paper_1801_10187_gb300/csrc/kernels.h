@@ -109,7 +109,8 @@ void launch_virtual(const BoxDev* boxes, const int2* tiles, int ntiles, cudaStre
 // ---- observables (k_obs.cu) ----
 struct ObsCells {
   uint32_t* cnt;
-  long long* mass;
+  long long* mass;     // NULL: the count times mass_fix = rne(m 2^32) (no beads)
+  long long mass_fix;
   long long* p;  // 3 per cell
   long long* k;
   int ncells;
