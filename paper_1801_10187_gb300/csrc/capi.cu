@@ -366,11 +366,11 @@ struct Engine {
       if (v & 64) {
         if (!mixed && !(v & (4 | 8 | 16 | 32)))
           cells_bps[m][v] = srdd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, m);
-        if (mixed && !(v & 32) && !(at && (v & (1 | 4 | 8))) && !((v & 4) && (v & (2 | 8))))
+        if (mixed && !(at && (v & (1 | 4 | 8 | 32))) && !(ang && (v & (4 | 8))) && !((v & 4) && (v & (2 | 8))))
           if (v & 8)
             srd_bead_bps[m][v & 7] = std::max(
-                1, srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, true, (v & 4) != 0, false, m));
-          cells_bps[m][v] = srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, at, m);
+                1, srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, true, (v & 4) != 0, false, false, m));
+          cells_bps[m][v] = srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, at, ang, m);
       } else if ((v & 4) && ang) {  // warp-spread angular correction: mixed SRD without beads
         if (mixed && !(v & (8 | 16)))
           cells_bps[m][v] = cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, false, true, m);
@@ -576,8 +576,9 @@ struct Engine {
   // Boxes that k_srd (mixed) or k_srd_d (FP64) steps.
   bool on_srd(const BoxDev& d) const {
     if (!mixed && (d.walls || d.nbead > 0 || d.K > SRDD_SLOTS || d.ncells > SRDD_MAX_CELLS)) return false;
-    if (d.collision == RULE_AT && (!mixed || d.nbead > 0)) return false;
-    return !d.angular && d.K <= SRD_SLOTS &&
+    if (d.collision == RULE_AT && (!mixed || d.nbead > 0 || d.angular)) return false;
+    if (d.angular && !mixed) return false;
+    return d.K <= SRD_SLOTS &&
            std::max(d.n[0], std::max(d.n[1], d.n[2])) < (1 << 22);
   }
 
@@ -623,10 +624,10 @@ struct Engine {
                     srd_cpw(), after, d_err, stream);
       } else if (v & 64) {
         const bool beads = (v & 8) && mode != MODE_P;  // then a second launch, over their groups
-        launch_srd((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, at, mode, d_boxes, d_spans[v],
+        launch_srd((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, at, (v & 32) != 0, mode, d_boxes, d_spans[v],
                    n_spans[v], grid, srd_cpw(), beads ? none : after, d_err, stream);
         if (beads)
-          launch_srd((v & 1) != 0, (v & 2) != 0, true, (v & 4) != 0, false, mode, d_boxes, d_spans[v],
+          launch_srd((v & 1) != 0, (v & 2) != 0, true, (v & 4) != 0, false, false, mode, d_boxes, d_spans[v],
                      n_spans[v], grid_for(srd_bead_items(n_spans[v]), srd_bead_bps[mode][v & 7]), 32,
                      after, d_err, stream);
       } else if ((v & 4) && mixed) {

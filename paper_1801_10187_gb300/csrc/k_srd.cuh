@@ -3,9 +3,10 @@
 // Sec. 3.6 rotation and thermostat, algorithm "SRD collision rule").
 //
 // For SRD boxes (body force, thermostat, and solute beads or channel walls
-// allowed), and boxes with the Andersen rule (Eq. at, Sec. 3.7; without solute),
-// whose rows hold at most SRD_SLOTS records; modes, records and results are
-// those of k_cells_warp.  A warp owns cpw consecutive cells (32, or 16, 8 or 4
+// allowed), and without solute and walls boxes with the Andersen rule (AT; Eq. at,
+// Sec. 3.7) or SRD with the angular-momentum correction (ANG), whose rows hold at
+// most SRD_SLOTS records; modes, records and results are those of k_cells_warp.
+// A warp owns cpw consecutive cells (32, or 16, 8 or 4
 // on small boxes) and takes them in sub-tiles of at most subc cells with at
 // most SRD_SLOTS members between them.  A map in shared memory gives each
 // member, numbered in cell order, its cell and place in the row.
@@ -24,6 +25,21 @@
 // enter a cell's sums as their number and exact totals, which k_virtual
 // (k_step.cu) has left in the box for the pending step; a particle that would
 // cross a wall bounces back.  k_cells draws them inside the cell's one thread.
+//
+// The Andersen rule draws a member's velocity once, in place of the staged one, which
+// only the sums needed (k_cells_warp draws those beyond its cache twice).  us a
+// step, k_cells_warp -> k_srd: 6.0 10^6 particles at density 10 313 -> 208, at
+// density 20 1340 -> 387, 16^3 cells 30 -> 13.
+//
+// The angular correction adds a pass over the staged members for their angular
+// momentum and inertia, added up by the lanes of a cell as the sums are; the members
+// then get omega x r as they are collided.  k_cells_warp reads the members of that
+// pass by itself, at two blocks an SM.  us a step, k_cells_warp -> k_srd: 64^3 cells
+// at density 10 161 -> 111 (thermostat 180 -> 137), 80^3 at density 20 888 -> 355
+// (1002 -> 445), 50^3 at density 5 53 -> 42 (61 -> 50), 16^3 37 -> 13 (41 -> 15).
+//
+// Both run at five blocks an SM and chunks of one window: the registers of their
+// longer members' phase would spill at seven.
 //
 // Solute boxes take two launches in modes F and C: one over the bead groups
 // without beads, one (BEADS) over those with.  In one launch the bead code's
@@ -55,6 +71,7 @@
 // two issues in ten on fetches), so chunks are one window there (SW), which
 // measured 236 us against 259 us for two.
 #pragma once
+#include "dev_angular.cuh"
 #include "dev_bin.cuh"
 #include "dev_collide.cuh"
 #include "dev_rows.cuh"
@@ -86,6 +103,7 @@ struct SrdBox {
   uint32_t* ovf_cell_out;
   uint32_t* ovf_n_out;
   int ovf_cap;
+  float sf[3], clo[3], chi[3];  // angular: the collision step's shift (rel_pos_f)
   int zb;  // walls: the bottom layer that the wall can cut in the collision step, -1: none
 };
 
@@ -101,15 +119,19 @@ struct SrdBeads {
   unsigned long long X[3][32], E[32];
   int nb[32], pad[4];
 };
+// Angular correction: centre of mass in the cell's frame and omega per cell.
+struct SrdAng {
+  float4 rc[32], om[32];
+};
 constexpr unsigned MAGIC_BITS = 0x4B400000u;  // bits of 1.5 2^23
 
 __host__ __device__ constexpr size_t srd_head() { return (sizeof(SrdBox) + 15) & ~(size_t)15; }
-__host__ __device__ constexpr size_t srd_warp(bool thermo, bool beads) {
+__host__ __device__ constexpr size_t srd_warp(bool thermo, bool beads, bool ang) {
   return (size_t)SRD_SLOTS * 34 + sizeof(SrdWarp) + (thermo ? sizeof(SrdThermo) : 0) +
-         (beads ? sizeof(SrdBeads) : 0);
+         (beads ? sizeof(SrdBeads) : 0) + (ang ? sizeof(SrdAng) : 0);
 }
-constexpr size_t srd_smem(bool thermo, bool beads) {
-  return srd_head() + SWARPS * srd_warp(thermo, beads);
+constexpr size_t srd_smem(bool thermo, bool beads, bool ang) {
+  return srd_head() + SWARPS * srd_warp(thermo, beads, ang);
 }
 
 // The two roundings of split32 (rne(x 2^32) = H 2^20 + L) with their magic
@@ -125,21 +147,22 @@ __device__ __forceinline__ void split_bits(float x, unsigned& th, unsigned& tl) 
 
 }  // namespace
 
-template <bool THERMO, int MODE, bool FORCE, bool BEADS, bool WALLS, bool AT>
-__global__ void __launch_bounds__(SB, AT ? 5 : BEADS ? 6 : 7) k_srd(const BoxDev* __restrict__ boxes,
-                                               const int2* __restrict__ spans, int nspans,
-                                               int cpw, AfterPass after, int* err) {
-  constexpr int SW = THERMO || AT ? 1 : 2;  // windows of 32 members per chunk
+template <bool THERMO, int MODE, bool FORCE, bool BEADS, bool WALLS, bool AT, bool ANG>
+__global__ void __launch_bounds__(SB, AT || ANG ? 5 : BEADS ? 6 : 7)
+    k_srd(const BoxDev* __restrict__ boxes, const int2* __restrict__ spans, int nspans, int cpw,
+          AfterPass after, int* err) {
+  constexpr int SW = THERMO || AT || ANG ? 1 : 2;  // windows of 32 members per chunk
   extern __shared__ __align__(16) unsigned char smem_[];
   SrdBox& H = *reinterpret_cast<SrdBox*>(smem_);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  unsigned char* wp = smem_ + srd_head() + wid * srd_warp(THERMO, BEADS);
+  unsigned char* wp = smem_ + srd_head() + wid * srd_warp(THERMO, BEADS, ANG);
   float4* sv = reinterpret_cast<float4*>(wp);                             // staged (v, tag)
   float4* sr = sv + SRD_SLOTS;                                             // staged (r, pad)
   unsigned short* map = reinterpret_cast<unsigned short*>(sr + SRD_SLOTS); // place in the row << 5 | cell
   SrdWarp& W = *reinterpret_cast<SrdWarp*>(wp + (size_t)SRD_SLOTS * 34);
   SrdThermo& TS = *reinterpret_cast<SrdThermo*>(&W + 1);
   SrdBeads& BS = *reinterpret_cast<SrdBeads*>(wp + (size_t)SRD_SLOTS * 34 + sizeof(SrdWarp) + (THERMO ? sizeof(SrdThermo) : 0));
+  SrdAng& AG = *reinterpret_cast<SrdAng*>(wp + srd_warp(THERMO, BEADS, false));
   // a block's work: a part of a 256-cell span (its warps next to each other), or,
   // with beads, SWARPS spans, one to a warp
   const int parts = BEADS ? 1 : BLOCK / (SWARPS * cpw);
@@ -168,6 +191,11 @@ __global__ void __launch_bounds__(SB, AT ? 5 : BEADS ? 6 : 7) k_srd(const BoxDev
           H.out[q] = s < 0 ? B.n[q] : -1;
           H.in[q] = s < 0 ? 0 : B.n[q] - 1;
           if (WALLS && q == 2) H.bias[q] += 1;  // layers 0 .. n_z + 1, no wrap
+        }
+        if (ANG && MODE != MODE_P) {
+          long long S[3];
+          shift_units(B, B.step, S);
+          shift_thresholds(q == 0 ? S[0] : q == 1 ? S[1] : S[2], H.sf[q], H.clo[q], H.chi[q]);
         }
       } else if (threadIdx.x == 32) {
         H.dt = B.dt_f; H.ca = B.ca_f; H.sa = B.sa_f; H.omc = B.omc_f; H.m = B.m_f;
@@ -334,6 +362,13 @@ __global__ void __launch_bounds__(SB, AT ? 5 : BEADS ? 6 : 7) k_srd(const BoxDev
         int slow = 0;  // beyond |v| < 2^10 (or NaN) the split fails: exact sums below
         unsigned hs[3] = {0u, 0u, 0u}, ls[3] = {0u, 0u, 0u};
         long long Shh = 0, Shl = 0, Sll = 0;  // thermostat: sums of H^2, H L and L^2
+        unsigned qh[3] = {0u, 0u, 0u}, ql[3] = {0u, 0u, 0u};  // angular: of the positions
+        // angular: position in the cell's frame (|x| < 2: its split never fails)
+        auto rel = [&](const float4& y, float x[3]) {
+          x[0] = rel_pos_f(y.x, H.sf[0], H.clo[0], H.chi[0]);
+          x[1] = rel_pos_f(y.y, H.sf[1], H.clo[1], H.chi[1]);
+          x[2] = rel_pos_f(y.z, H.sf[2], H.clo[2], H.chi[2]);
+        };
         auto sum_cells = [&] {
 #pragma unroll (THERMO ? 1 : 2)
           for (int k = part; k < nrowC; k += 1 << plog) {
@@ -353,6 +388,17 @@ __global__ void __launch_bounds__(SB, AT ? 5 : BEADS ? 6 : 7) k_srd(const BoxDev
                 Sll += (long long)l * l;
               }
             }
+            if (ANG) {
+              float x[3];
+              rel(sr[s0C + k], x);
+#pragma unroll
+              for (int q = 0; q < 3; ++q) {
+                unsigned th, tl;
+                split_bits(x[q], th, tl);
+                qh[q] += th;
+                ql[q] += tl;
+              }
+            }
           }
           for (int d = 1; d < (1 << plog); d <<= 1) {
             slow |= __shfl_xor_sync(FULL, slow, d);
@@ -360,6 +406,10 @@ __global__ void __launch_bounds__(SB, AT ? 5 : BEADS ? 6 : 7) k_srd(const BoxDev
             for (int q = 0; q < 3; ++q) {
               hs[q] += __shfl_xor_sync(FULL, hs[q], d);
               ls[q] += __shfl_xor_sync(FULL, ls[q], d);
+              if (ANG) {
+                qh[q] += __shfl_xor_sync(FULL, qh[q], d);
+                ql[q] += __shfl_xor_sync(FULL, ql[q], d);
+              }
             }
             if (THERMO) {
               Shh += __shfl_xor_sync(FULL, Shh, d);
@@ -451,6 +501,111 @@ __global__ void __launch_bounds__(SB, AT ? 5 : BEADS ? 6 : 7) k_srd(const BoxDev
           }
           W.prm[0][cc] = make_float4(u[0], u[1], u[2], xi);
         }
+        if (ANG) {
+          // ---- angular-momentum correction: centre of mass, then Pi omega = dL ----
+          if (cc < b && part == 0 && nC > 0) {
+            const unsigned magic = (unsigned)nrowC * MAGIC_BITS;
+            long long Qo[3] = {0, 0, 0};
+            if (nC > K)
+              for_overflow(c0 + cc, [&](const RecF* p) {
+                float x[3];
+                rel(reinterpret_cast<const float4*>(p)[1], x);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) Qo[q] += fix32_rne(x[q]);
+              });
+            float rc[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q)
+              rc[q] = (split_sum_to_float((int)(qh[q] - magic), (int)(ql[q] - magic), Qo[q]) * 0x1p-32f) /
+                      small_to_float(nC);
+            AG.rc[cc] = make_float4(rc[0], rc[1], rc[2], 0.0f);
+          }
+          __syncwarp();
+          // r_c x (v - v') and the inertia-tensor entries of a member of this
+          // lane's cell, v' by the same operations as below
+          auto terms = [&](const float4& a4, const float4& b4, float tm[9]) {
+            const float4 pa = W.prm[0][cc], pb = W.prm[1][cc], c = AG.rc[cc];
+            const float v[3] = {a4.x, a4.y, a4.z}, nn[3] = {pb.x, pb.y, pb.z}, uu[3] = {pa.x, pa.y, pa.z};
+            float x[3], d[3], rr[3], dv[3];
+            rel(b4, x);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) d[q] = v[q] - uu[q];
+            rotate(nn, H.ca, H.sa, H.omc, d, rr);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) dv[q] = v[q] - (uu[q] + (THERMO ? pa.w * rr[q] : rr[q]));
+            const float rc[3] = {x[0] - c.x, x[1] - c.y, x[2] - c.z};
+            tm[0] = rc[1] * dv[2] - rc[2] * dv[1];
+            tm[1] = rc[2] * dv[0] - rc[0] * dv[2];
+            tm[2] = rc[0] * dv[1] - rc[1] * dv[0];
+            tm[3] = rc[1] * rc[1] + rc[2] * rc[2];
+            tm[4] = rc[0] * rc[1];
+            tm[5] = rc[0] * rc[2];
+            tm[6] = rc[0] * rc[0] + rc[2] * rc[2];
+            tm[7] = rc[1] * rc[2];
+            tm[8] = rc[0] * rc[0] + rc[1] * rc[1];
+          };
+          unsigned ah[9] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u}, al[9] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+          int far = 0;  // a term of 1024 or more (or NaN): exact sums below
+#pragma unroll 1
+          for (int k = part; k < nrowC; k += 1 << plog) {
+            float tm[9];
+            terms(sv[s0C + k], sr[s0C + k], tm);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+              unsigned th, tl;
+              far |= !(fabsf(tm[q]) < 1024.0f);
+              split_bits(tm[q], th, tl);
+              ah[q] += th;
+              al[q] += tl;
+            }
+          }
+          for (int d = 1; d < (1 << plog); d <<= 1) {
+            far |= __shfl_xor_sync(FULL, far, d);
+#pragma unroll
+            for (int q = 0; q < 9; ++q) {
+              ah[q] += __shfl_xor_sync(FULL, ah[q], d);
+              al[q] += __shfl_xor_sync(FULL, al[q], d);
+            }
+          }
+          if (cc < b && part == 0 && nC > 0) {
+            const unsigned magic = (unsigned)nrowC * MAGIC_BITS;
+            float tot[9];
+            if (__builtin_expect(far || nC > K, 0)) {
+              long long Lo[9];
+#pragma unroll
+              for (int q = 0; q < 9; ++q)
+                Lo[q] = far ? 0ll : (long long)(int)(ah[q] - magic) * 1048576LL + (int)(al[q] - magic);
+              auto add = [&](const float4& a4, const float4& b4) {
+                float tm[9];
+                terms(a4, b4, tm);
+#pragma unroll
+                for (int q = 0; q < 9; ++q) Lo[q] += fix32_rne(tm[q]);
+              };
+              if (far)
+                for (int k = 0; k < nrowC; ++k) add(sv[s0C + k], sr[s0C + k]);
+              if (nC > K)
+                for_overflow(c0 + cc, [&](const RecF* p) {
+                  add(reinterpret_cast<const float4*>(p)[0], reinterpret_cast<const float4*>(p)[1]);
+                });
+#pragma unroll
+              for (int q = 0; q < 9; ++q) tot[q] = i64_to_float(Lo[q]);
+            } else {
+#pragma unroll
+              for (int q = 0; q < 9; ++q)
+                tot[q] = split_sum_to_float((int)(ah[q] - magic), (int)(al[q] - magic), 0);
+            }
+            float dL[3], P6[6], om[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) dL[k] = H.m * (tot[k] * 0x1p-32f);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+              const float e = H.m * (tot[3 + k] * 0x1p-32f);
+              P6[k] = (k == 1 || k == 2 || k == 4) ? -e : e;
+            }
+            solve_omega<float>(nC, P6, dL, om);
+            AG.om[cc] = make_float4(om[0], om[1], om[2], 0.0f);
+          }
+        }
         if (AT) {
           // Eq. at: every member's random velocity takes the place of its own,
           // which only the sums needed; dbar = sum dv / n the same way
@@ -535,6 +690,15 @@ __global__ void __launch_bounds__(SB, AT ? 5 : BEADS ? 6 : 7) k_srd(const BoxDev
             rotate(nn, H.ca, H.sa, H.omc, d, rr);
 #pragma unroll
             for (int q = 0; q < 3; ++q) w[q] = uu[q] + (THERMO ? pa.w * rr[q] : rr[q]);
+            if (ANG) {  // v'' = v' + omega x r_c
+              const float4 c = AG.rc[o], om = AG.om[o];
+              const float rc[3] = {rel_pos_f(x[0], H.sf[0], H.clo[0], H.chi[0]) - c.x,
+                                   rel_pos_f(x[1], H.sf[1], H.clo[1], H.chi[1]) - c.y,
+                                   rel_pos_f(x[2], H.sf[2], H.clo[2], H.chi[2]) - c.z};
+              w[0] = w[0] + (om.y * rc[2] - om.z * rc[1]);
+              w[1] = w[1] + (om.z * rc[0] - om.x * rc[2]);
+              w[2] = w[2] + (om.x * rc[1] - om.y * rc[0]);
+            }
           }
         }
         if constexpr (MODE == MODE_C) {

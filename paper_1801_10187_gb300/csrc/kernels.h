@@ -39,16 +39,17 @@ void launch_cells_warp(bool thermo, bool force, bool beads, bool at, bool ang, i
                        const BoxDev* boxes, const int2* spans, int nspans, int grid, int* err,
                        cudaStream_t s);
 // The same step for mixed SRD boxes (walls: with channel walls, then without
-// beads) and mixed boxes with the Andersen rule (at, without beads), with rows of at most SRD_SLOTS records (k_srd.cu).  cpw: cells per warp (32, 16,
+// beads) and, without walls and beads, mixed boxes with the Andersen rule (at) or the
+// angular correction (ang), with rows of at most SRD_SLOTS records (k_srd.cu).  cpw: cells per warp (32, 16,
 // 8 or 4); a 256-cell span is then taken in srd_parts(cpw) parts, one block
 // each: grid sizes count parts.  A solute box takes a launch without beads, over
 // the bead groups that hold none, and one with (cpw 32), over the others; mode P
 // only the first.  SRD_MIN_WARPS: see srd_cpw() in capi.cu.
 constexpr int SRD_MIN_WARPS = 16, SRDD_MIN_WARPS = 6;
-int srd_blocks_per_sm(bool thermo, bool force, bool beads, bool walls, bool at, int mode);
+int srd_blocks_per_sm(bool thermo, bool force, bool beads, bool walls, bool at, bool ang, int mode);
 int srd_parts(int cpw);
 int srd_bead_items(int nspans);  // blocks' work of the bead launch
-void launch_srd(bool thermo, bool force, bool beads, bool walls, bool at, int mode, const BoxDev* boxes,
+void launch_srd(bool thermo, bool force, bool beads, bool walls, bool at, bool ang, int mode, const BoxDev* boxes,
                 const int2* spans, int nspans, int grid, int cpw, AfterPass after, int* err,
                 cudaStream_t s);
 // The FP64 model's counterpart of k_srd (k_srd_d.cu), for periodic SRD boxes

@@ -62,3 +62,120 @@ def test_beads_in_narrow_sub_tiles():
     np.testing.assert_array_equal(got[1], ref.vel)
     np.testing.assert_allclose(got[2], ref.spos, rtol=0, atol=1e-10)
     np.testing.assert_allclose(got[3], ref.svel, rtol=0, atol=1e-10 * max(1.0, np.abs(ref.svel).max()))
+
+
+RULES = [dict(collision="at"), dict(angular=True), dict(angular=True, thermostat=True)]
+
+
+@pytest.mark.parametrize("rule", RULES)
+@pytest.mark.parametrize("n,rho", [((5, 3, 2), 1), ((23, 17, 9), 6), ((9, 4, 5), 13), ((6, 5, 4), 36),
+                                   ((3, 2, 2), 121), ((3, 2, 2), 122), ((40, 40, 50), 3)])
+def test_other_rules_match_the_oracle(n, rho, rule):
+    s = inputs.solvent(n, rho, seed=rho + 5, mixed=True)
+    box = pkg.Box(n=n, seed=rho + 5, precision="mixed", body_force=(0.01, -0.02, 0.03), **rule)
+    box.set_state(s.pos, s.vel, step=7)
+    box.step(3)
+    pos, vel, _, _, step = box.get_state()
+    box.close()
+    kw = dict(rule)
+    if kw.get("collision") == "at":
+        kw["collision"] = oracle.AT
+    ref = oracle.State(s.pos.copy(), s.vel.copy(), step=7)
+    oracle.step(oracle.Params(n=n, seed=rho + 5, precision=oracle.MIXED, g=(0.01, -0.02, 0.03), **kw), ref, 3)
+    assert step == ref.step
+    np.testing.assert_array_equal(pos, ref.pos)
+    np.testing.assert_array_equal(vel, ref.vel)
+
+
+@pytest.mark.parametrize("rule", RULES)
+def test_other_rules_with_large_velocities_and_a_full_row(rule):
+    """The exact sums (|v|, dv or a term of the correction beyond 1024) and the overflow list."""
+    n = (4, 4, 4)
+    s = inputs.solvent(n, 6, seed=3, mixed=True)
+    rng = np.random.default_rng(4)
+    pos, vel = s.pos.copy(), s.vel.copy()
+    pos[:120] = (1.3 + 0.4 * rng.random((120, 3))).astype(np.float32)
+    vel[::9] = rng.uniform(1024.0, 1500.0, vel[::9].shape).astype(np.float32)
+    kT = 4e6 if rule.get("collision") == "at" else 1.0
+    box = pkg.Box(n=n, seed=3, precision="mixed", kT=kT, **rule)
+    box.set_state(pos, vel)
+    box.step(1)
+    p, v, *_ = box.get_state()
+    box.close()
+    kw = dict(rule)
+    if kw.get("collision") == "at":
+        kw["collision"] = oracle.AT
+    ref = oracle.State(pos.copy(), vel.copy())
+    oracle.step(oracle.Params(n=n, seed=3, precision=oracle.MIXED, kT=kT, **kw), ref, 1)
+    np.testing.assert_array_equal(p, ref.pos)
+    np.testing.assert_array_equal(v, ref.vel)
+
+
+@pytest.mark.parametrize("n,rho,density", [((5, 4, 1), 10, 10.0), ((7, 5, 2), 3, 0.0), ((9, 7, 3), 30, 45.5),
+                                           ((40, 40, 8), 5, 5.0)])
+def test_walls_match_the_oracle(n, rho, density):
+    """Channel walls, from one layer of cells on: cells exact; velocities to the rounding
+    that double log and cospi of the virtual particles leave in float (2e-6 a step, as the
+    other wall tests state)."""
+    s = inputs.solvent(n, rho, seed=5, mixed=True)
+    kw = dict(n=n, seed=5, thermostat=True, walls_z=True, virt_density=density)
+    box = pkg.Box(precision="mixed", body_force=(0.01, 0.02, 0.0), **kw)
+    box.set_state(s.pos, s.vel)
+    box.step(4)
+    pos, vel, *_ = box.get_state()
+    cells, counts = box.last_cells()
+    box.close()
+    ref = oracle.State(s.pos.copy(), s.vel.copy())
+    kw["virt_density"] = density or float(rho)  # (0: the library's default, N / V)
+    rc, rk = oracle.step(oracle.Params(precision=oracle.MIXED, g=(0.01, 0.02, 0.0), **kw), ref, 4,
+                         want_cells=True)
+    np.testing.assert_array_equal(cells, rc)
+    np.testing.assert_array_equal(counts, rk)
+    scale = np.maximum(np.linalg.norm(ref.vel, axis=1), 1.0)
+    assert (np.linalg.norm(vel - ref.vel, axis=1) / scale).max() <= 8e-6
+    assert np.all((pos[:, 2] >= 0) & (pos[:, 2] < n[2]))
+
+
+@pytest.mark.parametrize("precision,rho", [("mixed", 6), ("mixed", 700), ("fp64", 6)])
+def test_read_out_of_large_and_small_states(precision, rho):
+    """The state comes back in input order through buckets of 4096 (FP64: 2048)
+    tags, the last one partly filled, as through the direct scatter; overflowing
+    rows and cell numbers included."""
+    n = (61, 43, 47) if rho == 6 else (11, 10, 10)
+    s = inputs.solvent(n, rho, seed=2, mixed=precision == "mixed")
+    pos = s.pos.copy()
+    pos[:500] = pos[0]  # one cell beyond its row
+    box = pkg.Box(n=n, seed=2, precision=precision)
+    box.set_state(pos, s.vel)
+    p, v, *_ = box.get_state()
+    np.testing.assert_array_equal(p, pos)
+    np.testing.assert_array_equal(v, s.vel)
+    box.step(1)
+    p, v, *_ = box.get_state()
+    cells, counts = box.last_cells()
+    box.close()
+    assert np.array_equal(np.bincount(cells, minlength=len(counts)), counts)
+    d = np.abs(p - (pos + 0.1 * s.vel))
+    L = np.array(n, dtype=float)
+    assert np.minimum(d, np.abs(d - L)).max() < 1e-4
+
+
+def test_many_steps_in_one_call_equal_single_steps():
+    """Runs long enough for the graph of many steps, beads and all, against steps
+    one at a time."""
+    n = (6, 6, 6)
+    s = inputs.solvent(n, 5, seed=12, mixed=True)
+    sp, sv = inputs.chains(n, 4, 8, 0.5, bead_mass=5.0, seed=13)
+    got = []
+    for split in ([1] * 75, [75], [3, 33, 39]):
+        box = pkg.Box(n=n, seed=12, precision="mixed", thermostat=True, chain_len=8, md_substeps=5,
+                      solute_mass=5.0, bond_k=300.0, bond_r0=0.5)
+        box.set_state(s.pos, s.vel, sp, sv)
+        for k in split:
+            box.step(k)
+        got.append(box.get_state())
+        box.close()
+    for g in got[1:]:
+        assert g[4] == got[0][4] == 75
+        for a, b in zip(g[:4], got[0][:4]):
+            np.testing.assert_array_equal(a, b)
