@@ -79,7 +79,7 @@ size_t footprint_bytes(const mpcd_params& p, int64_t nsol, int64_t nbead) {
   b += 2 * (size_t)std::max<int64_t>(nsol, 1) * (rec_size(mixed) + 4);     // overflow lists
   b += (size_t)nsol * 6 * elem_size(mixed);                               // staging (r, v)
   b += (size_t)xbuckets(mixed, nsol) * XCNT_STRIDE * sizeof(uint32_t);    // read-out buckets
-  if (mixed && p.walls_z) b += 2 * (size_t)p.n[0] * p.n[1] * (4 * sizeof(long long) + 4);
+  if (mixed && p.walls_z) b += 4 * (size_t)p.n[0] * p.n[1] * (4 * sizeof(long long) + 4);
   if (nbead > 0) {
     b += (size_t)nbead * (9 * sizeof(double) + 2 * sizeof(int32_t) + sizeof(uint64_t) +
                           sizeof(uint32_t));
@@ -310,7 +310,9 @@ struct Engine {
   unsigned long long* d_gscan = nullptr;
   uint32_t* d_toff = nullptr;
   int* d_err = nullptr;
-  unsigned* d_done = nullptr;  // finished blocks of the launch that ends a pass
+  unsigned* d_done = nullptr;  // finished blocks of the launch that ends a pass, of k_virtual
+  cudaStream_t side = nullptr;  // k_virtual beside the fused pass, between two events
+  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   double* d_partials = nullptr;
   bool any_beads = false;
   int wca_substeps = 0;  // most MD substeps of a box with the WCA repulsion (0: none)
@@ -344,8 +346,8 @@ struct Engine {
     CUDA_TRY(cudaMalloc(&d_err, sizeof(int)));
     CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), stream));
     CUDA_TRY(cudaMalloc(&d_partials, sizeof(double) * 4 * 4096));
-    CUDA_TRY(cudaMalloc(&d_done, sizeof(unsigned)));
-    CUDA_TRY(cudaMemsetAsync(d_done, 0, sizeof(unsigned), stream));
+    CUDA_TRY(cudaMalloc(&d_done, 2 * sizeof(unsigned)));
+    CUDA_TRY(cudaMemsetAsync(d_done, 0, 2 * sizeof(unsigned), stream));
     CUDA_TRY(cudaMalloc(&d_wsync, sizeof(unsigned) * 4));
     wca_bps = std::max(1, wca_blocks_per_sm());
     // keep freed box memory cached in the pool for quick re-admission
@@ -411,6 +413,9 @@ struct Engine {
   ~Engine() {
     if (stream) cudaStreamSynchronize(stream);
     drop_graphs();
+    if (side) cudaStreamDestroy(side);  // (joined to stream at every pass)
+    if (ev_fork) cudaEventDestroy(ev_fork);
+    if (ev_join) cudaEventDestroy(ev_join);
     for (Box* b : slots) release_box(b);
     free_tables();
     if (d_err) cudaFree(d_err);
@@ -558,6 +563,11 @@ struct Engine {
     if ((rc = up(bt, d_btiles, &n_btiles))) return rc;
     if ((rc = up(mt, d_mdtiles, &n_mdtiles))) return rc;
     if ((rc = up(vt, d_vtiles, &n_vtiles))) return rc;
+    if (n_vtiles > 0 && !side) {
+      CUDA_TRY(cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming));
+      CUDA_TRY(cudaEventCreateWithFlags(&ev_join, cudaEventDisableTiming));
+      CUDA_TRY(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
+    }
     if ((rc = up(wt, d_wtiles, &n_wtiles))) return rc;
     if (n_bstiles > 0) {
       CUDA_TRY(cudaMalloc(&d_tsum, sizeof(uint32_t) * n_bstiles));
@@ -644,10 +654,8 @@ struct Engine {
       launch_after_pass(d_boxes, (int)live.size(), mode != MODE_C, mode != MODE_P, stream);
   }
 
-  // What the collision of the step in the records needs beside the solvent:
-  // virtual wall particles; solute MD substeps and bead grouping.
+  // Solute: MD substeps and bead grouping for the step in the records.
   void launch_beads() {
-    launch_virtual(d_boxes, d_vtiles, n_vtiles, stream);
     if (!any_beads) return;
     if (wca_substeps > 0)
       launch_wca_md(d_boxes, d_wtiles, n_wtiles, wca_substeps, wca_bps * nsm, d_wsync, d_err, stream);
@@ -660,7 +668,18 @@ struct Engine {
   // One pass over every live box (plain launches; captured into the graphs).
   void enqueue_pass(int mode) {
     if (live.empty()) return;
+    // Virtual wall particles: the first pass needs them before its collision can
+    // follow; a fused pass draws those of the next step beside itself.
+    if (n_vtiles > 0 && mode == MODE_F) {
+      cudaEventRecord(ev_fork, stream);
+      cudaStreamWaitEvent(side, ev_fork, 0);
+      launch_virtual(d_boxes, (int)live.size(), d_vtiles, n_vtiles, 0, d_done + 1, side);
+      cudaEventRecord(ev_join, side);
+    }
     launch_cells_all(mode);
+    if (n_vtiles > 0 && mode == MODE_F) cudaStreamWaitEvent(stream, ev_join, 0);
+    if (n_vtiles > 0 && mode == MODE_P)
+      launch_virtual(d_boxes, (int)live.size(), d_vtiles, n_vtiles, 1, d_done + 1, stream);
     if (mode != MODE_C) launch_beads();
   }
 
@@ -813,6 +832,8 @@ struct Engine {
     for (auto& e : ev) CUDA_TRY(cudaEventCreate(&e));
     for (int64_t s = 0; s < n; ++s) {
       CUDA_TRY(cudaEventRecord(ev[0], stream));
+      if (n_vtiles > 0)
+        launch_virtual(d_boxes, (int)live.size(), d_vtiles, n_vtiles, 0, d_done + 1, stream);
       launch_cells_all(MODE_F);
       CUDA_TRY(cudaEventRecord(ev[1], stream));
       CUDA_TRY(cudaEventRecord(ev[2], stream));  // (the record updates are part of the pass)
@@ -943,8 +964,10 @@ struct Engine {
     if ((rc = alloc(b, d.xcnt, (size_t)xbuckets(mixed, nsol) * XCNT_STRIDE))) return rc;
     if (d.walls && on_srd(d)) {
       const size_t cut = 2 * (size_t)d.n[0] * d.n[1];
-      if ((rc = alloc(b, d.virt_n, cut))) return rc;
-      if ((rc = alloc(b, d.virt_sum, 4 * cut))) return rc;
+      for (int k = 0; k < 2; ++k) {
+        if ((rc = alloc(b, d.virt_n[k], cut))) return rc;
+        if ((rc = alloc(b, d.virt_sum[k], 4 * cut))) return rc;
+      }
     }
     if ((rc = alloc_bytes(b, b->stage_r, (size_t)nsol * 3 * es))) return rc;
     if ((rc = alloc_bytes(b, b->stage_v, (size_t)nsol * 3 * es))) return rc;
@@ -1004,7 +1027,7 @@ struct Engine {
   int place(Box* b, const void* dpos, const void* dvel, const double* spos, const double* svel,
             uint64_t step) {
     BoxDev& d = b->d;
-    d.step = step;
+    d.step = d.virt_step = step;
     d.cur = 0;
     BoxDev* tmp = nullptr;
     CUDA_TRY(cudaMallocAsync((void**)&tmp, sizeof(BoxDev), stream));

@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(SB, AT || ANG ? 5 : BEADS ? 6 : 7)
           const int side = cz == H.zb ? 0 : cz == H.zb + B.n[2] ? 1 : -1;
           if (side >= 0) {
             virt = side * nxy + (c0 + lane - cz * nxy);
-            nb = B.virt_n[virt];  // (walls exclude beads)
+            nb = B.virt_n[B.step & 1][virt];  // (walls exclude beads)
           }
         }
         // the per-cell draws need only the member count: the axis (Sec. 3.6)
@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(SB, AT || ANG ? 5 : BEADS ? 6 : 7)
             }
           }
           const bool bd = BEADS && gnb > 0, vp = WALLS && nbC > 0;
-          const long long* vs = vp ? B.virt_sum + 4 * (size_t)virtC : nullptr;
+          const long long* vs = vp ? B.virt_sum[B.step & 1] + 4 * (size_t)virtC : nullptr;
           float M = H.m * small_to_float(nC);
           if (BEADS) M = M + (small_to_float(nbC) * B.Mb_f + 0.0f * H.m);
           if (WALLS) M = M + (0.0f * B.Mb_f + small_to_float(nbC) * H.m);

@@ -102,10 +102,13 @@ void launch_bead_scatter(const BoxDev* boxes, const int2* tiles, int ntiles, cud
 // (after modes F and C).
 void launch_after_pass(BoxDev* boxes, int nboxes, bool flip, bool advance, cudaStream_t s);
 
-// Virtual wall particles of the pending step, for the boxes of the tiles (box,
-// first of VIRT_CELLS cells of its two wall-cut layers); mixed boxes on k_srd.
+// Virtual wall particles of the boxes of the tiles (box, first of VIRT_CELLS
+// cells of its two wall-cut layers; mixed boxes on k_srd), of the step in the
+// records (fresh) or of the step virt_step; virt_step is then the one after it.
+// done: a word at zero, left at zero.
 constexpr int VIRT_CELLS = 8;
-void launch_virtual(const BoxDev* boxes, const int2* tiles, int ntiles, cudaStream_t s);
+void launch_virtual(BoxDev* boxes, int nboxes, const int2* tiles, int ntiles, int fresh,
+                    unsigned* done, cudaStream_t s);
 
 // ---- observables (k_obs.cu) ----
 struct ObsCells {

@@ -97,11 +97,13 @@ struct BoxDev {
   void* ovf_rec[2];     // overflow records
   uint32_t* ovf_cell[2];
   uint32_t* ovf_n;      // two counters
-  // channel walls, mixed model: virtual particles of the pending step in the
-  // two layers a wall can cut, n_x n_y cells each: their number, exact sums of
-  // rne(m v 2^32) and of rne(m v^2 2^32) (four words a cell)
-  int32_t* virt_n;
-  long long* virt_sum;
+  // channel walls, mixed model: virtual particles of a step in the two layers a
+  // wall can cut, n_x n_y cells each: their number, exact sums of rne(m v 2^32)
+  // and of rne(m v^2 2^32) (four words a cell); of the pending step and the one
+  // after it, by the step's last bit
+  int32_t* virt_n[2];
+  long long* virt_sum[2];
+  unsigned long long virt_step;  // the step k_virtual draws next
   uint32_t* xcnt;       // records per tag bucket of a state read-out
   // solute
   double* spos;
