@@ -1124,11 +1124,19 @@ struct Engine {
     ObsCells oc;
     char* base = (char*)b->obs;
     oc.mass = b->nbead > 0 ? (long long*)base : nullptr;
-    oc.mass_fix = std::llrint(p.mass * 4294967296.0);
+    oc.mass_one = p.mass * 4294967296.0;
     oc.p = (long long*)base + nc;
     oc.k = oc.p + 3 * (size_t)nc;
     oc.cnt = (uint32_t*)(oc.k + nc);
     oc.ncells = nc;
+    oc.p_unit = 0x1p-32;
+    oc.v_scale = 0.0f;
+    if (mixed && b->nbead == 0 && p.mass > 0x1p-100 && p.mass < 0x1p100) {
+      int e;
+      const double f = std::frexp(p.mass, &e);  // in [1/2, 1)
+      oc.v_scale = std::ldexp(1.0f, f == 0.5 ? e - 1 : e);
+      oc.p_unit = p.mass / (double)oc.v_scale * 0x1p-32;
+    }
     CUDA_TRY(cudaMemsetAsync(b->obs, 0, need, stream));
     const BoxDev* rec = d_boxes + b->dev_index;
     const int ntot = (int)(b->nsol + b->nbead);

@@ -113,11 +113,13 @@ void launch_virtual(BoxDev* boxes, int nboxes, const int2* tiles, int ntiles, in
 // ---- observables (k_obs.cu) ----
 struct ObsCells {
   uint32_t* cnt;
-  long long* mass;     // NULL: the count times mass_fix = rne(m 2^32) (no beads)
-  long long mass_fix;
-  long long* p;  // 3 per cell
+  long long* mass;   // NULL: the count times mass_one = m 2^32 (no beads)
+  double mass_one;
+  long long* p;  // 3 per cell, in units of p_unit
   long long* k;
   int ncells;
+  double p_unit;  // 2^-32; with v_scale m 2^-32 / v_scale
+  float v_scale;  // not 0 (mixed, no beads): p sums rne(v v_scale 2^32), a power of two in [m, 2 m)
 };
 void launch_obs_particles(bool mixed, const BoxDev* box, const void* pos, const void* vel,
                           ObsCells oc, double* partials, int nblocks, cudaStream_t s);

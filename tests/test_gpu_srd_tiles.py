@@ -179,3 +179,34 @@ def test_many_steps_in_one_call_equal_single_steps():
         assert g[4] == got[0][4] == 75
         for a, b in zip(g[:4], got[0][:4]):
             np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("mass", [1.0, 0.3, 1e-3, 4096.0, 5000.0])
+def test_observables_of_any_mass(mass):
+    """Mixed observables, summed from velocities and multiplied by the mass at the end, against
+    plain NumPy: the totals to the rounding of a double sum; the cells' temperatures to their
+    fixed point: 2^-32 m' a particle and component (m <= m' < 2 m, m' |v| < 2 max(m |v|)), over
+    M (n - 1) >= 2 m, times the centre's speed.  Speeds that leave the split range included."""
+    n = (9, 7, 5)
+    s = inputs.solvent(n, 6, seed=9, mixed=True)
+    vel = (s.vel / np.sqrt(mass)).astype(np.float32)
+    vel[:40] *= 3000.0
+    box = pkg.Box(n=n, seed=9, precision="mixed", mass=mass)
+    box.set_state(s.pos, vel.astype(np.float64))
+    ob = box.observables()
+    box.close()
+    v = vel.astype(np.float64)
+    np.testing.assert_allclose(ob["P"], mass * v.sum(axis=0), atol=1e-13 * mass * np.abs(v).sum(), rtol=0)
+    np.testing.assert_allclose(ob["KE"], 0.5 * mass * (v * v).sum(), rtol=1e-13)
+    c = np.minimum(np.floor(s.pos), np.array(n) - 1).astype(int)
+    c = c[:, 0] + n[0] * (c[:, 1] + n[1] * c[:, 2])
+    cnt = np.bincount(c, minlength=np.prod(n))
+    ok = cnt >= 2
+    u = np.stack([np.bincount(c, v[:, k], cnt.size) for k in range(3)], 1)[ok] / cnt[ok, None]
+    full = np.zeros((cnt.size, 3))
+    full[ok] = u
+    T = np.bincount(c, mass * ((v - full[c]) ** 2).sum(1), cnt.size)[ok] / (3.0 * (cnt[ok] - 1))
+    err = 2.0 * cnt[ok] * 2.0 ** -32 * (1.0 + np.linalg.norm(u, axis=1) * 2) / (3.0 * (cnt[ok] - 1))
+    kk = np.bincount(c, mass * (v * v).sum(1), cnt.size)[ok] / (3.0 * (cnt[ok] - 1))
+    assert abs(ob["T_cell_mean"] - T.mean()) <= err.mean() + 1e-13 * kk.mean()
+    assert ob["occupied_cells"] == int((cnt > 0).sum())
