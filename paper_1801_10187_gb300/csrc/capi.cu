@@ -82,7 +82,7 @@ size_t footprint_bytes(const mpcd_params& p, int64_t nsol, int64_t nbead) {
   if (mixed && p.walls_z) b += 4 * (size_t)p.n[0] * p.n[1] * (4 * sizeof(long long) + 4);
   if (nbead > 0) {
     b += (size_t)nbead * (9 * sizeof(double) + 2 * sizeof(int32_t) + sizeof(uint64_t) +
-                          sizeof(uint32_t));
+                          2 * sizeof(uint32_t));
     b += (size_t)ng * sizeof(uint32_t) + (size_t)(ng + 1) * sizeof(uint32_t);
     if (p.lj_epsilon > 0.0)  // neighbour list: buckets, next, key, count, list, build r, forces
       b += (size_t)(2 * ((nbead + PTILE - 1) / PTILE) * PTILE) * sizeof(int32_t) +
@@ -981,6 +981,7 @@ struct Engine {
       if ((rc = alloc(b, d.bgv, (size_t)nbead * 3))) return rc;
       if ((rc = alloc(b, d.bcount, (size_t)d.nctiles))) return rc;
       if ((rc = alloc(b, d.bstart, (size_t)d.nctiles + 1))) return rc;
+      if ((rc = alloc(b, d.bgroup, (size_t)nbead))) return rc;
       CUDA_TRY(cudaMemsetAsync(d.bcount, 0, sizeof(uint32_t) * d.nctiles, stream));
       CUDA_TRY(cudaMemsetAsync(d.bstart, 0, sizeof(uint32_t) * (d.nctiles + 1), stream));
       if (p.lj_epsilon > 0.0) {  // non-bonded WCA repulsion (Sec. 4.3 reading)
@@ -1028,6 +1029,7 @@ struct Engine {
             uint64_t step) {
     BoxDev& d = b->d;
     d.step = d.virt_step = step;
+    d.nbgroup = 0u;
     d.cur = 0;
     BoxDev* tmp = nullptr;
     CUDA_TRY(cudaMallocAsync((void**)&tmp, sizeof(BoxDev), stream));

@@ -60,7 +60,10 @@ __device__ __forceinline__ void after_pass(BoxDev& B, int flip, int advance) {
     B.ovf_n[B.cur] = 0u;
     B.cur ^= 1;
   }
-  if (advance) B.step += 1ull;
+  if (advance) {
+    B.step += 1ull;
+    B.nbgroup = 0u;
+  }
 }
 
 // At the end of a launch: the block that finishes last does the updates of the

@@ -49,7 +49,7 @@ int srd_blocks_per_sm(bool thermo, bool force, bool beads, bool walls, bool at, 
 }
 
 int srd_parts(int cpw) { return BLOCK / (SWARPS * cpw); }
-int srd_bead_items(int nspans) { return (nspans + SWARPS - 1) / SWARPS; }
+int srd_bead_items(int nspans) { return nspans * (BLOCK / (SWARPS * BEAD_TILE)); }
 
 void launch_srd(bool thermo, bool force, bool beads, bool walls, bool at, bool ang, int mode, const BoxDev* boxes,
                 const int2* spans, int nspans, int grid, int cpw, AfterPass after, int* err, cudaStream_t s) {

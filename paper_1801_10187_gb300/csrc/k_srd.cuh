@@ -45,6 +45,9 @@
 // without beads, one (BEADS) over those with.  In one launch the bead code's
 // registers cost every cell: 2.69 ms a step at 7.8 10^7 particles with 2000 chains
 // and the thermostat, against 2.14 ms for the same box without beads.
+// The second takes its groups from k_bead_scatter's list, one a warp by turns: with
+// a span of 256 cells to a warp it lasted as long as the warp with the most groups
+// (2.61 against 2.46 ms for the step with its bead MD).
 //
 // What bounds it: neither DRAM (44 % of its peak at 10^7 particles) nor the
 // issue slots (53 %) nor the L1 pipe (63 %), but the chain count -> stage ->
@@ -164,15 +167,15 @@ __global__ void __launch_bounds__(SB, AT || ANG ? 5 : BEADS ? 6 : 7)
   SrdBeads& BS = *reinterpret_cast<SrdBeads*>(wp + (size_t)SRD_SLOTS * 34 + sizeof(SrdWarp) + (THERMO ? sizeof(SrdThermo) : 0));
   SrdAng& AG = *reinterpret_cast<SrdAng*>(wp + srd_warp(THERMO, BEADS, false));
   // a block's work: a part of a 256-cell span (its warps next to each other), or,
-  // with beads, SWARPS spans, one to a warp
-  const int parts = BEADS ? 1 : BLOCK / (SWARPS * cpw);
-  const int items = BEADS ? (nspans + SWARPS - 1) / SWARPS : nspans * parts;
+  // with beads, SWARPS of the groups that hold some, one to a warp
+  const int parts = BLOCK / (SWARPS * cpw);
+  const int ngroups = BEADS ? min((int)boxes[spans[0].x].nbgroup, boxes[spans[0].x].nbead) : 0;  // (one box)
+  const int items = BEADS ? (ngroups + SWARPS - 1) / SWARPS : nspans * parts;
   int box_of_params = -1;
   const unsigned lt = (1u << lane) - 1u;
   for (int it = blockIdx.x; it < items; it += gridDim.x) {
     const int sp = it / parts, part = it - sp * parts;
-    // (with beads there is one box: a warp without a span takes the last's box)
-    const int2 tt = spans[BEADS ? min(it * SWARPS + wid, nspans - 1) : sp];
+    const int2 tt = spans[BEADS ? 0 : sp];
     const BoxDev& B = boxes[tt.x];
     if (tt.x != box_of_params) {  // block-uniform
       __syncthreads();
@@ -220,20 +223,14 @@ __global__ void __launch_bounds__(SB, AT || ANG ? 5 : BEADS ? 6 : 7)
       box_of_params = tt.x;
     }
     // Solute boxes: the groups of 32 cells that hold beads are left to a second
-    // launch (BEADS), which takes only them; so the bead code and its registers
-    // weigh on no other cell.
-    unsigned groups = 1u;
-    if (BEADS) {
-      const int g = tt.y / BEAD_TILE + lane;
-      groups = __ballot_sync(FULL, it * SWARPS + wid < nspans && lane < BLOCK / BEAD_TILE &&
-                                       g < B.nctiles && B.bstart[g + 1] != B.bstart[g]);
-    }
-    for (; groups; groups &= groups - 1) {
-    const int c0 = BEADS ? tt.y + BEAD_TILE * (__ffs(groups) - 1) : tt.y + (part * SWARPS + wid) * cpw;
-    if (c0 >= B.ncells) break;  // warp-uniform
+    // launch (BEADS), which takes only them, from k_bead_scatter's list; so the bead
+    // code and its registers weigh on no other cell.
+    if (BEADS && it * SWARPS + wid >= ngroups) continue;
+    const int c0 = BEADS ? BEAD_TILE * (int)B.bgroup[it * SWARPS + wid] : tt.y + (part * SWARPS + wid) * cpw;
+    if (c0 >= B.ncells) continue;  // warp-uniform
     if (!BEADS && MODE != MODE_P && B.nbead > 0) {
       const int g = c0 / BEAD_TILE;
-      if (B.bstart[g + 1] != B.bstart[g]) break;
+      if (B.bstart[g + 1] != B.bstart[g]) continue;
     }
     const int K = H.K;
     uint32_t n = 0u;
@@ -255,7 +252,7 @@ __global__ void __launch_bounds__(SB, AT || ANG ? 5 : BEADS ? 6 : 7)
       if (lane >= d) incl += y;
     }
     const int N = __shfl_sync(FULL, incl, 31);
-    if (N == 0 && gnb == 0) continue;  // (the next group)
+    if (N == 0 && gnb == 0) continue;
     RecF* rows = H.rows_cur + (size_t)c0 * K;
     // f(record) for the members of cell c in the overflow list (rare)
     auto for_overflow = [&](int c, auto&& f) {
@@ -843,7 +840,6 @@ __global__ void __launch_bounds__(SB, AT || ANG ? 5 : BEADS ? 6 : 7)
           else emit(x, w, tg, c, atomicAdd(&H.cnt_out[c], 1u));
         });
       a = b;
-    }
     }
   }
   finish_pass(after);

@@ -253,14 +253,16 @@ __global__ void __launch_bounds__(BLOCK) k_scan_down(const ScanSeg* __restrict__
 // ---------------------------------------------------------------------------
 // Beads: border[bstart[group] + slot] = bead.
 // ---------------------------------------------------------------------------
-__global__ void k_bead_scatter(const BoxDev* __restrict__ boxes, const int2* __restrict__ tiles,
+__global__ void k_bead_scatter(BoxDev* boxes, const int2* __restrict__ tiles,
                                int ntiles) {
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int2 tt = tiles[tile];
-    const BoxDev& B = boxes[tt.x];
+    BoxDev& B = boxes[tt.x];
     const int b1 = min(tt.y + PTILE, B.nbead);
     for (int b = tt.y + threadIdx.x; b < b1; b += blockDim.x) {
       const uint64_t k = B.bkey[b];
+      if ((uint32_t)k == 0u)  // the group's first bead
+        B.bgroup[min(atomicAdd(&B.nbgroup, 1u), (uint32_t)B.nbead - 1u)] = (uint32_t)(k >> 32);
       const uint32_t slot = B.bstart[(uint32_t)(k >> 32)] + (uint32_t)k;
       B.border[slot] = (uint32_t)b;
       B.bgc[slot] = B.bcell[b];
@@ -403,7 +405,7 @@ void launch_scan(const ScanSeg* segs, const int2* tiles, int ntiles, uint32_t* t
   k_scan_down<<<grid, BLOCK, 0, s>>>(segs, tiles, ntiles, toff);
 }
 
-void launch_bead_scatter(const BoxDev* boxes, const int2* tiles, int ntiles, cudaStream_t s) {
+void launch_bead_scatter(BoxDev* boxes, const int2* tiles, int ntiles, cudaStream_t s) {
   if (ntiles <= 0) return;
   k_bead_scatter<<<ntiles, BLOCK, 0, s>>>(boxes, tiles, ntiles);
 }

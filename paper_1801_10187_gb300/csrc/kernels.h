@@ -48,7 +48,7 @@ void launch_cells_warp(bool thermo, bool force, bool beads, bool at, bool ang, i
 constexpr int SRD_MIN_WARPS = 16, SRDD_MIN_WARPS = 6;
 int srd_blocks_per_sm(bool thermo, bool force, bool beads, bool walls, bool at, bool ang, int mode);
 int srd_parts(int cpw);
-int srd_bead_items(int nspans);  // blocks' work of the bead launch
+int srd_bead_items(int nspans);  // most blocks' work of the bead launch
 void launch_srd(bool thermo, bool force, bool beads, bool walls, bool at, bool ang, int mode, const BoxDev* boxes,
                 const int2* spans, int nspans, int grid, int cpw, AfterPass after, int* err,
                 cudaStream_t s);
@@ -97,7 +97,7 @@ void launch_md_bin(const BoxDev* boxes, const int2* tiles, int ntiles, int chain
                    int threads, int* err, cudaStream_t s);
 void launch_scan(const ScanSeg* segs, const int2* tiles, int ntiles, uint32_t* tsum,
                  unsigned long long* gscan, uint32_t* toff, int grid, cudaStream_t s);
-void launch_bead_scatter(const BoxDev* boxes, const int2* tiles, int ntiles, cudaStream_t s);
+void launch_bead_scatter(BoxDev* boxes, const int2* tiles, int ntiles, cudaStream_t s);
 // flip: the output set becomes current (after modes P and F); advance: step += 1
 // (after modes F and C).
 void launch_after_pass(BoxDev* boxes, int nboxes, bool flip, bool advance, cudaStream_t s);
