@@ -54,9 +54,11 @@ METRIC = "MPCD particle-steps/s"
 # the 50M+ particle mixed-precision box: 7.8e7 particles, thermostat, solute
 DEFAULT_WORKLOAD = "srd-250c-rho5-mixed-solute"
 UNIT = "particle-steps/s"
-# kernels launched per step: the fused cell kernel and the record update; the
-# solute adds MD + bead grouping, 3 bead-scan phases and the bead scatter
-LAUNCHES_PER_STEP = 2
+# kernels launched per step: k_srd and k_srd_d, which do the record update
+# themselves, take one launch, the other cell kernels two with the update; the
+# solute takes two (k_srd without and with beads, or the cell kernel and the
+# update), MD + bead grouping, 3 bead-scan phases and the bead scatter, and one
+# more for the MD with the repulsion
 LAUNCHES_PER_STEP_SOLUTE = 7
 
 
@@ -380,12 +382,15 @@ def main():
     dom = "fused_step"
     dom_ms = phases[dom]
     achieved = step_bytes * s.pos.shape[0] / (dom_ms * 1e-3) / 1e9
-    # the warp-spread kernel runs mixed-model boxes without walls
-    if cfg.get("angular") and not (cfg["precision"] == "mixed"
-                                   and cfg.get("collision", "srd") == "srd"):
-        kname = "k_cells"  # one thread per cell
+    # k_srd runs the mixed model's boxes (k_cells, one thread per cell, the
+    # Andersen rule with the angular correction); FP64 boxes of this size run
+    # k_cells_warp_d, with the angular correction k_cells
+    at = cfg.get("collision", "srd") == "at"
+    if cfg["precision"] == "mixed":
+        kname = "k_cells" if cfg.get("angular") and at else "k_srd"
     else:
-        kname = "k_cells_warp" if cfg["precision"] == "mixed" else "k_cells_warp_d"
+        small = int(np.prod(cfg["n"])) <= 200000 and not cfg.get("n_chains") and not at
+        kname = ("k_cells" if cfg.get("angular") else "k_srd_d" if small else "k_cells_warp_d")
     traffic = kernel_traffic(kname, args.workload)
     roofline = {"bound": "hbm", "kernel": f"{kname} (collide t + stream/bin t+1)",
                 "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
@@ -442,9 +447,11 @@ def main():
         rate, sample, dt, nsteps = oracle_rate(cfg, 20.0)
         cpu = {"value": rate, "unit": UNIT, "cores": 1, "kind": "oracle", "sample": sample}
 
-    per_step = LAUNCHES_PER_STEP_SOLUTE if cfg.get("n_chains") else LAUNCHES_PER_STEP
-    if cfg.get("lj_epsilon"):  # neighbour-list build (3), first force, 3 per MD substep
-        per_step += 4 + 3 * cfg["md_substeps"]
+    per_step = 1 if kname in ("k_srd", "k_srd_d") else 2
+    if cfg.get("n_chains"):
+        per_step = LAUNCHES_PER_STEP_SOLUTE
+    if cfg.get("lj_epsilon"):
+        per_step += 1
     launches = per_step * K
     config["l2"] = (f"state {s.pos.shape[0] * 6 * es / 1e6:.0f} MB > 129 MB L2 (inputs larger "
                     "than L2; no flush)")
@@ -674,8 +681,8 @@ def _run_batch(pkg, torch, stream, sampler, args, cfg, K, W, rank, world, dist):
                     "d2h_bytes_per_step": len(specs) * 96 / K,
                     "note": "add_thermal (states drawn on device) + warm-up + K steps + "
                             "observables of every box, wall clock"},
-            "gpu_launches": 2 * K,
-            "roofline": {"bound": "hbm", "kernel": "k_cells_warp (all boxes in one launch)",
+            "gpu_launches": K,
+            "roofline": {"bound": "hbm", "kernel": "k_srd (all boxes in one launch)",
                          "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
                          "traffic": None, "peak_source": src,
                          "alg_bytes_per_particle": step_bytes},

@@ -245,7 +245,7 @@ class Box:
     def tune(self, steps_per_candidate=2):
         """Launch tuner (mpcd_tune): returns (blocks per SM or -1, ms per
         step of the choice, steps the simulation advanced, pass-2 chunk
-        depth, cells per warp)."""
+        depth (always 3), cells per warp)."""
         return _tune(lib().mpcd_tune, self._ctx, steps_per_candidate)
 
     def get_state(self):
