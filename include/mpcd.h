@@ -71,7 +71,7 @@ typedef enum { MPCD_FP64 = 0, MPCD_MIXED = 1 } mpcd_precision;
  * angular momentum; a two-member or collinear cell takes omega = 2 dL /
  * tr(Pi).  The mixed model sums in int64 fixed point and solves in float.
  * Not with walls or solute (EINVAL).  Mixed-model SRD boxes take it in the
- * fused warp-spread pass; the Andersen rule and FP64 on a kernel with one
+ * fused pass; the Andersen rule and FP64 on a kernel with one
  * thread per cell (slower; same results). */
 typedef enum { MPCD_SRD = 0, MPCD_AT = 1 } mpcd_collision;
 

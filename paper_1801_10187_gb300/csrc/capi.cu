@@ -739,9 +739,8 @@ struct Engine {
   // Launch tuner.  The paper tunes its kernels' launch parameters at run time
   // on real steps (Sec. 3.5, Sec. 4).  Here each candidate of the fused pass
   // -- grid (1 .. occupancy-limit blocks per SM, and one block per span part)
-  // times, for the mixed SRD variants, the cells per warp and pass-2 chunk
-  // depth (32 cells with 2, 3 or 4 windows of members in flight; 16 and 8
-  // cells with 3) -- runs `reps` real steps, timed with CUDA events on the
+  // times, for k_srd and k_srd_d, the cells per warp (32, 16 or 8)
+  // -- runs `reps` real steps, timed with CUDA events on the
   // stream; the fastest is kept and the step graph re-captured.  Results do
   // not depend on the candidate: the mixed model's cell sums are exact, the
   // FP64 ones differ at rounding.
