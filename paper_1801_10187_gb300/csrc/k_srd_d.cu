@@ -6,19 +6,22 @@
 // For periodic SRD boxes without solute, of at most SRDD_MAX_CELLS cells, whose
 // rows hold at most SRDD_SLOTS records; modes, records and results (to rounding)
 // are those of k_cells_warp_d.  An FP64 warp instruction holds GB300's FP64 pipe for 16 cycles,
-// in which an SM issues 64 others, so k_cells_warp_d (77 % of the pipe busy) is
-// bound by its 28 FP64 instructions a particle.  Here a sub-tile of cells shares
-// one exponent E with |v| < 2^E for all its members, and a velocity becomes the
-// 60-bit integer V = v 2^(59 - E), truncated:
+// in which an SM issues 64 others, so k_cells_warp_d (82 % of the pipe busy) is
+// bound by its 28 FP64 instructions a particle.  Here a cell has an exponent E
+// with |v| < 2^E for all its members, and a velocity becomes the 60-bit integer
+// V = v 2^(59 - E), truncated:
 //   sums     Sum V per cell, exact (two 64-bit words a component)
 //   cell     the axis and the rotation matrix R (in double, then as integers
 //            R 2^62) for the warp's cells at once, one a lane, before the sums;
 //            u = Sum V / n in double, then as an integer U
 //   members  V' = U + R (V - U) in 32 x 32 -> 64 bit products of signed halves;
 //            what is dropped (low x low) is below 3 units of 2^(E - 59)
-// V resolves the largest component of the sub-tile to 2^-59, 64 times finer
-// than a double's rounding of it, so the only rounding of the size of the FP64
-// path's is the one of V' back to double; streaming is the same fma.  With the
+// V resolves the cell's largest component to 2^-59, 64 times finer than a
+// double's rounding of it, and a cell's mean, differences and products in double
+// carry that rounding to all its members; so the only rounding of the size of the
+// FP64 path's is the one of V' back to double.  (An exponent shared by the cells
+// of a sub-tile would cost a cell beside a faster one its low bits.)  A lone member
+// keeps its velocity, as v - u = 0 leaves it.  Streaming is the same fma.  With the
 // thermostat the energy about u and the scaling by xi stay in double.  What bounds
 // it now: at 64^3 cells (density 10) 101 M warp instructions, 39 % of the issue
 // slots, the FP64 pipe 46 % busy and 16 warps an SM (115 registers, 46 KB a block)
@@ -26,9 +29,9 @@
 // k_cells_warp_d's 760, so large boxes stay there.  On small boxes a tile's latency
 // is what counts, and 4 to 32 cells a warp spread them over the SMs (us a step):
 // 10^3 cells at density 5 34 -> 15, with the thermostat 57 -> 24; 16^3 at density 10
-// 51 -> 19; 24^3 52 -> 29; 50^3 142 -> 121.  A sub-tile
+// 51 -> 19; 24^3 52 -> 29; 50^3 142 -> 121.  A cell
 // with an overflowing row, a non-finite velocity or an exponent beyond +-900 takes
-// the same steps in double, one cell a lane.
+// the same steps in double.
 #include "dev_collide.cuh"
 #include "dev_rows.cuh"
 #include "dev_stream.cuh"
@@ -43,6 +46,7 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 constexpr int DB = 128;  // threads per block
 constexpr int DWARPS = DB / 32;
 constexpr int VBITS = 59;
+constexpr int LONE = 1 << 20, DOUBLE = LONE + 1;  // in place of a cell's exponent
 
 struct DBox {
   double dt, ca, sa, omc, m;
@@ -60,7 +64,8 @@ struct DBox {
 };
 
 // q: quarters of the staged records, (x, y), (z, v_x), (v_y, v_z), (tag, ..);
-// after the conversion v_* hold the integers V.  R: rotation matrix as signed
+// after the conversion v_* hold the integers V.  E: the cell's exponent, or LONE or
+// DOUBLE (its members' v_* stay doubles).  R: rotation matrix as signed
 // halves (hi, lo) of R 2^62, row by row; U: the cell's mean velocity as an integer;
 // u, xi: in double (thermostat and the double path).
 struct DWarp {
@@ -68,6 +73,7 @@ struct DWarp {
   int2 R[9][32];
   long long U[3][32];
   double u[3][32], xi[32];
+  int E[32];
   unsigned short map[SRDD_SLOTS];  // place in the row << 5 | cell
 };
 
@@ -235,71 +241,66 @@ __global__ void __launch_bounds__(DB, 4) k_srd_d(const BoxDev* __restrict__ boxe
 
       double* const vx = reinterpret_cast<double*>(&W.q[1][0]) + 1;  // member m: vx[2 m]
       double2* const vyz = reinterpret_cast<double2*>(&W.q[2][0]);
-      int E = 0;
-      bool plain = true;  // integers; else the whole sub-tile in double
       if (MODE != MODE_P) {
-        // ---- the sub-tile's exponent; velocities to integers in place ----
-        unsigned top = 0u;
-        for (int m = lane; m < cnt; m += 32) {
-          const double2 w = vyz[m];
-          top = max(top, max((unsigned)__double2hiint(vx[2 * m]) & 0x7FFFFFFFu,
-                             max((unsigned)__double2hiint(w.x) & 0x7FFFFFFFu,
-                                 (unsigned)__double2hiint(w.y) & 0x7FFFFFFFu)));
-        }
-        E = (int)(__reduce_max_sync(FULL, top) >> 20) - 1022;
-        plain = E > -900 && E < 900 && !__any_sync(FULL, mine && (int)n > K);
-        if (plain)
-          for (int m = lane; m < cnt; m += 32) {
-            const double2 w = vyz[m];
-            vx[2 * m] = __longlong_as_double(to_fixed(vx[2 * m], E));
-            vyz[m] = make_double2(__longlong_as_double(to_fixed(w.x, E)),
-                                  __longlong_as_double(to_fixed(w.y, E)));
-          }
-        __syncwarp();
-
-        // ---- sums: 2^plog lanes add up a cell; the first of them goes on ----
+        // 2^plog lanes add up a cell; the first of them goes on
         const int cc = a + (lane >> plog), part_ = lane & ((1 << plog) - 1);
         const int src = cc < b ? cc : a;
         const int nC = __shfl_sync(FULL, (int)n, src), s0C = __shfl_sync(FULL, s0, src);
         const int nrowC = cc < b ? min(nC, K) : 0;
         const double ehatC = THERMO ? __shfl_sync(FULL, ehat, src) : 0.0;
+        // ---- the cell's exponent ----
+        unsigned top = 0u;
+        for (int k = part_; k < nrowC; k += 1 << plog) {
+          const double2 w = vyz[s0C + k];
+          top = max(top, max((unsigned)__double2hiint(vx[2 * (s0C + k)]) & 0x7FFFFFFFu,
+                             max((unsigned)__double2hiint(w.x) & 0x7FFFFFFFu,
+                                 (unsigned)__double2hiint(w.y) & 0x7FFFFFFFu)));
+        }
+        for (int d = 1; d < (1 << plog); d <<= 1) top = max(top, __shfl_xor_sync(FULL, top, d));
+        int E = (int)(top >> 20) - 1022;
+        if (nC < 2 && E < 1025) E = LONE;  // (1025: not finite)
+        else if (E <= -900 || E >= 900 || nC > K) E = DOUBLE;
+        const bool plain = nrowC > 0 && E < LONE, dbl = nrowC > 0 && E == DOUBLE;
+
+        // ---- velocities to integers in place, and their sums ----
         double u[3] = {0.0, 0.0, 0.0}, Ek = 0.0;
-        if (plain) {
-          unsigned long long lo[3] = {0ull, 0ull, 0ull};
-          long long hi[3] = {0ll, 0ll, 0ll};
+        unsigned long long lo[3] = {0ull, 0ull, 0ull};
+        long long hi[3] = {0ll, 0ll, 0ll};
+        if (plain)
           for (int k = part_; k < nrowC; k += 1 << plog) {
             const double2 w = vyz[s0C + k];
-            const long long V[3] = {__double_as_longlong(vx[2 * (s0C + k)]),
-                                    __double_as_longlong(w.x), __double_as_longlong(w.y)};
+            const long long V[3] = {to_fixed(vx[2 * (s0C + k)], E), to_fixed(w.x, E),
+                                    to_fixed(w.y, E)};
+            vx[2 * (s0C + k)] = __longlong_as_double(V[0]);
+            vyz[s0C + k] = make_double2(__longlong_as_double(V[1]), __longlong_as_double(V[2]));
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
               lo[q] += (unsigned)V[q];
               hi[q] += (int)(V[q] >> 32);
             }
           }
-          for (int d = 1; d < (1 << plog); d <<= 1) {
+        for (int d = 1; d < (1 << plog); d <<= 1) {
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-              lo[q] += __shfl_xor_sync(FULL, lo[q], d);
-              hi[q] += __shfl_xor_sync(FULL, hi[q], d);
-            }
+          for (int q = 0; q < 3; ++q) {
+            lo[q] += __shfl_xor_sync(FULL, lo[q], d);
+            hi[q] += __shfl_xor_sync(FULL, hi[q], d);
           }
-          if (nrowC > 0) {
-            // u = Sum V / n: the sum (below 2^67) rounded once to double; every
-            // lane of the cell forms it
-            const double iM = 1.0 / ll2d_exact((long long)nC);
+        }
+        if (plain) {
+          // u = Sum V / n: the sum (below 2^67) rounded once to double; every
+          // lane of the cell forms it
+          const double iM = 1.0 / ll2d_exact((long long)nC);
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-              const __int128 T = ((__int128)hi[q] << 32) + (__int128)lo[q];
-              const double D = u128_to_double((unsigned __int128)(T < 0 ? -T : T));
-              const double uf = (T < 0 ? -D : D) * iM;  // in units of 2^(E - VBITS)
-              const long long U = truncate(uf);
-              u[q] = from_fixed(U, E);
-              if (part_ == 0) W.U[q][cc] = U;
-              if (THERMO) lo[q] = (unsigned long long)U;
-            }
+          for (int q = 0; q < 3; ++q) {
+            const __int128 T = ((__int128)hi[q] << 32) + (__int128)lo[q];
+            const double D = u128_to_double((unsigned __int128)(T < 0 ? -T : T));
+            const double uf = (T < 0 ? -D : D) * iM;  // in units of 2^(E - VBITS)
+            const long long U = truncate(uf);
+            if (THERMO) u[q] = from_fixed(U, E);
+            if (part_ == 0) W.U[q][cc] = U;
+            if (THERMO) lo[q] = (unsigned long long)U;
           }
-          if (THERMO) {  // energy about u, from the exact differences
+          if (THERMO)  // energy about u, from the exact differences
             for (int k = part_; k < nrowC; k += 1 << plog) {
               const double2 w = vyz[s0C + k];
               const long long V[3] = {__double_as_longlong(vx[2 * (s0C + k)]),
@@ -310,29 +311,31 @@ __global__ void __launch_bounds__(DB, 4) k_srd_d(const BoxDev* __restrict__ boxe
                 Ek = fma(d, d, Ek);
               }
             }
-          }
-        } else {
+        }
+        if (__any_sync(FULL, dbl)) {  // cells in double
           auto each = [&](auto&& f) {
+            if (!dbl) return;
             for (int k = part_; k < nrowC; k += 1 << plog) f(vx[2 * (s0C + k)], vyz[s0C + k]);
-            if (part_ == 0 && cc < b && nC > K)
+            if (part_ == 0 && nC > K)
               for_overflow(c0 + cc, [&](const RecD* p) {
                 double w[3];
                 load_v(p, w);
                 f(w[0], make_double2(w[1], w[2]));
               });
           };
+          double su[3] = {0.0, 0.0, 0.0};
           each([&](double x, double2 y) {
-            u[0] += x;
-            u[1] += y.x;
-            u[2] += y.y;
+            su[0] += x;
+            su[1] += y.x;
+            su[2] += y.y;
           });
           for (int d = 1; d < (1 << plog); d <<= 1)
 #pragma unroll
-            for (int q = 0; q < 3; ++q) u[q] += __shfl_xor_sync(FULL, u[q], d);
-          if (nC > 0) {
+            for (int q = 0; q < 3; ++q) su[q] += __shfl_xor_sync(FULL, su[q], d);
+          if (dbl) {
             const double iM = 1.0 / ll2d_exact((long long)nC);
 #pragma unroll
-            for (int q = 0; q < 3; ++q) u[q] = u[q] * iM;
+            for (int q = 0; q < 3; ++q) u[q] = su[q] * iM;
           }
           if (THERMO)
             each([&](double x, double2 y) {
@@ -349,10 +352,13 @@ __global__ void __launch_bounds__(DB, 4) k_srd_d(const BoxDev* __restrict__ boxe
             else atomicOr(err, ERR_GAMMA_CAP);
           }
         }
-        if (cc < b && part_ == 0 && (THERMO || !plain)) {
+        if (cc < b && part_ == 0) {
+          W.E[cc] = E;
+          if (THERMO || dbl) {
 #pragma unroll
-          for (int q = 0; q < 3; ++q) W.u[q][cc] = u[q];
-          W.xi[cc] = xi;
+            for (int q = 0; q < 3; ++q) W.u[q][cc] = u[q];
+            W.xi[cc] = xi;
+          }
         }
         __syncwarp();
       }
@@ -425,7 +431,8 @@ __global__ void __launch_bounds__(DB, 4) k_srd_d(const BoxDev* __restrict__ boxe
           w[2] = yz.y;
           tag = __float_as_uint(W.q[3][m].x);
           if (MODE != MODE_P) {
-            if (plain) {
+            const int E = W.E[o];
+            if (E < LONE) {
               // V' = U + R (V - U): |V - U| < 2^60, |R 2^62| <= 2^62, so the three
               // high products stay below 2^60 and the six mixed ones below 2^63
               int2 d[3];
@@ -446,7 +453,7 @@ __global__ void __launch_bounds__(DB, 4) k_srd_d(const BoxDev* __restrict__ boxe
                 w[i] = THERMO ? fma(W.xi[o], from_fixed(D, E), W.u[i][o])
                               : from_fixed(W.U[i][o] + D, E);
               }
-            } else {
+            } else if (E == DOUBLE) {
               collide_double(w, o);
             }
           }

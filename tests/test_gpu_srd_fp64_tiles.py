@@ -79,3 +79,36 @@ def test_exponents_beyond_the_integers_and_overflowing_rows():
     pos = s.pos.copy()
     pos[:200] = 1.3 + 0.4 * np.random.default_rng(2).random((200, 3))  # one cell, a full row and more
     compare(n, pos, s.vel, 1, seed=9, thermostat=True)
+
+
+@pytest.mark.parametrize("thermostat", [False, True])
+@pytest.mark.parametrize("n,rho", [((8, 6, 5), 6), ((23, 17, 9), 2), ((4, 3, 3), 58)])
+@pytest.mark.parametrize("fast", [1e6, 1e9, 1e12, 1e18])
+def test_a_fast_particle_costs_no_other_cell_precision(fast, n, rho, thermostat):
+    """One particle `fast` times faster than the rest, in one cell: every particle within the
+    parity bound of its own cell, 1e-12 of the largest speed that the cell's members had or got
+    (a collision rounds a handful of times at 2^-53 of that), and a particle alone in its
+    cell keeps its velocity to the bit, small components beside large ones included."""
+    s = inputs.solvent(n, rho, seed=21)
+    vel = s.vel.copy()
+    vel[::5, 1] *= 1e-14
+    vel[0] *= fast / np.linalg.norm(vel[0])
+    box = pkg.Box(n=n, seed=21, precision="fp64", thermostat=thermostat)
+    box.set_state(s.pos, vel, step=5)
+    box.step(1)
+    p, v, _, _, _ = box.get_state()
+    cells, counts = box.last_cells()
+    box.close()
+    ref = oracle.State(s.pos.copy(), vel.copy(), step=5)
+    rc, rk = oracle.step(oracle.Params(n=n, seed=21, precision=oracle.FP64, thermostat=thermostat), ref, 1,
+                         want_cells=True)
+    np.testing.assert_array_equal(cells, rc)
+    np.testing.assert_array_equal(counts, rk)
+    np.testing.assert_array_equal(p, ref.pos)
+    speed = np.maximum(np.linalg.norm(vel, axis=1), np.linalg.norm(ref.vel, axis=1))
+    largest = np.zeros(len(rk))
+    np.maximum.at(largest, rc, speed)
+    assert (np.linalg.norm(v - ref.vel, axis=1) / largest[rc]).max() <= 1e-12
+    lone = rk[rc] == 1
+    assert lone.any() or rho > 10
+    np.testing.assert_array_equal(v[lone], vel[lone])
