@@ -364,7 +364,10 @@ __global__ void __launch_bounds__(WT, 4) k_wca_md(const BoxDev* __restrict__ box
   };
 
   for_beads([&](const BoxDev& B, int b) {
-    const double r[3] = {B.spos[3 * (size_t)b], B.spos[3 * (size_t)b + 1], B.spos[3 * (size_t)b + 2]};
+    // a given state may lie outside the box; cells, fractions and min_image take it inside
+    double r[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) r[k] = wrap_bits(B.spos[3 * (size_t)b + k], B.L[k]);
     put(B, 0, b, r);
   });
   rebuild(0, 0);

@@ -116,3 +116,28 @@ def test_wca_invalid_parameters():
         pkg.Box(n=(8, 8, 8), **dict(KW, chain_len=5, lj_sigma=0.6))  # cutoff + buffer > 1
     with pytest.raises(pkg.MpcdError):
         pkg.Box(n=(2, 8, 8), **dict(KW, chain_len=5))  # fewer than 3 cells on an axis
+
+
+def bead_error(n, s, sp, sv, steps, **kw):
+    """Largest distance of bead positions and velocities (relative to max(|v|, thermal)) from the oracle."""
+    box = pkg.Box(n=n, seed=17, precision="fp64", **kw)
+    box.set_state(s.pos, s.vel, sp, sv)
+    box.step(steps)
+    _, _, spos, svel, _ = box.get_state()
+    box.close()
+    ref = oracle.State(s.pos.copy(), s.vel.copy(), sp.copy(), sv.copy())
+    oracle.step(oracle.Params(n=n, seed=17, precision=oracle.FP64, **kw), ref, steps)
+    d = np.abs(spos - ref.spos)
+    return np.minimum(d, np.array(n, dtype=float) - d).max(), rel_err(svel, ref.svel, m=5.0)
+
+
+@pytest.mark.parametrize("far", [1, 3])
+def test_wca_beads_given_outside_the_box(far):
+    """Each bead of the chains moved by up to `far` box lengths along every axis: the images that
+    the first forces see are those of the beads inside."""
+    n = (6, 7, 8)
+    s = inputs.solvent(n, 4, seed=17)
+    sp, sv = inputs.avoiding_chains(n, 20, 10, 0.5, 0.45, bead_mass=5.0, seed=18)
+    sp = sp + np.random.default_rng(5).integers(-far, far + 1, sp.shape) * np.array(n, dtype=float)
+    dr, dv = bead_error(n, s, sp, sv, 1, **dict(KW, chain_len=10, bond_k=30.0))
+    assert dr <= 1e-10 and dv <= 1e-10
