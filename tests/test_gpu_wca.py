@@ -141,3 +141,14 @@ def test_wca_beads_given_outside_the_box(far):
     sp = sp + np.random.default_rng(5).integers(-far, far + 1, sp.shape) * np.array(n, dtype=float)
     dr, dv = bead_error(n, s, sp, sv, 1, **dict(KW, chain_len=10, bond_k=30.0))
     assert dr <= 1e-10 and dv <= 1e-10
+
+
+def test_wca_bonds_of_half_the_box():
+    """Bonds of exactly half an edge point along the given difference, as d - L rint(d / L) has it,
+    and not across the boundary."""
+    n = (4, 6, 8)
+    s = inputs.solvent(n, 4, seed=17)
+    sp = np.array([[0.5, 1.0, 1.0], [2.5, 1.0, 1.0], [1.25, 4.5, 3.0], [1.25, 1.5, 3.0],
+                   [3.0, 2.0, 6.5], [3.0, 2.0, 2.5], [0.75, 5.25, 0.25], [2.75, 2.25, 4.25]])
+    dr, dv = bead_error(n, s, sp, np.zeros_like(sp), 1, **dict(KW, chain_len=2, bond_k=30.0))
+    assert dr <= 1e-10 and dv <= 1e-10
