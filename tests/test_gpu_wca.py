@@ -152,3 +152,23 @@ def test_wca_bonds_of_half_the_box():
                    [3.0, 2.0, 6.5], [3.0, 2.0, 2.5], [0.75, 5.25, 0.25], [2.75, 2.25, 4.25]])
     dr, dv = bead_error(n, s, sp, np.zeros_like(sp), 1, **dict(KW, chain_len=2, bond_k=30.0))
     assert dr <= 1e-10 and dv <= 1e-10
+
+
+def test_wca_bonds_and_kicks_take_the_oracle_s_operations():
+    """Beads further apart than the cutoff all along: a step's MD is bonds and kicks alone, and the
+    positions it leaves are the oracle's to the bit."""
+    n = (9, 8, 7)
+    kw = dict(KW, chain_len=8, bond_r0=0.9)
+    s = inputs.solvent(n, 4, seed=17)
+    sp, sv = inputs.avoiding_chains(n, 6, 8, 0.9, 0.8, bead_mass=5.0, seed=19)
+    box = pkg.Box(n=n, seed=17, precision="fp64", **kw)
+    box.set_state(s.pos, s.vel, sp, sv)
+    box.step(1)
+    spos = box.get_state()[2]
+    box.close()
+    ref = oracle.State(s.pos.copy(), s.vel.copy(), sp.copy(), sv.copy())
+    oracle.step(oracle.Params(n=n, seed=17, precision=oracle.FP64, **kw), ref, 1)
+    d = ref.spos[:, None, :] - ref.spos[None, :, :]
+    d -= np.array(n) * np.round(d / np.array(n))
+    assert np.sqrt((d * d).sum(-1) + 9.0 * np.eye(len(d))).min() > 0.6
+    np.testing.assert_array_equal(spos, ref.spos)
