@@ -16,6 +16,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -128,6 +129,35 @@ int validate(const mpcd_params* p, int precision_expected) {
   const int64_t C = cells_of(*p);
   if (C > 2000000000LL) return fail(MPCD_EINVAL, "too many cells (max 2e9)");
   return MPCD_OK;
+}
+
+// Whether a kernel of this device may store `bytes` bytes of elements of size `es`
+// at p: aligned device memory of its own, all of them within one allocation.  A copy
+// is checked by the driver, and reaches other devices' memory; a kernel's store is not.
+bool own_device_memory(const void* p, size_t bytes, size_t es, int device) {
+  using Range = int (*)(unsigned long long*, size_t*, unsigned long long);  // cuMemGetAddressRange
+  static const Range range = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) !=
+            cudaSuccess || q != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return (Range)f;
+  }();
+  if (!range || (uintptr_t)p % es != 0) return false;
+  cudaPointerAttributes at{};
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();  // not this call's failure: the copy will say
+    return false;
+  }
+  if (at.type != cudaMemoryTypeDevice || at.device != device) return false;
+  unsigned long long base = 0;
+  size_t size = 0;
+  if (range(&base, &size, (unsigned long long)(uintptr_t)p) != 0) return false;
+  const unsigned long long off = (unsigned long long)(uintptr_t)p - base;
+  return off <= size && bytes <= size - off;
 }
 
 // ---------------------------------------------------------------------------
@@ -1297,7 +1327,22 @@ int mpcd_get_state_device(mpcd_ctx* ctx, void* pos, void* vel) {
   if (!ctx->box->has_state) return fail(MPCD_ESTATE, "no state set");
   Engine& E = ctx->eng;
   Box* b = ctx->box;
-  return E.extract(b, nullptr, pos, vel);  // straight into the caller's arrays
+  // straight into the caller's arrays where a kernel may store there, else (another
+  // device's memory, a pointer that the driver has to judge, arrays that overlap)
+  // through the staging arrays and a copy
+  const size_t es = elem_size(E.mixed), bytes = (size_t)b->nsol * 3 * es;
+  const bool apart = !pos || !vel || (const char*)pos + bytes <= (const char*)vel ||
+                     (const char*)vel + bytes <= (const char*)pos;
+  void* dp = pos && apart && own_device_memory(pos, bytes, es, E.device) ? pos : nullptr;
+  void* dv = vel && apart && own_device_memory(vel, bytes, es, E.device) ? vel : nullptr;
+  int rc = E.extract(b, nullptr, dp, dv);
+  if (rc) return rc;
+  if (bytes == 0 || (dp == pos && dv == vel)) return MPCD_OK;
+  if (dp != pos) CUDA_TRY(cudaMemcpyAsync(pos, b->stage_r, bytes, cudaMemcpyDeviceToDevice, E.stream));
+  if (dv != vel) CUDA_TRY(cudaMemcpyAsync(vel, b->stage_v, bytes, cudaMemcpyDeviceToDevice, E.stream));
+  CUDA_TRY(cudaStreamSynchronize(E.stream));
+  CUDA_TRY(cudaGetLastError());
+  return MPCD_OK;
 }
 
 int mpcd_observables(mpcd_ctx* ctx, mpcd_obs* out) {

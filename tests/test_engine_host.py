@@ -1,0 +1,114 @@
+"""The host engine (capi.cu) on a CPU: its launch rules and what it does with the errors that
+a CUDA call returns, on a stand-in for the CUDA runtime and the kernels' launchers
+(tests/host_engine).  Nothing is computed: a launch is a line of a log."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+import paper_1801_10187_gb300 as pkg
+from paper_1801_10187_gb300 import _build
+
+HERE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "host_engine")
+DEVICE, HOST = 2, 1  # cudaMemoryType
+P, I64, I32, U64 = ctypes.c_void_p, ctypes.c_int64, ctypes.c_int32, ctypes.c_uint64
+
+
+@pytest.fixture(scope="module")
+def engine(tmp_path_factory):
+    if not (shutil.which("nvcc") or os.path.exists("/usr/local/cuda/bin/nvcc")):
+        pytest.skip("nvcc is needed to compile the engine's host code")
+    _build.build()
+    out = tmp_path_factory.mktemp("engine")
+    nvcc = _build._nvcc()
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(nvcc)))
+
+    def run(*cmd):
+        r = subprocess.run(cmd, capture_output=True, text=True)
+        assert r.returncode == 0, r.stdout + r.stderr
+
+    run("g++", "-O1", "-std=c++17", "-fPIC", "-I", os.path.join(cuda, "include"), "-c",
+        os.path.join(HERE, "fake_runtime.cpp"), "-o", str(out / "runtime.o"))
+    run(nvcc, *_build.ARCH, "-O1", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC", "-c",
+        os.path.join(HERE, "fake_launchers.cu"), "-o", str(out / "launchers.o"))
+    run("g++", "-shared", "-Wl,-Bsymbolic", os.path.join(_build.BUILD, "capi.o"), str(out / "runtime.o"),
+        str(out / "launchers.o"), "-o", str(out / "engine.so"), "-lpthread")
+    L = ctypes.CDLL(str(out / "engine.so"))
+    L.fake_log.restype = ctypes.c_char_p
+    L.mpcd_last_error.restype = ctypes.c_char_p
+    L.fake_alloc.restype = P
+    L.fake_alloc.argtypes = [ctypes.c_size_t, ctypes.c_int, ctypes.c_int]
+    L.fake_cost.argtypes = [ctypes.c_int, ctypes.c_double]
+    L.mpcd_get_state_device.argtypes = [P, P, P]
+    L.mpcd_set_state_thermal.argtypes = [P, I64, U64, U64]
+    L.mpcd_step.argtypes = [P, I64]
+    L.mpcd_destroy.argtypes = [P]
+    return L
+
+
+class Box:
+    """A box of the engine; solute: beads at random places in chains of kw's chain_len."""
+
+    def __init__(self, L, n_solvent, n_solute=0, **kw):
+        self.L, self.ctx, p = L, P(), pkg.make_params(**kw)
+        assert L.mpcd_create(ctypes.byref(p), None, ctypes.byref(self.ctx)) == 0
+        if n_solute:
+            x = [np.random.default_rng(1).random((m, 3)) for m in (n_solvent, n_solvent, n_solute, n_solute)]
+            a, b, c, d = (v.ctypes.data_as(P) for v in x)
+            assert L.mpcd_set_state(self.ctx, I64(n_solvent), a, b, I64(n_solute), c, d, U64(0)) == 0
+        else:
+            assert L.mpcd_set_state_thermal(self.ctx, n_solvent, 1, 0) == 0
+        self.log()
+
+    def step(self, n=1):
+        return self.L.mpcd_step(self.ctx, n)
+
+    def log(self):
+        return self.L.fake_log().decode().split("\n")[:-1]
+
+    def close(self):
+        self.L.mpcd_destroy(self.ctx)
+
+
+@pytest.mark.parametrize("precision", ["mixed", "fp64"])
+def test_the_state_is_stored_by_a_kernel_only_into_memory_it_may_write(engine, precision):
+    """mpcd_get_state_device: into this device's own memory directly; into another device's, or where
+    two arrays overlap or are not aligned, through a copy; what the driver refuses, and an
+    array that is too small, comes back as an error."""
+    n, es = 1000, 4 if precision == "mixed" else 8
+    real, bytes_ = np.float32 if es == 4 else np.float64, 3 * 1000 * es
+    box = Box(engine, n, n=(5, 5, 5), precision=precision)
+    box.step(1)
+
+    def read(pos, vel):
+        box.log()
+        rc = engine.mpcd_get_state_device(box.ctx, pos, vel)
+        return rc, [x for x in box.log() if x.startswith("copy")]
+
+    def values(p):
+        return np.frombuffer(ctypes.string_at(p, bytes_), dtype=real)
+
+    own = [engine.fake_alloc(bytes_, DEVICE, 0) for _ in range(2)]
+    other = [engine.fake_alloc(bytes_, DEVICE, 1) for _ in range(2)]
+    assert read(*own) == (0, [])
+    assert read(own[0], None) == (0, []) and read(None, own[1]) == (0, [])
+    rc, copies = read(*other)
+    assert rc == 0 and len(copies) == 2
+    rc, copies = read(own[0], other[1])
+    assert rc == 0 and len(copies) == 1
+    for pos, vel in (own, other):
+        assert np.all(values(pos) == 1) and np.all(values(vel) == 2)
+    both = engine.fake_alloc(2 * bytes_, DEVICE, 0)
+    assert read(both, both + bytes_) == (0, [])
+    rc, copies = read(both, both + es)  # overlapping: the velocities are written last
+    assert rc == 0 and len(copies) == 2 and np.all(values(both)[1:] == 2) and values(both)[0] == 1
+    rc, copies = read(both + es // 2, None)  # not aligned
+    assert rc == 0 and len(copies) == 1
+    small = engine.fake_alloc(bytes_ - 1, DEVICE, 0)
+    for bad in (small, own[0] + es, 1 << 40, engine.fake_alloc(bytes_ // 2, HOST, 0)):
+        assert read(bad, own[1])[0] == pkg.MPCD_ECUDA
+    assert read(*own) == (0, [])
+    box.close()
