@@ -684,20 +684,24 @@ struct Engine {
       launch_after_pass(d_boxes, (int)live.size(), mode != MODE_C, mode != MODE_P, stream);
   }
 
-  // Solute: MD substeps and bead grouping for the step in the records.
-  void launch_beads() {
-    if (!any_beads) return;
+  // Solute: MD substeps and bead grouping for the step in the records.  Returns the
+  // error of the cooperative launch, which a device may refuse where it takes others.
+  cudaError_t launch_beads() {
+    if (!any_beads) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
     if (wca_substeps > 0)
-      launch_wca_md(d_boxes, d_wtiles, n_wtiles, wca_substeps, wca_bps * nsm, d_wsync, d_err, stream);
+      e = (cudaError_t)launch_wca_md(d_boxes, d_wtiles, n_wtiles, wca_substeps, wca_bps * nsm, d_wsync,
+                                     d_err, stream);
     launch_md_bin(d_boxes, d_mdtiles, n_mdtiles, md_chains_per_block, md_threads, d_err, stream);
     launch_scan(d_bsegs, d_bstiles, n_bstiles, d_tsum, d_gscan, d_toff, grid_for(n_bstiles, 8),
                 stream);
     launch_bead_scatter(d_boxes, d_btiles, n_btiles, stream);
+    return e;
   }
 
   // One pass over every live box (plain launches; captured into the graphs).
-  void enqueue_pass(int mode) {
-    if (live.empty()) return;
+  cudaError_t enqueue_pass(int mode) {
+    if (live.empty()) return cudaSuccess;
     // Virtual wall particles: the first pass needs them before its collision can
     // follow; a fused pass draws those of the next step beside itself.
     if (n_vtiles > 0 && mode == MODE_F) {
@@ -710,7 +714,7 @@ struct Engine {
     if (n_vtiles > 0 && mode == MODE_F) cudaStreamWaitEvent(stream, ev_join, 0);
     if (n_vtiles > 0 && mode == MODE_P)
       launch_virtual(d_boxes, (int)live.size(), d_vtiles, n_vtiles, 1, d_done + 1, stream);
-    if (mode != MODE_C) launch_beads();
+    return mode != MODE_C ? launch_beads() : cudaSuccess;
   }
 
   int ensure_tables() {
@@ -724,11 +728,15 @@ struct Engine {
     if (gexec[mode]) return MPCD_OK;
     cudaGraph_t g = nullptr;
     CUDA_TRY(cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal));
-    if (mode == GRAPH_MANY)
-      for (int i = 0; i < GRAPH_STEPS; ++i) enqueue_pass(MODE_F);
-    else
-      enqueue_pass(mode);
+    cudaError_t le = cudaSuccess;  // of a launch: the graph would lack it
+    for (int i = 0; i < (mode == GRAPH_MANY ? GRAPH_STEPS : 1) && le == cudaSuccess; ++i)
+      le = enqueue_pass(mode == GRAPH_MANY ? MODE_F : mode);
     cudaError_t e = cudaStreamEndCapture(stream, &g);
+    if (le != cudaSuccess) {
+      if (e == cudaSuccess) cudaGraphDestroy(g);
+      cudaGetLastError();
+      return fail(MPCD_ECUDA, std::string("launch: ") + cudaGetErrorString(le));
+    }
     if (e != cudaSuccess) return fail(MPCD_ECUDA, std::string("capture: ") + cudaGetErrorString(e));
     e = cudaGraphInstantiate(&gexec[mode], g, 0);
     cudaGraphDestroy(g);
@@ -810,7 +818,7 @@ struct Engine {
       for (int c : cand) {
         tuned_grid = c;
         CUDA_TRY(cudaEventRecord(e0, stream));
-        for (int64_t r = 0; r < reps; ++r) enqueue_pass(MODE_F);
+        for (int64_t r = 0; r < reps; ++r) CUDA_TRY(enqueue_pass(MODE_F));
         CUDA_TRY(cudaEventRecord(e1, stream));
         CUDA_TRY(cudaEventSynchronize(e1));
         float ms = 0.f;
@@ -855,7 +863,7 @@ struct Engine {
     for (int i = 0; i < kPhases; ++i) ms[i] = 0.0;
     if (live.empty() || n <= 0) return kPhases;
     // the first pass streams and bins (it is not one of the timed steps)
-    enqueue_pass(MODE_P);
+    CUDA_TRY(enqueue_pass(MODE_P));
     pending = true;
     cudaEvent_t ev[kPhases + 1];
     for (auto& e : ev) CUDA_TRY(cudaEventCreate(&e));
@@ -866,7 +874,7 @@ struct Engine {
       launch_cells_all(MODE_F);
       CUDA_TRY(cudaEventRecord(ev[1], stream));
       CUDA_TRY(cudaEventRecord(ev[2], stream));  // (the record updates are part of the pass)
-      launch_beads();
+      CUDA_TRY(launch_beads());
       CUDA_TRY(cudaEventRecord(ev[3], stream));
       CUDA_TRY(cudaEventSynchronize(ev[3]));
       for (int i = 0; i < kPhases; ++i) {
@@ -1688,7 +1696,7 @@ extern "C" int mpcd_profile_noalloc(mpcd_ctx* ctx, int32_t nbins, double* out) {
   // is written in input order into the box's existing staging arrays: no
   // allocation on either path.
   if (E.pending) {
-    E.enqueue_pass(MODE_C);
+    CUDA_TRY(E.enqueue_pass(MODE_C));
     E.pending = false;
   }
   const int n = (int)b->nsol;

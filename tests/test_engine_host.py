@@ -73,6 +73,23 @@ class Box:
         self.L.mpcd_destroy(self.ctx)
 
 
+def test_a_refused_launch_is_an_error_of_every_step(engine):
+    """The cooperative launch of the solute's MD fails during capture: no graph without it is kept,
+    so the next steps fail as well, and the first one after that takes it."""
+    box = Box(engine, 500, 40, n=(5, 5, 5), precision="fp64", chain_len=10, md_substeps=5, solute_mass=5.0,
+              bond_k=100.0, bond_r0=0.5, lj_epsilon=1.0, lj_sigma=0.5)
+    for passes in (1, 40):
+        engine.fake_fail(b"wca", 720)  # cudaErrorCooperativeLaunchTooLarge
+        for _ in range(2):
+            assert box.step(passes) == pkg.MPCD_ECUDA
+            assert "graph" not in box.log()
+        engine.fake_fail(b"wca", 0)
+        assert box.step(passes) == 0
+        log = box.log()
+        assert "wca" in log and "graph" in log
+    box.close()
+
+
 @pytest.mark.parametrize("precision", ["mixed", "fp64"])
 def test_the_state_is_stored_by_a_kernel_only_into_memory_it_may_write(engine, precision):
     """mpcd_get_state_device: into this device's own memory directly; into another device's, or where
