@@ -396,13 +396,14 @@ struct Engine {
       const bool at = (v & 16) != 0, ang = (v & 32) != 0;
       cells_bps[m][v] = 1;
       if (v & 64) {
-        if (!mixed && !(v & (4 | 8 | 16 | 32)))
+        if (!mixed) {
           cells_bps[m][v] = srdd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, m);
-        if (mixed && !(at && (v & (1 | 4 | 8 | 32))) && !(ang && (v & (4 | 8))) && !((v & 4) && (v & (2 | 8))))
-          if (v & 8)
-            srd_bead_bps[m][v & 7] = std::max(
-                1, srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, true, (v & 4) != 0, false, false, m));
+        } else {
           cells_bps[m][v] = srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, (v & 4) != 0, at, ang, m);
+          if (v & 8)
+            srd_bead_bps[m][v & 7] =
+                std::max(1, srd_blocks_per_sm((v & 1) != 0, (v & 2) != 0, true, false, false, false, m));
+        }
       } else if ((v & 4) && ang) {  // warp-spread angular correction: mixed SRD without beads
         if (mixed && !(v & (8 | 16)))
           cells_bps[m][v] = cells_warp_blocks_per_sm((v & 1) != 0, (v & 2) != 0, false, false, true, m);

@@ -23,13 +23,12 @@
 // of a sub-tile would cost a cell beside a faster one its low bits.)  A lone member
 // keeps its velocity, as v - u = 0 leaves it.  Streaming is the same fma.  With the
 // thermostat the energy about u and the scaling by xi stay in double.  What bounds
-// it now: at 64^3 cells (density 10) 101 M warp instructions, 39 % of the issue
-// slots, the FP64 pipe 46 % busy and 16 warps an SM (115 registers, 46 KB a block)
-// that wait on them in turn; at 10^7 particles that is 823 us against
-// k_cells_warp_d's 760, so large boxes stay there.  On small boxes a tile's latency
-// is what counts, and 4 to 32 cells a warp spread them over the SMs (us a step):
-// 10^3 cells at density 5 34 -> 15, with the thermostat 57 -> 24; 16^3 at density 10
-// 51 -> 19; 24^3 52 -> 29; 50^3 142 -> 121.  A cell
+// it now: 16 warps an SM (115 registers, 47 KB a block) that wait on the FP64 pipe
+// and the integer pipes in turn, neither of them half busy; the line beyond which
+// k_cells_warp_d is taken is at SRDD_MAX_CELLS (kernels.h).  On small boxes a tile's
+// latency is what counts, and 4 to 32 cells a warp spread them over the SMs (us a
+// step): 10^3 cells at density 5 35 -> 12, with the thermostat 57 -> 22; 16^3 at
+// density 10 51 -> 17; 24^3 52 -> 27; 50^3 143 -> 114.  A cell
 // with an overflowing row, a non-finite velocity or an exponent beyond +-900 takes
 // the same steps in double.
 #include "dev_collide.cuh"

@@ -55,8 +55,11 @@ void launch_srd(bool thermo, bool force, bool beads, bool walls, bool at, bool a
 // The FP64 model's counterpart of k_srd (k_srd_d.cu), for periodic SRD boxes
 // without solute and rows of at most SRDD_SLOTS records.
 // It pays where the latency of a tile counts and not the FP64 pipe's rate:
-// against k_cells_warp_d (us a step, density 10) 16^3 cells 19 to 51, 24^3 29 to
-// 52, 40^3 71 to 75, 50^3 121 to 142, 64^3 229 to 229, 100^3 823 to 760.
+// against k_cells_warp_d (us a step, density 10) 16^3 cells 17 to 51, 24^3 27 to
+// 52, 40^3 72 to 75, 50^3 114 to 143, 64^3 217 to 230, 100^3 743 to 757, 128^3
+// 1551 to 1495.  How full its sub-tiles are tells beyond the line: at 100^3 434 to
+// 489 at density 5, but 1045 to 872 at density 12.  The boxes of a batch are taken
+// each by itself (16 boxes of 50^3 in a launch: 1452 to 1516, 64 of 16^3 221 to 244).
 constexpr int SRDD_SLOTS = 112, SRDD_MAX_CELLS = 200000;
 int srdd_blocks_per_sm(bool thermo, bool force, int mode);
 void launch_srdd(bool thermo, bool force, int mode, const BoxDev* boxes, const int2* spans,

@@ -73,6 +73,27 @@ class Box:
         self.L.mpcd_destroy(self.ctx)
 
 
+def fused(log, mode=1):
+    """(launcher, spans, grid, cells per warp) of the fused launches of a mode (1: stream after collide)."""
+    out = []
+    for line in log:
+        name, *kv = line.split()
+        kv = {k: int(v) for k, _, v in (x.partition("=") for x in kv)}
+        if kv.get("mode") == mode:
+            out.append((name, kv["spans"], kv["grid"], kv["cpw"]))
+    return out
+
+
+@pytest.mark.parametrize("precision,kernel,per_sm", [("fp64", "srdd", 4), ("mixed", "srd", 7)])
+def test_a_large_launch_is_as_many_blocks_as_fit(engine, precision, kernel, per_sm):
+    """Blocks per SM are those of the kernel that is launched (in the stand-in 4 and 7)."""
+    box = Box(engine, 1000, n=(57, 57, 57), precision=precision)
+    assert box.step(2) == 0
+    (name, spans, grid, cpw), = fused(box.log())
+    assert (name, spans, cpw) == (kernel, 724, 32) and grid == per_sm * 152
+    box.close()
+
+
 def test_a_refused_launch_is_an_error_of_every_step(engine):
     """The cooperative launch of the solute's MD fails during capture: no graph without it is kept,
     so the next steps fail as well, and the first one after that takes it."""
