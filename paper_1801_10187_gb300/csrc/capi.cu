@@ -635,12 +635,18 @@ struct Engine {
     return cpw;
   }
 
+  // Mixed SRD variants of k_cells_warp, whose mode F takes the tuner's cells per warp.
+  bool narrows(int v) const { return mixed && (v & 4) && !(v & (16 | 32 | 64)); }
+  int warp_cpw(int v, int mode) const {
+    return narrows(v) && mode == MODE_F && tuned_cpw ? std::max(tuned_cpw, 8) : 32;
+  }
+
   // Grid of the fused pass: tuned_grid 0 = the occupancy limit (blocks per
   // SM that fit), k > 0 = at most k blocks per SM, -1 = one block per span
-  // part (the k_srd takes a 256-cell span in parts).
+  // part (a 256-cell span is taken in parts where a warp has fewer than 32 cells).
   int tuned_grid = 0;
   int grid_of(int v, int mode) const {
-    const int items = n_spans[v] * ((v & 64) ? srd_parts(srd_cpw()) : 1);
+    const int items = n_spans[v] * ((v & 64) ? srd_parts(srd_cpw()) : 32 / warp_cpw(v, mode));
     if (mode == MODE_F && tuned_grid == -1) return std::max(items, 1);
     const int limit = cells_bps[mode][v];
     return grid_for(items, (mode == MODE_F && tuned_grid > 0) ? std::min(tuned_grid, limit) : limit);
@@ -673,7 +679,7 @@ struct Engine {
                      after, d_err, stream);
       } else if ((v & 4) && mixed) {
         launch_cells_warp((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, (v & 32) != 0, mode,
-                          d_boxes, d_spans[v], n_spans[v], grid, d_err, stream);
+                          d_boxes, d_spans[v], n_spans[v], grid, warp_cpw(v, mode), d_err, stream);
       } else if (v & 4) {
         launch_cells_warpd((v & 1) != 0, (v & 2) != 0, (v & 8) != 0, at, mode, d_boxes,
                            d_spans[v], n_spans[v], grid, d_err, stream);
@@ -778,7 +784,8 @@ struct Engine {
   // Launch tuner.  The paper tunes its kernels' launch parameters at run time
   // on real steps (Sec. 3.5, Sec. 4).  Here each candidate of the fused pass
   // -- grid (1 .. occupancy-limit blocks per SM, and one block per span part)
-  // times, for k_srd and k_srd_d, the cells per warp (32, 16 or 8)
+  // times, for k_srd, k_srd_d and the SRD variants of k_cells_warp, the cells per
+  // warp (32, 16 or 8)
   // -- runs `reps` real steps, timed with CUDA events on the
   // stream; the fastest is kept and the step graph re-captured.  Results do
   // not depend on the candidate: the mixed model's cell sums are exact, the
@@ -798,11 +805,11 @@ struct Engine {
       pending = true;
       taken += 1;
     }
-    bool any_reg = false;
-    for (int v = 64; v < NVAR; ++v)
-      if (n_spans[v] > 0) any_reg = true;
+    bool any_width = false;
+    for (int v = 0; v < NVAR; ++v)
+      if (n_spans[v] > 0 && ((v & 64) || narrows(v))) any_width = true;
     std::vector<int> widths = {32};  // cells per warp
-    if (any_reg) widths = {32, 16, 8};
+    if (any_width) widths = {32, 16, 8};
     cudaEvent_t e0, e1;
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));

@@ -43,10 +43,10 @@ int cells_warp_blocks_per_sm(bool thermo, bool force, bool beads, bool at, bool 
 }
 
 void launch_cells_warp(bool thermo, bool force, bool beads, bool at, bool ang, int mode,
-                       const BoxDev* boxes, const int2* spans, int nspans, int grid, int* err,
+                       const BoxDev* boxes, const int2* spans, int nspans, int grid, int cpw, int* err,
                        cudaStream_t s) {
   if (nspans <= 0) return;
-  void* args[] = {(void*)&boxes, (void*)&spans, (void*)&nspans, (void*)&err};
+  void* args[] = {(void*)&boxes, (void*)&spans, (void*)&nspans, (void*)&cpw, (void*)&err};
   cudaLaunchKernel(warp_variant(thermo, force, beads, at, ang, mode), dim3(grid), dim3(BLOCK), args,
                    block_smem(beads, at, ang, thermo), s);
 }

@@ -6,8 +6,11 @@
 // Same modes, records and results as k_cells (one thread per cell), for boxes
 // without walls (solute beads allowed): the Andersen rule, the angular
 // correction, and SRD with rows beyond the SRD_SLOTS records that k_srd, the
-// faster kernel for plain SRD, takes.  A warp owns 32 consecutive cells.  Their
-// row members are numbered 0 .. N-1 in cell order (a warp prefix sum of the row
+// faster kernel for plain SRD, takes.  A warp owns cpw consecutive cells: 32, or
+// for SRD in mode F 16 or 8 where the launch tuner finds that faster (a 256-cell
+// span is then taken in 32 / cpw parts, one block each; results do not depend on
+// it).  With rows this long a warp's cells take it long, so narrow warps pay: 32^3
+// cells at density 150 292 -> 137 us a step, 96^3 2942 -> 2743.  Their row members are numbered 0 .. N-1 in cell order (a warp prefix sum of the row
 // counts); a byte map gives each member's cell.
 //   pass 1   the (v, tag) words of up to 192 members are copied into shared
 //            memory asynchronously in member order (neighbouring lanes,
@@ -203,8 +206,9 @@ __host__ __device__ constexpr size_t block_smem(bool beads, bool at, bool ang = 
 template <bool THERMO, int MODE, bool FORCE, bool BEADS, bool AT, bool ANG>
 __global__ void __launch_bounds__(BLOCK, (AT || ANG) ? 2 : 4) k_cells_warp(const BoxDev* __restrict__ boxes,
                                                          const int2* __restrict__ spans,
-                                                         int nspans, int* err) {
+                                                         int nspans, int width, int* err) {
   using R = RecF;
+  const int cpw = MODE == MODE_F && !AT && !ANG ? width : 32;  // cells per warp
   extern __shared__ __align__(16) unsigned char smem_[];
   SpanParams& sp_ = *reinterpret_cast<SpanParams*>(smem_);
   const int lane = threadIdx.x & 31;
@@ -222,7 +226,9 @@ __global__ void __launch_bounds__(BLOCK, (AT || ANG) ? 2 : 4) k_cells_warp(const
   constexpr bool EARLY = !AT && !ANG;
   constexpr int SB = EARLY ? STAGE4 : STAGE;
   int box_of_params = -1;  // the span parameters depend on the box only
-  for (int sp = blockIdx.x; sp < nspans; sp += gridDim.x) {
+  const int parts = 32 / cpw;  // of a 256-cell span
+  for (int it = blockIdx.x; it < nspans * parts; it += gridDim.x) {
+    const int sp = it / parts, part = it - sp * parts;
     const int2 tt = spans[sp];
     const BoxDev& B = boxes[tt.x];
     const unsigned long long t = B.step;
@@ -257,10 +263,10 @@ __global__ void __launch_bounds__(BLOCK, (AT || ANG) ? 2 : 4) k_cells_warp(const
       __syncthreads();
       box_of_params = tt.x;
     }
-    const int c0 = tt.y + (int)(threadIdx.x & ~31u);
+    const int c0 = tt.y + (part * WARPS + (int)(threadIdx.x >> 5)) * cpw;
     if (c0 >= B.ncells) continue;  // warp-uniform
     const int cell = c0 + lane;
-    const bool valid = cell < B.ncells;
+    const bool valid = lane < cpw && cell < B.ncells;
     const int cur = B.cur;
     const int K = H.K;
     const uint32_t n = valid ? B.cnt[cur][cell] : 0u;
@@ -394,15 +400,18 @@ __global__ void __launch_bounds__(BLOCK, (AT || ANG) ? 2 : 4) k_cells_warp(const
     if (EARLY && MODE != MODE_P) stage_async(0, min(STAGE4, N));
 
     // Solute beads join their cell's collision with mass M (Sec. 3.6).  The
-    // warp's cells are one bead group of 32 cells; the group's beads are
-    // handled one per lane (grouped copies of cell and velocity): first their
-    // count per cell.
+    // warp's cells lie in one bead group of 32 cells; the group's beads are
+    // handled one per lane (grouped copies of cell and velocity), those of this
+    // warp's cells only: first their count per cell.
     const int gnb = gb1 - gb0;
     int nb = 0;
     auto for_beads = [&](auto&& f) {  // f(slot in the group order, local cell)
       for (int j0 = 0; j0 < gnb; j0 += 32) {
         const int j = gb0 + j0 + lane;
-        if (j0 + lane < gnb) f(j, B.bgc[j] - c0);
+        if (j0 + lane < gnb) {
+          const int lc = B.bgc[j] - c0;  // beads of the group's other cells: another warp's
+          if ((unsigned)lc < (unsigned)cpw) f(j, lc);
+        }
       }
     };
     if (BEADS && MODE != MODE_P) {

@@ -34,9 +34,11 @@ constexpr int WARP_MAX_K = 448;
 // Members that a warp of k_srd stages at a time, and the longest row it takes.
 constexpr int SRD_SLOTS = 192;
 // ang (mixed model, SRD without beads): the angular-momentum correction.
+// cpw: cells per warp (32, 16 or 8); a 256-cell span is taken in 32 / cpw parts, one block
+// each: grid sizes count parts.
 int cells_warp_blocks_per_sm(bool thermo, bool force, bool beads, bool at, bool ang, int mode);
 void launch_cells_warp(bool thermo, bool force, bool beads, bool at, bool ang, int mode,
-                       const BoxDev* boxes, const int2* spans, int nspans, int grid, int* err,
+                       const BoxDev* boxes, const int2* spans, int nspans, int grid, int cpw, int* err,
                        cudaStream_t s);
 // The same step for mixed SRD boxes (walls: with channel walls, then without
 // beads) and, without walls and beads, mixed boxes with the Andersen rule (at) or the

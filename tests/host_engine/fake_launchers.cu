@@ -62,9 +62,9 @@ void launch_srdd(bool, bool, int mode, const BoxDev*, const int2*, int nspans, i
                  cudaStream_t) {
   fused("srdd", mode, nspans, grid, cpw);
 }
-void launch_cells_warp(bool, bool, bool, bool, bool, int mode, const BoxDev*, const int2*, int nspans, int grid, int*,
-                       cudaStream_t) {
-  fused("warp", mode, nspans, grid, 32);
+void launch_cells_warp(bool, bool, bool, bool, bool, int mode, const BoxDev*, const int2*, int nspans, int grid,
+                       int cpw, int*, cudaStream_t) {
+  fused("warp", mode, nspans, grid, cpw);
 }
 void launch_cells_warpd(bool, bool, bool, bool, int mode, const BoxDev*, const int2*, int nspans, int grid, int*,
                         cudaStream_t) {

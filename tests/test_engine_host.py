@@ -69,6 +69,12 @@ class Box:
     def log(self):
         return self.L.fake_log().decode().split("\n")[:-1]
 
+    def tune(self, reps=1):
+        """mpcd_tune: (blocks per SM, cells per warp)."""
+        bps, cpw = I32(), I32()
+        assert self.L.mpcd_tune(self.ctx, I64(reps), ctypes.byref(bps), None, None, None, ctypes.byref(cpw)) == 0
+        return bps.value, cpw.value
+
     def close(self):
         self.L.mpcd_destroy(self.ctx)
 
@@ -91,6 +97,21 @@ def test_a_large_launch_is_as_many_blocks_as_fit(engine, precision, kernel, per_
     assert box.step(2) == 0
     (name, spans, grid, cpw), = fused(box.log())
     assert (name, spans, cpw) == (kernel, 724, 32) and grid == per_sm * 152
+    box.close()
+
+
+def test_the_tuner_tries_narrow_warps_on_long_rows(engine):
+    """Rows of 193 to 448 records, which k_cells_warp takes: 32 cells a warp untuned, and 16 and 8
+    among the tuner's candidates; the steps after it take what it chose."""
+    box = Box(engine, 150000, n=(10, 10, 10), precision="mixed")
+    assert box.step(2) == 0
+    assert fused(box.log()) == [("warp", 4, 4, 32)]
+    engine.fake_cost(8, 0.25)
+    bps, cpw = box.tune()
+    engine.fake_cost(8, 1.0)
+    assert cpw == 8 and {x[3] for x in fused(box.log())} == {32, 16, 8}
+    assert box.step(2) == 0
+    assert fused(box.log()) == [("warp", 4, 16, 8)]
     box.close()
 
 

@@ -210,3 +210,28 @@ def test_observables_of_any_mass(mass):
     kk = np.bincount(c, mass * (v * v).sum(1), cnt.size)[ok] / (3.0 * (cnt[ok] - 1))
     assert abs(ob["T_cell_mean"] - T.mean()) <= err.mean() + 1e-13 * kk.mean()
     assert ob["occupied_cells"] == int((cnt > 0).sum())
+
+
+@pytest.mark.parametrize("beads", [False, True])
+def test_narrow_warps_on_long_rows_keep_results(beads):
+    """Rows beyond 192 records under the tuner's candidates of 16 and 8 cells a warp (idle lanes, a
+    ragged last part, a bead group shared by warps): real steps, bit for bit those of 32."""
+    n, rho, kw, sp, sv = (6, 5, 4), 130, {}, None, None
+    s = inputs.solvent(n, rho, seed=31, mixed=True)
+    if beads:
+        kw = dict(chain_len=10, md_substeps=4, solute_mass=5.0, bond_k=300.0, bond_r0=0.5)
+        sp, sv = inputs.chains(n, 12, 10, 0.5, bead_mass=5.0, seed=32)
+    got = []
+    for tuned in (True, False):
+        box = pkg.Box(n=n, seed=31, precision="mixed", thermostat=True, body_force=(0.01, 0.0, -0.02), **kw)
+        box.set_state(s.pos, s.vel, sp, sv)
+        if tuned:
+            taken = box.tune(1)[2]
+        else:
+            box.step(taken)
+        box.step(2)
+        got.append(box.get_state())
+        box.close()
+    assert got[0][4] == got[1][4] == taken + 2
+    for a, b in zip(got[0][:4], got[1][:4]):
+        np.testing.assert_array_equal(a, b)
