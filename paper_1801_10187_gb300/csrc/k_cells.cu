@@ -21,6 +21,7 @@
 // at): a second pass over the cell's members forms dL = sum m r_c x (v - v')
 // and the inertia tensor about the cell's centre of mass, and every member
 // then receives omega x r_c with Pi omega = dL.
+#define MPCD_PHILOX_HALVES  // see philox()
 #include <algorithm>
 
 #include "dev_angular.cuh"

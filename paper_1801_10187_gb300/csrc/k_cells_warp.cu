@@ -1,5 +1,6 @@
 // k_cells_warp.cu -- instances and launch dispatch of the warp-spread SRD step
 // of the mixed model (kernel template: k_cells_warp.cuh).
+#define MPCD_PHILOX_HALVES  // see philox()
 #include "k_cells_warp.cuh"
 
 namespace mpcd {

@@ -164,15 +164,25 @@ struct ScanSeg {
 
 // ---------------------------------------------------------------------------
 // Philox4x32-10 (Salmon, Moraes, Dror & Shaw, SC11).  Each 32 x 32 -> 64 product is
-// one wide multiply; low half and __umulhi apart cost the thermostat's step, two to
-// four blocks a cell, 2.5 % (237 against 231 us for 10^7 particles).
+// one wide multiply; low half and __umulhi apart cost the thermostat's step of k_srd,
+// two to four blocks a cell, 2.5 % (237 against 231 us for 10^7 particles).  In
+// k_cells_warp and k_cells, whose registers are spent, the pairs of registers that
+// wide products take cost the thermostat's step more than they save (48^3 cells at
+// density 150 485 against 464 us, at density 300 978 against 933): they ask for halves
+// (MPCD_PHILOX_HALVES, set by a file before it includes this one).  The same numbers.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint4 philox(uint4 c, uint2 k) {
 #pragma unroll
   for (int round = 0; round < 10; ++round) {
+#ifdef MPCD_PHILOX_HALVES
+    const uint32_t al = 0xD2511F53u * c.x, ah = __umulhi(0xD2511F53u, c.x);
+    const uint32_t bl = 0xCD9E8D57u * c.z, bh = __umulhi(0xCD9E8D57u, c.z);
+    c = make_uint4(bh ^ c.y ^ k.x, bl, ah ^ c.w ^ k.y, al);
+#else
     const unsigned long long a = 0xD2511F53ull * c.x, b = 0xCD9E8D57ull * c.z;
     c = make_uint4((uint32_t)(b >> 32) ^ c.y ^ k.x, (uint32_t)b, (uint32_t)(a >> 32) ^ c.w ^ k.y,
                    (uint32_t)a);
+#endif
     k.x += 0x9E3779B9u;
     k.y += 0xBB67AE85u;
   }
