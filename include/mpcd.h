@@ -172,15 +172,15 @@ int mpcd_step(mpcd_ctx* ctx, int64_t nsteps);
  * the threads per cell, on real steps at run time, Sec. 3.5 and Sec. 4): each
  * candidate of the fused step kernel -- its grid (1 up to the occupancy limit
  * of blocks per SM, and one block per span part) times, where the kernel
- * leaves the choice, the cells each warp owns (32, 16 or 8: a 256-cell span is
- * then taken in 2, 4 or 8 parts, one block each: more blocks for a small box,
- * idle lanes in the per-cell work) -- runs steps_per_candidate real steps, timed
+ * leaves the choice, the cells each warp owns (32, 16 or 8, and 4 on boxes that
+ * have 4 untuned: a 256-cell span is then taken in parts, one block each: more
+ * blocks for a small box, idle lanes in the per-cell work) -- runs steps_per_candidate real steps, timed
  * with CUDA events; the fastest is kept for later steps.  The simulation
  * advances by *steps_taken steps (one more when the first step must stream and
  * bin).  Results do not depend on the candidate (mixed model bit for bit; FP64
  * to rounding).  Outputs may be NULL: *blocks_per_sm (-1 = one block per span
  * part), *ms_per_step of the winner, *pass2_chunk (always 3: no longer a
- * choice), *cells_per_warp (32, 16 or 8).
+ * choice), *cells_per_warp (32, 16 or 8; 8 also stands for 4).
  * Synchronises.  Errors: EINVAL, ESTATE, ECUDA, EDEVICE. */
 int mpcd_tune(mpcd_ctx* ctx, int64_t steps_per_candidate, int32_t* blocks_per_sm,
               double* ms_per_step, int64_t* steps_taken, int32_t* pass2_chunk,

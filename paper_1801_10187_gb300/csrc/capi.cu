@@ -785,9 +785,9 @@ struct Engine {
   // on real steps (Sec. 3.5, Sec. 4).  Here each candidate of the fused pass
   // -- grid (1 .. occupancy-limit blocks per SM, and one block per span part)
   // times, for k_srd, k_srd_d and the SRD variants of k_cells_warp, the cells per
-  // warp (32, 16 or 8)
-  // -- runs `reps` real steps, timed with CUDA events on the
-  // stream; the fastest is kept and the step graph re-captured.  Results do
+  // warp (32, 16 or 8, and 4 where that is the width by size) -- runs `reps` real
+  // steps, timed with CUDA events on the stream; the fastest is kept and the step
+  // graph re-captured.  Results do
   // not depend on the candidate: the mixed model's cell sums are exact, the
   // FP64 ones differ at rounding.
   int tune(int64_t reps, int32_t* chosen, double* best_ms, int64_t* steps_taken,
@@ -805,11 +805,17 @@ struct Engine {
       pending = true;
       taken += 1;
     }
-    bool any_width = false;
+    bool any_srd = false, any_width = false;
     for (int v = 0; v < NVAR; ++v)
-      if (n_spans[v] > 0 && ((v & 64) || narrows(v))) any_width = true;
+      if (n_spans[v] > 0) {
+        any_srd |= (v & 64) != 0;
+        any_width |= (v & 64) || narrows(v);
+      }
+    tuned_cpw = 0;
+    const int by_size = srd_cpw();
     std::vector<int> widths = {32};  // cells per warp
     if (any_width) widths = {32, 16, 8};
+    if (any_srd && by_size < 8) widths.push_back(by_size);  // what the boxes have untuned
     cudaEvent_t e0, e1;
     CUDA_TRY(cudaEventCreate(&e0));
     CUDA_TRY(cudaEventCreate(&e1));
@@ -847,7 +853,7 @@ struct Engine {
     CUDA_TRY(cudaGetLastError());
     if (chosen) *chosen = best_c;
     if (chosen_chunk) *chosen_chunk = 3;
-    if (chosen_cpw) *chosen_cpw = best_cpw;
+    if (chosen_cpw) *chosen_cpw = std::max(best_cpw, 8);  // 8 stands for the narrower too
     if (best_ms) *best_ms = best;
     if (steps_taken) *steps_taken = taken;
     return check_err();

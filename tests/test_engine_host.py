@@ -115,6 +115,23 @@ def test_the_tuner_tries_narrow_warps_on_long_rows(engine):
     box.close()
 
 
+@pytest.mark.parametrize("precision,n,kernel", [("mixed", 16, "srd"), ("fp64", 10, "srdd")])
+def test_the_tuner_can_keep_the_width_of_a_small_box(engine, precision, n, kernel):
+    """A box that takes four cells a warp untuned takes them after the tuner, too, where they are
+    the fastest; the width that the call returns has no value for them and is its smallest."""
+    box = Box(engine, 10 * n ** 3, n=(n, n, n), precision=precision)
+    assert box.step(2) == 0
+    (name, spans, grid, cpw), = fused(box.log())
+    assert (name, cpw) == (kernel, 4)
+    engine.fake_cost(4, 0.25)
+    assert box.tune()[1] == 8
+    engine.fake_cost(4, 1.0)
+    assert {x[3] for x in fused(box.log())} == {32, 16, 8, 4}
+    assert box.step(2) == 0
+    assert fused(box.log())[0][3] == 4
+    box.close()
+
+
 def test_a_refused_launch_is_an_error_of_every_step(engine):
     """The cooperative launch of the solute's MD fails during capture: no graph without it is kept,
     so the next steps fail as well, and the first one after that takes it."""
