@@ -37,6 +37,7 @@ void launch_cell_counts(const BoxDev*, int, int, int32_t*, int32_t*, cudaStream_
 void launch_profile(bool, const void*, const void*, int, int, double*, unsigned long long*, double, cudaStream_t) {}
 // puts 1 in every position and 2 in every velocity
 void launch_extract(bool mixed, const BoxDev*, void* pos, void* vel, int32_t*, int, int nsol, uint32_t*, cudaStream_t) {
+  fake_say("extract");
   for (size_t i = 0; i < 3 * (size_t)nsol; ++i)
     if (mixed) {
       ((float*)pos)[i] = 1.0f;

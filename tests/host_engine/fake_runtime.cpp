@@ -100,6 +100,9 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind kin
       if (!b || (uintptr_t)p + n > b->first + b->second.bytes) return cudaErrorInvalidValue;
     }
     say("copy" + num("bytes", n));
+  } else if (kind == cudaMemcpyDeviceToHost) {
+    std::lock_guard<std::mutex> lk(mu);
+    say("read" + num("bytes", n));
   }
   std::memcpy(d, s, n);
   return cudaSuccess;
@@ -120,7 +123,7 @@ cudaError_t cudaGetDriverEntryPointByVersion(const char*, void** f, unsigned, un
 }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = (cudaStream_t)next_handle++; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { say("wait"); return cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { say("capture"); return cudaSuccess; }
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) { *g = (cudaGraph_t)next_handle++; say("end"); return cudaSuccess; }

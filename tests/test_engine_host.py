@@ -132,6 +132,23 @@ def test_the_tuner_can_keep_the_width_of_a_small_box(engine, precision, n, kerne
     box.close()
 
 
+@pytest.mark.parametrize("n_solvent,ahead", [(200000, True), (1000, False)])
+def test_cells_of_large_boxes_are_copied_behind_the_read_out(engine, n_solvent, ahead):
+    """mpcd_last_cells: a large box's copies are queued while its kernels work (device errors of the
+    step looked at before), a small one's after the one wait for both."""
+    box = Box(engine, n_solvent, n=(20, 20, 20), precision="mixed")
+    assert box.step(2) == 0
+    box.log()
+    cells, counts = np.empty(n_solvent, np.int32), np.empty(8000, np.int32)
+    assert engine.mpcd_last_cells(box.ctx, cells.ctypes.data_as(P), counts.ctypes.data_as(P)) == 0
+    log = [x for x in box.log() if x in ("extract", "wait") or x.startswith("read")]
+    sized = [i for i, x in enumerate(log) if x == f"read bytes={4 * n_solvent}"]
+    between = log[log.index("extract") + 1:sized[0]]
+    assert ("wait" in between) != ahead
+    assert ("read bytes=4" in log[:log.index("extract")]) == ahead
+    box.close()
+
+
 def test_a_refused_launch_is_an_error_of_every_step(engine):
     """The cooperative launch of the solute's MD fails during capture: no graph without it is kept,
     so the next steps fail as well, and the first one after that takes it."""
