@@ -1140,9 +1140,12 @@ struct Engine {
   int download_state(Box* b, double* pos, double* vel, double* spos, double* svel, uint64_t* step) {
     // a caller that wants only the beads does not pay for the solvent
     const bool solvent = b->nsol > 0 && (pos || vel);
-    int rc = solvent ? extract(b, nullptr) : complete();
-    if (!rc && !solvent) rc = check_err();
-    if (!rc && step) rc = pull_records();
+    // (ahead: the threads of a long transfer start while the read-out runs)
+    const bool ahead = solvent && 3 * (size_t)b->nsol > XFER_ELEMS;
+    int rc = complete();
+    if (!rc && ahead && step) rc = pull_records();
+    if (!rc) rc = solvent ? extract(b, nullptr, nullptr, nullptr, ahead) : check_err();
+    if (!rc && !ahead && step) rc = pull_records();
     if (rc) return rc;
     const size_t n3 = (size_t)b->nsol * 3;
     if (solvent) {

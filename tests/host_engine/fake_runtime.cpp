@@ -11,7 +11,7 @@
 #include <sys/mman.h>
 
 namespace {
-std::mutex mu;
+std::mutex mu, text_mu;
 std::string text;
 struct Block { size_t bytes; int type, device; };  // type: a cudaMemoryType
 std::map<uintptr_t, Block> blocks;
@@ -21,7 +21,10 @@ double now_ms = 0.0;
 std::map<uintptr_t, double> event_ms;
 uintptr_t next_handle = 16;
 
-void say(const std::string& line) { text += line + "\n"; }
+void say(const std::string& line) {
+  std::lock_guard<std::mutex> lk(text_mu);
+  text += line + "\n";
+}
 std::string num(const char* key, long long v) { return std::string(" ") + key + "=" + std::to_string(v); }
 
 const std::pair<const uintptr_t, Block>* block_of(const void* p) {

@@ -149,6 +149,24 @@ def test_cells_of_large_boxes_are_copied_behind_the_read_out(engine, n_solvent, 
     box.close()
 
 
+@pytest.mark.parametrize("n_solvent,ahead", [(200000, True), (1000, False)])
+def test_the_host_s_threads_start_beside_a_long_read_out(engine, n_solvent, ahead):
+    """mpcd_get_state: the transfer of a large state begins while its read-out runs, the step's
+    errors and its counter looked at before; a small one's after the one wait for all."""
+    box = Box(engine, n_solvent, n=(20, 20, 20), precision="fp64")
+    assert box.step(2) == 0
+    box.log()
+    pos, vel, step = np.empty((n_solvent, 3)), np.empty((n_solvent, 3)), U64()
+    assert engine.mpcd_get_state(box.ctx, pos.ctypes.data_as(P), vel.ctypes.data_as(P), None, None,
+                                 ctypes.byref(step)) == 0
+    log = [x for x in box.log() if x in ("extract", "wait") or x.startswith("read")]
+    first = min(i for i, x in enumerate(log) if x.startswith("read") and int(x.split("=")[1]) > 20000)
+    assert ("wait" in log[log.index("extract") + 1:first]) != ahead
+    assert ("read bytes=4" in log[:log.index("extract")]) == ahead
+    assert np.all(pos == 1.0) and np.all(vel == 2.0)
+    box.close()
+
+
 def test_a_refused_launch_is_an_error_of_every_step(engine):
     """The cooperative launch of the solute's MD fails during capture: no graph without it is kept,
     so the next steps fail as well, and the first one after that takes it."""
