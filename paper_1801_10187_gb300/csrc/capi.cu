@@ -947,13 +947,25 @@ struct Engine {
     d.K = row_capacity(p, nsol);
     d.angular = p.angular ? 1 : 0;
     // k_srd, k_srd_d: cells per sub-tile, as many as rarely have more members than the
-    // staging area holds
-    d.subc = 32;
-    while (d.subc > 1) {
-      const double mean = (double)nsol / (double)C * d.subc;
-      if (mean + 2.5 * std::sqrt(mean) <= (mixed ? SRD_SLOTS : SRDD_SLOTS)) break;
-      d.subc >>= 1;
-    }
+    // staging area holds (subc).  With 32 cells a warp the area has to be full in FP64
+    // and with the thermostat (subw): there a sub-tile of half its slots costs nearly as
+    // much as one of all (us a step: 100^3 cells with the thermostat, density 11 291 ->
+    // 257 with 16 cells for 8, 45 1053 -> 839 with 4 for 2; FP64 58^3, density 12 225 ->
+    // 192), so a few cells may not fit and wait for the next one.  One lane a cell (32)
+    // and one of two cells left over are not worth that; nor are the mixed model's other
+    // rules, which would lose 2 to 5 % at 64^3.
+    auto widest = [&](auto&& fits) {
+      int c = 32;
+      while (c > 1 && !fits(c, (double)nsol / (double)C * c)) c >>= 1;
+      return c;
+    };
+    const double slots = mixed ? SRD_SLOTS : SRDD_SLOTS;
+    auto rarely = [&](int, double mean) { return mean + 2.5 * std::sqrt(mean) <= slots; };
+    auto full = [&](int c, double mean) {
+      return c == 32 ? rarely(c, mean) : mean <= (c > 2 ? (mixed ? 1.25 : 1.3) * slots : slots);
+    };
+    d.subc = d.subw = widest(rarely);
+    if (!mixed || (d.thermostat && !d.angular && !d.walls)) d.subw = widest(full);
     if (d.collision == RULE_AT && nbead > 0 &&
         (d.K > WARP_MAX_K || std::max(p.n[0], std::max(p.n[1], p.n[2])) >= (1 << 22)))
       return fail(MPCD_EINVAL, "the Andersen rule with solute needs a row capacity <= 448 "

@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(SB, AT || ANG ? 5 : BEADS ? 6 : 7)
     };
     int nb = 0;     // beads of this lane's cell; with walls its virtual particles
     int virt = -1;  // with walls: their place in the box's sums
-    const int subc = min(B.subc, cpw);  // most cells per sub-tile, a power of two
+    const int subc = cpw == 32 ? B.subw : min(B.subc, cpw);  // most cells per sub-tile, a power of two
     const int plog = __clz(subc) - 26;  // 2^plog = 32 / subc lanes add up a cell
 
     for (int a = 0; a < cpw;) {

@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(DB, 4) k_srd_d(const BoxDev* __restrict__ boxe
       for (uint32_t j = 0; j < novf; ++j)
         if (oc[j] == (uint32_t)c) f(ovf + j);
     };
-    const int subc = min(B.subc, cpw);  // most cells per sub-tile, a power of two
+    const int subc = cpw == 32 ? B.subw : min(B.subc, cpw);  // most cells per sub-tile, a power of two
     const int plog = __clz(subc) - 26;  // 2^plog = 32 / subc lanes add up a cell
     double ehat = -1.0;                 // thermostat: this lane's cell's draw, < 0: none
 

@@ -130,7 +130,7 @@ struct BoxDev {
   // WCA: epsilon, sigma^2, cutoff^2, list radius^2 (cutoff + buffer), (buffer/2)^2
   double lj_eps, lj_sig2, wca_rc2, wca_rl2, wca_half_skin2;
   int32_t nl_hsize;     // hash buckets of the bead grid (2 per bead, tile-rounded)
-  int32_t subc;         // k_srd: most cells per sub-tile (a power of two)
+  int32_t subc;         // k_srd, k_srd_d: most cells per sub-tile (a power of two)
   int32_t* nl_head;     // bucket -> first bead (-1 empty)
   int32_t* nl_next;     // bead -> next bead in its bucket
   int32_t* nl_key;      // bead -> its cell (edge 1, unshifted) at the build
@@ -142,7 +142,7 @@ struct BoxDev {
   int4* wfix[2];        // the same as 32-bit fractions of the box (x, y, z, 0)
   double wfrac[3];      // 2^32 / L
   float wca_rc2f;       // cutoff^2 with a margin for float distances of wfix
-  int32_t pad_x;
+  int32_t subw;         // the same of a warp of 32 cells
 };
 
 // What a pass leaves to do once all its blocks are done (see finish_pass), passed

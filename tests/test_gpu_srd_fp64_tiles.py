@@ -112,3 +112,13 @@ def test_a_fast_particle_costs_no_other_cell_precision(fast, n, rho, thermostat)
     lone = rk[rc] == 1
     assert lone.any() or rho > 10
     np.testing.assert_array_equal(v[lone], vel[lone])
+
+
+@pytest.mark.parametrize("thermostat", [False, True])
+@pytest.mark.parametrize("rho", [7, 12, 18, 36, 58])
+def test_sub_tiles_that_may_not_fit(rho, thermostat):
+    """Sub-tiles of 32 cells a warp that take up to 16, 8, 4 or 2 cells (mean 96 to 146 of 112 members):
+    what does not fit waits for the next, which starts at any cell."""
+    n = (31, 32, 31)
+    s = inputs.solvent(n, rho, seed=rho)
+    compare(n, s.pos, s.vel, 2, seed=rho, thermostat=thermostat)

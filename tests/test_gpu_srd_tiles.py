@@ -235,3 +235,22 @@ def test_narrow_warps_on_long_rows_keep_results(beads):
     assert got[0][4] == got[1][4] == taken + 2
     for a, b in zip(got[0][:4], got[1][:4]):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("n,rho", [((41, 39, 53), 11), ((43, 41, 45), 14), ((53, 40, 37), 30), ((45, 43, 41), 45),
+                                   ((44, 42, 43), 90)])
+def test_sub_tiles_that_may_not_fit(n, rho):
+    """With the thermostat and 32 cells a warp a sub-tile takes up to 16, 8, 4 or 2 cells whose members
+    fill the staging area (mean 176 to 240 of 192): the cells that do not fit wait for the next,
+    and a sub-tile starts at any cell."""
+    s = inputs.solvent(n, rho, seed=rho, mixed=True)
+    kw = dict(n=n, seed=rho, thermostat=True)
+    box = pkg.Box(precision="mixed", **kw)
+    box.set_state(s.pos, s.vel, step=7)
+    box.step(2)
+    pos, vel, *_ = box.get_state()
+    box.close()
+    ref = oracle.State(s.pos.copy(), s.vel.copy(), step=7)
+    oracle.step(oracle.Params(precision=oracle.MIXED, **kw), ref, 2)
+    np.testing.assert_array_equal(pos, ref.pos)
+    np.testing.assert_array_equal(vel, ref.vel)
