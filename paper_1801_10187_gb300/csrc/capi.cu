@@ -614,11 +614,38 @@ struct Engine {
     return n < g ? std::max(n, 1) : g;
   }
 
+  // Solute boxes (mixed): whether k_srd's two launches, over the bead groups without
+  // beads and with, beat k_cells_warp's one.  What they save grows with the cells, more
+  // so with long rows and with the thermostat of short ones; what they cost is a
+  // launch and dearer bead groups, and with the thermostat sub-tiles whose cells often
+  // do not all fit.  Time of k_srd over that of k_cells_warp either side of the lines,
+  // with w = 0.2 / 0.7 / 2 beads a group: density 5 to 10, 90^3 cells 1.01 / 1.01 / 1.08,
+  // 100^3 0.98 / 1.02 / 1.04, 112^3 0.94 / 0.98 / 1.04, 160^3 0.92 / 0.95 / 0.99; with the
+  // thermostat density 5 80^3 1.02 / 0.99 / 1.00, 90^3 0.97 / 0.96 / 0.98, density 12 to 15
+  // 100^3 1.02 / 1.08 / 1.11, 128^3 0.97 / 1.03 / 1.09; density 20 64^3 0.94 / 0.94 / 0.97, with
+  // the thermostat 64^3 1.03 / 1.02 / 1.05, 80^3 0.91 / 0.91 / 1.01, 100^3 0.82 / 0.88 / 0.96.
+  bool solute_pays(const BoxDev& d) const {
+    const double rho = (double)d.nsol / (double)d.ncells, mean = rho * d.subw;
+    const double w = (double)d.nbead / (double)d.nctiles;
+    const bool few = w <= 0.45, many = w > 1.3, fits = mean + std::sqrt(mean) <= SRD_SLOTS;
+    double cells;
+    if (rho >= 18.0)
+      cells = !d.thermostat ? 0.23e6 : !many ? 0.45e6 : fits ? 0.9e6 : 5e6;
+    else if (d.thermostat && !fits)
+      cells = few ? 1.2e6 : 5e6;
+    else if (d.thermostat && rho < 6.0)
+      cells = 0.6e6;
+    else
+      cells = few ? 0.9e6 : many ? 3.5e6 : 1.2e6;
+    return (double)d.ncells >= cells;
+  }
+
   // Boxes that k_srd (mixed) or k_srd_d (FP64) steps.
   bool on_srd(const BoxDev& d) const {
     if (!mixed && (d.walls || d.nbead > 0 || d.K > SRDD_SLOTS || d.ncells > SRDD_MAX_CELLS)) return false;
     if (d.collision == RULE_AT && (!mixed || d.nbead > 0 || d.angular)) return false;
     if (d.angular && !mixed) return false;
+    if (d.nbead > 0 && !solute_pays(d)) return false;
     return d.K <= SRD_SLOTS &&
            std::max(d.n[0], std::max(d.n[1], d.n[2])) < (1 << 22);
   }
@@ -1044,7 +1071,8 @@ struct Engine {
       if ((rc = alloc(b, d.bgv, (size_t)nbead * 3))) return rc;
       if ((rc = alloc(b, d.bcount, (size_t)d.nctiles))) return rc;
       if ((rc = alloc(b, d.bstart, (size_t)d.nctiles + 1))) return rc;
-      if ((rc = alloc(b, d.bgroup, (size_t)nbead))) return rc;
+      d.listed = mixed && on_srd(d) ? 1 : 0;
+      if (d.listed && (rc = alloc(b, d.bgroup, (size_t)nbead))) return rc;
       CUDA_TRY(cudaMemsetAsync(d.bcount, 0, sizeof(uint32_t) * d.nctiles, stream));
       CUDA_TRY(cudaMemsetAsync(d.bstart, 0, sizeof(uint32_t) * (d.nctiles + 1), stream));
       if (p.lj_epsilon > 0.0) {  // non-bonded WCA repulsion (Sec. 4.3 reading)

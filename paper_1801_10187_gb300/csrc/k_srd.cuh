@@ -41,8 +41,9 @@
 // Both run at five blocks an SM and chunks of one window: the registers of their
 // longer members' phase would spill at seven.
 //
-// Solute boxes take two launches in modes F and C: one over the bead groups
-// without beads, one (BEADS) over those with.  In one launch the bead code's
+// Large solute boxes (solute_pays in capi.cu; k_cells_warp takes the others) take
+// two launches in modes F and C: one over the bead groups without beads, one (BEADS)
+// over those with.  In one launch the bead code's
 // registers cost every cell: 2.69 ms a step at 7.8 10^7 particles with 2000 chains
 // and the thermostat, against 2.14 ms for the same box without beads.
 // The second takes its groups from k_bead_scatter's list, one a warp by turns: with

@@ -261,7 +261,7 @@ __global__ void k_bead_scatter(BoxDev* boxes, const int2* __restrict__ tiles,
     const int b1 = min(tt.y + PTILE, B.nbead);
     for (int b = tt.y + threadIdx.x; b < b1; b += blockDim.x) {
       const uint64_t k = B.bkey[b];
-      if ((uint32_t)k == 0u)  // the group's first bead
+      if (B.listed && (uint32_t)k == 0u)  // the group's first bead
         B.bgroup[min(atomicAdd(&B.nbgroup, 1u), (uint32_t)B.nbead - 1u)] = (uint32_t)(k >> 32);
       const uint32_t slot = B.bstart[(uint32_t)(k >> 32)] + (uint32_t)k;
       B.border[slot] = (uint32_t)b;

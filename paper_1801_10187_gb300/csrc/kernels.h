@@ -44,9 +44,9 @@ void launch_cells_warp(bool thermo, bool force, bool beads, bool at, bool ang, i
 // beads) and, without walls and beads, mixed boxes with the Andersen rule (at) or the
 // angular correction (ang), with rows of at most SRD_SLOTS records (k_srd.cu).  cpw: cells per warp (32, 16,
 // 8 or 4); a 256-cell span is then taken in srd_parts(cpw) parts, one block
-// each: grid sizes count parts.  A solute box takes a launch without beads, over
+// each: grid sizes count parts.  A large solute box takes a launch without beads, over
 // the bead groups that hold none, and one with (cpw 32), over the others; mode P
-// only the first.  SRD_MIN_WARPS: see srd_cpw() in capi.cu.
+// only the first; smaller ones stay with k_cells_warp.  SRD_MIN_WARPS: see srd_cpw() in capi.cu.
 constexpr int SRD_MIN_WARPS = 16, SRDD_MIN_WARPS = 6;
 int srd_blocks_per_sm(bool thermo, bool force, bool beads, bool walls, bool at, bool ang, int mode);
 int srd_parts(int cpw);

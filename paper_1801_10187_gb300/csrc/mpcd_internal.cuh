@@ -115,9 +115,10 @@ struct BoxDev {
   double* bgv;      // velocity of each grouped bead, 3 per bead
   uint32_t* bcount; // per bead group histogram
   uint32_t* bstart; // nctiles + 1
-  uint32_t* bgroup; // the bead groups that hold beads, in any order (at most nbead)
+  uint32_t* bgroup; // listed: the bead groups that hold beads, in any order (at most nbead)
   // updated on the device
   uint32_t nbgroup;  // groups in bgroup; 0 once the step's collision is done
+  int32_t listed;    // 1: k_srd steps the box and takes the groups with beads from bgroup
   unsigned long long step;
   int32_t cur;
   int32_t collision;    // RULE_SRD or RULE_AT

@@ -167,6 +167,19 @@ def test_the_host_s_threads_start_beside_a_long_read_out(engine, n_solvent, ahea
     box.close()
 
 
+@pytest.mark.parametrize("n,chains,thermostat,split", [
+    (40, 40, True, False), (64, 1000, True, False), (100, 128, True, True), (100, 1000, True, True),
+    (80, 60, False, False), (100, 128, False, True), (100, 1000, False, False)])
+def test_solute_boxes_take_the_faster_kernel(engine, n, chains, thermostat, split):
+    """Density 5: two launches of the fused kernel on large boxes, one of the warp-spread kernel on
+    small ones and, without the thermostat, on those full of beads."""
+    box = Box(engine, 5 * n ** 3, 50 * chains, n=(n, n, n), precision="mixed", thermostat=thermostat,
+              chain_len=50, md_substeps=4, solute_mass=5.0, bond_k=100.0, bond_r0=0.5)
+    assert box.step(2) == 0
+    assert [x[0] for x in fused(box.log())] == (["srd", "srd_beads"] if split else ["warp"])
+    box.close()
+
+
 def test_a_refused_launch_is_an_error_of_every_step(engine):
     """The cooperative launch of the solute's MD fails during capture: no graph without it is kept,
     so the next steps fail as well, and the first one after that takes it."""

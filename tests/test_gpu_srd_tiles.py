@@ -254,3 +254,25 @@ def test_sub_tiles_that_may_not_fit(n, rho):
     oracle.step(oracle.Params(precision=oracle.MIXED, **kw), ref, 2)
     np.testing.assert_array_equal(pos, ref.pos)
     np.testing.assert_array_equal(vel, ref.vel)
+
+
+@pytest.mark.parametrize("n,rho,nch,thermostat", [((100, 80, 76), 1, 300, True), ((100, 80, 76), 5, 3000, True),
+                                                  ((64, 63, 58), 18, 300, False), ((64, 63, 58), 45, 2000, False)])
+def test_beads_of_large_boxes(n, rho, nch, thermostat):
+    """Solute boxes large enough for the fused kernel's two launches, over the bead groups without
+    beads and, from the list, with: sub-tiles of 32, 16, 8 and 2 cells, few beads and many."""
+    s = inputs.solvent(n, rho, seed=9, mixed=True)
+    sp, sv = inputs.chains(n, nch, 10, 0.5, bead_mass=5.0, seed=10)
+    kw = dict(n=n, seed=9, thermostat=thermostat, chain_len=10, md_substeps=4, solute_mass=5.0, bond_k=300.0,
+              bond_r0=0.5)
+    box = pkg.Box(precision="mixed", **kw)
+    box.set_state(s.pos, s.vel, sp, sv)
+    box.step(2)
+    got = box.get_state()
+    box.close()
+    ref = oracle.State(s.pos.copy(), s.vel.copy(), sp.copy(), sv.copy())
+    oracle.step(oracle.Params(precision=oracle.MIXED, **kw), ref, 2)
+    np.testing.assert_array_equal(got[0], ref.pos)
+    np.testing.assert_array_equal(got[1], ref.vel)
+    np.testing.assert_allclose(got[2], ref.spos, rtol=0, atol=1e-10)
+    np.testing.assert_allclose(got[3], ref.svel, rtol=0, atol=1e-10 * max(1.0, np.abs(ref.svel).max()))
