@@ -232,8 +232,9 @@ int mpcd_last_cells(mpcd_ctx* ctx, int32_t* cell_out, int32_t* count_out);
 
 /* Internal profiler: advance nsteps SRD steps with plain launches and a CUDA
  * event between phases; ms[i] receives the mean time of phase i per step
- * (phases: md_bin, stream_bin, scan, scatter, permute, collide, end_step;
- * see mpcd_phase_name).  nmax: capacity of ms (>= 7).  Synchronises.  The
+ * (phases: fused_step, with the virtual wall particles; after_pass, the record
+ * updates where the fused launch does not do them itself; solute; see
+ * mpcd_phase_name).  nmax: capacity of ms (>= 3).  Synchronises.  The
  * steps are real steps: the state advances. */
 int mpcd_phase_times(mpcd_ctx* ctx, int64_t nsteps, double* ms, int32_t nmax, int32_t* nphases);
 const char* mpcd_phase_name(int32_t i);

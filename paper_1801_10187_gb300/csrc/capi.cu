@@ -679,15 +679,13 @@ struct Engine {
     return grid_for(items, (mode == MODE_F && tuned_grid > 0) ? std::min(tuned_grid, limit) : limit);
   }
 
-  // One pass over every box, with the record updates that end it: by the last
-  // launch itself where that is k_srd or k_srd_d (they come last), else by a
-  // kernel of their own.
+  // One pass over every box.  The record updates that end it are done by the last
+  // launch itself where that is k_srd or k_srd_d (they come last), else left to
+  // end_pass, by a kernel of their own.
   void launch_cells_all(int mode) {
     const AfterPass none{};
     AfterPass end{d_boxes, (int)live.size(), mode != MODE_C, mode != MODE_P, d_done};
-    int last = -1;
-    for (int v = 0; v < NVAR; ++v)
-      if (n_spans[v] > 0) last = v;
+    const int last = last_variant();
     for (int v = 0; v < NVAR; ++v) {
       if (n_spans[v] == 0) continue;
       const int grid = grid_of(v, mode);
@@ -714,8 +712,16 @@ struct Engine {
         launch_cells(mixed, v, mode, d_boxes, d_spans[v], n_spans[v], grid, d_err, stream);
       }
     }
-    if (last < 64)
+  }
+  void end_pass(int mode) {
+    if (last_variant() < 64)
       launch_after_pass(d_boxes, (int)live.size(), mode != MODE_C, mode != MODE_P, stream);
+  }
+  int last_variant() const {
+    int last = -1;
+    for (int v = 0; v < NVAR; ++v)
+      if (n_spans[v] > 0) last = v;
+    return last;
   }
 
   // Solute: MD substeps and bead grouping for the step in the records.  Returns the
@@ -745,6 +751,7 @@ struct Engine {
       cudaEventRecord(ev_join, side);
     }
     launch_cells_all(mode);
+    end_pass(mode);
     if (n_vtiles > 0 && mode == MODE_F) cudaStreamWaitEvent(stream, ev_join, 0);
     if (n_vtiles > 0 && mode == MODE_P)
       launch_virtual(d_boxes, (int)live.size(), d_vtiles, n_vtiles, 1, d_done + 1, stream);
@@ -914,7 +921,8 @@ struct Engine {
         launch_virtual(d_boxes, (int)live.size(), d_vtiles, n_vtiles, 0, d_done + 1, stream);
       launch_cells_all(MODE_F);
       CUDA_TRY(cudaEventRecord(ev[1], stream));
-      CUDA_TRY(cudaEventRecord(ev[2], stream));  // (the record updates are part of the pass)
+      end_pass(MODE_F);
+      CUDA_TRY(cudaEventRecord(ev[2], stream));
       CUDA_TRY(launch_beads());
       CUDA_TRY(cudaEventRecord(ev[3], stream));
       CUDA_TRY(cudaEventSynchronize(ev[3]));

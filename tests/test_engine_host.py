@@ -180,6 +180,19 @@ def test_solute_boxes_take_the_faster_kernel(engine, n, chains, thermostat, spli
     box.close()
 
 
+@pytest.mark.parametrize("density,after", [(150, 0.125), (10, 0.0)])
+def test_phase_times_of_the_record_updates(engine, density, after):
+    """mpcd_phase_times: the kernel that ends a pass of the warp-spread kernel is a phase of its own, and
+    no part of the fused step's; the fused kernel does without."""
+    box = Box(engine, 1000 * density, n=(10, 10, 10), precision="mixed")
+    engine.fake_cost(-1, 0.125)
+    ms, n = (ctypes.c_double * 8)(), I32()
+    assert engine.mpcd_phase_times(box.ctx, I64(4), ms, 8, ctypes.byref(n)) == 0
+    engine.fake_cost(-1, 1.0)
+    assert n.value == 3 and list(ms[:3]) == [1.0, after, 0.0]
+    box.close()
+
+
 def test_a_refused_launch_is_an_error_of_every_step(engine):
     """The cooperative launch of the solute's MD fails during capture: no graph without it is kept,
     so the next steps fail as well, and the first one after that takes it."""
