@@ -283,7 +283,7 @@ def main():
     ap.add_argument("--no-sweep", action="store_true", help="served workload: skip the rate sweep")
     ap.add_argument("--no-tune", action="store_true",
                     help="skip the launch tuner: the engine's default launch (blocks per SM at "
-                         "the occupancy limit, pass-2 chunks of 3, 32 cells per warp); for "
+                         "the occupancy limit, cells per warp by the size of the box); for "
                          "profiling a fixed configuration")
     args = ap.parse_args()
     cfg = workload_cfg(args.workload)
@@ -344,7 +344,7 @@ def main():
     # re-captured step graph warms up again
     if args.no_tune:
         config["launch"] = {"blocks_per_sm": "occupancy limit", "pass2_chunk": 3,
-                            "cells_per_warp": 32, "tuner": "off"}
+                            "cells_per_warp": "by size", "tuner": "off"}
     else:
         tuned_bps, tuned_ms, _, tuned_chunk, tuned_cpw = box.tune(2)
         config["launch"] = {"blocks_per_sm": tuned_bps if tuned_bps > 0 else "one per span part",
