@@ -253,7 +253,8 @@ const char* mpcd_last_error(void);
 /* (one launch per phase covers every resident box).  Boxes differ in size, */
 /* density, rotation angle, seed and thermostat; one precision per batch.   */
 /* A box gives the same result alone and in any batch (counter-based draws  */
-/* keyed by the box's own seed, step and cell).                             */
+/* keyed by the box's own seed, step and cell), in the FP64 model to        */
+/* rounding: how a cell's energy is summed goes with the launch.            */
 /* ---------------------------------------------------------------------- */
 typedef struct mpcd_batch mpcd_batch;
 

@@ -1,5 +1,5 @@
-// k_srd.cu -- instances and launch dispatch of the fused SRD step with the
-// members in registers (kernel template: k_srd.cuh).
+// k_srd.cu -- instances and launch dispatch of the fused SRD step of the mixed
+// model (kernel template: k_srd.cuh).
 #include "k_srd.cuh"
 
 namespace mpcd {

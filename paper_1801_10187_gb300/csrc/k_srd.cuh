@@ -50,8 +50,8 @@
 // a span of 256 cells to a warp it lasted as long as the warp with the most groups
 // (2.61 against 2.46 ms for the step with its bead MD).
 //
-// What bounds it: neither DRAM (44 % of its peak at 10^7 particles) nor the
-// issue slots (53 %) nor the L1 pipe (63 %), but the chain count -> stage ->
+// What bounds it: neither DRAM (46 % of its peak at 10^7 particles) nor the
+// issue slots (52 %) nor the L1 pipe (64 %), but the chain count -> stage ->
 // sums -> slot -> store of global latencies, covered by the 28 warps that
 // registers and shared memory leave room for.  A stand-in with the same reads,
 // slot atomics and scattered writes and no arithmetic takes 131 us at 10^7

@@ -24,7 +24,8 @@
 // keeps its velocity, as v - u = 0 leaves it.  Streaming is the same fma.  With the
 // thermostat the energy about u and the scaling by xi stay in double.  What bounds
 // it now: 16 warps an SM (115 registers, 47 KB a block) that wait on the FP64 pipe
-// and the integer pipes in turn, neither of them half busy; the line beyond which
+// (44 % busy at 50^3 cells) and the integer pipes (37 % of the issue slots) in turn,
+// and on how many of its slots a sub-tile fills; the line beyond which
 // k_cells_warp_d is taken is at SRDD_MAX_CELLS (kernels.h).  On small boxes a tile's
 // latency is what counts, and 4 to 32 cells a warp spread them over the SMs (us a
 // step): 10^3 cells at density 5 35 -> 12, with the thermostat 57 -> 22; 16^3 at

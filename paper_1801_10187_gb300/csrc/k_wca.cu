@@ -21,8 +21,8 @@
 // ERR_NLIST.  The later binning of the beads for the collision (k_md_bin) skips
 // its own MD for these boxes.
 //
-// What bounds it: the FP64 pipe (a warp instruction every 16 cycles of an SM) and
-// the launches.  The first form took five launches a substep, of which three
+// What bounds it: the FP64 pipe (51 % busy; a warp instruction every 16 cycles of an
+// SM) and the barriers.  The first form took five launches a substep, of which three
 // returned at once in nearly every one, and 45 us of force kernel: distances of
 // all listed pairs in double, each bond from both its sides with a square root
 // and a division.  Here pairs are sorted out by their distance in float from
@@ -62,8 +62,8 @@ __device__ __forceinline__ int grid_coord(double x, int n) {
 // the same as d - L rint(d / L), where a difference of just L / 2 stays (ties to
 // even).  L / 2 has no low word, so the words of d settle the comparison off the
 // FP64 pipe; and in this form the subtraction is branched over, as nearly always,
-// and not computed and dropped: the solute MD of a step takes 2.0 and not 2.5 ms
-// for 1024 chains of 50 beads.
+// and not computed and dropped: four steps of 1024 chains of 50 beads and the read
+// 11.35 -> 9.74 ms.
 __device__ __forceinline__ double min_image(double d, double L) {
   const int h = __double2hiint(L) - 0x00100000;  // of L / 2
   const int e = __double2hiint(d) & 0x7FFFFFFF;

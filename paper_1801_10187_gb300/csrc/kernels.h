@@ -12,16 +12,6 @@ namespace mpcd {
 // variant = (thermostat ? 1 : 0) | (solute beads or walls ? 2 : 0) |
 // (Andersen rule ? 16 : 0) | (angular-momentum correction ? 32 : 0); the last
 // two without solute or walls.
-// Solute MD of one collision step for the boxes with the non-bonded WCA
-// repulsion (k_wca.cu): neighbour-list build, then max_substeps velocity-
-// Verlet substeps (each box takes its own md_substeps).
-// tiles: (box, first of WCA_BEADS beads); sync: four device words, zeroed here;
-// max_blocks: blocks that fit on the device together (wca_blocks_per_sm per
-// SM; the launch is cooperative).  Returns a cudaError_t.
-constexpr int WCA_BEADS = 127;
-int wca_blocks_per_sm();
-int launch_wca_md(const BoxDev* boxes, const int2* tiles, int ntiles, int max_substeps, int max_blocks,
-                  unsigned* sync, int* err, cudaStream_t s);
 int cells_blocks_per_sm(bool mixed, int variant, int mode);
 void launch_cells(bool mixed, int variant, int mode, const BoxDev* boxes, const int2* spans,
                   int nspans, int grid, int* err, cudaStream_t s);
@@ -94,6 +84,17 @@ void launch_extract(bool mixed, const BoxDev* box, void* pos, void* vel, int32_t
 // type); sums: 3 device words of scratch.
 void launch_init_thermal(bool mixed, int n, uint64_t seed, const double L[3], double sigma,
                          void* pos, void* vel, unsigned long long* sums, cudaStream_t s);
+
+// Solute MD of one collision step for the boxes with the non-bonded WCA
+// repulsion (k_wca.cu): neighbour-list build, then max_substeps velocity-
+// Verlet substeps (each box takes its own md_substeps).
+// tiles: (box, first of WCA_BEADS beads); sync: four device words, zeroed here;
+// max_blocks: blocks that fit on the device together (wca_blocks_per_sm per
+// SM; the launch is cooperative).  Returns a cudaError_t.
+constexpr int WCA_BEADS = 127;
+int wca_blocks_per_sm();
+int launch_wca_md(const BoxDev* boxes, const int2* tiles, int ntiles, int max_substeps, int max_blocks,
+                  unsigned* sync, int* err, cudaStream_t s);
 
 // ---- solute and pass bookkeeping (k_step.cu) ----
 // Allows k_md_bin the shared memory of 1024-thread blocks; returns a cudaError_t.
