@@ -1404,8 +1404,8 @@ int mpcd_get_state_device(mpcd_ctx* ctx, void* pos, void* vel) {
   Engine& E = ctx->eng;
   Box* b = ctx->box;
   // straight into the caller's arrays where a kernel may store there, else (another
-  // device's memory, a pointer that the driver has to judge, arrays that overlap)
-  // through the staging arrays and a copy
+  // device's memory, a pointer that may be none, arrays that overlap) through the
+  // staging arrays and a copy
   const size_t es = elem_size(E.mixed), bytes = (size_t)b->nsol * 3 * es;
   const bool apart = !pos || !vel || (const char*)pos + bytes <= (const char*)vel ||
                      (const char*)vel + bytes <= (const char*)pos;

@@ -4,13 +4,14 @@
 // Sec. 3.6 rotation and thermostat, algorithm "SRD collision rule").
 //
 // Same modes, records and results as k_cells (one thread per cell), for boxes
-// without walls (solute beads allowed): the Andersen rule, the angular
-// correction, and SRD with rows beyond the SRD_SLOTS records that k_srd, the
-// faster kernel for plain SRD, takes.  A warp owns cpw consecutive cells: 32, or
-// for SRD in mode F 16 or 8 where the launch tuner finds that faster (a 256-cell
-// span is then taken in 32 / cpw parts, one block each; results do not depend on
-// it).  With rows this long a warp's cells take it long, so narrow warps pay: 32^3
-// cells at density 150 292 -> 137 us a step, 96^3 2942 -> 2743.  Their row members are numbered 0 .. N-1 in cell order (a warp prefix sum of the row
+// without walls (solute beads allowed): solute boxes below the size at which the two
+// launches of k_srd, the faster kernel for plain SRD, pay, the Andersen rule with
+// solute, and SRD and the angular correction with rows beyond the SRD_SLOTS records
+// that k_srd takes.  A warp owns cpw consecutive cells: 32, or for SRD in mode F 16 or
+// 8 where the launch tuner finds that faster (a 256-cell span is then taken in 32 / cpw
+// parts, one block each; results do not depend on it).  Long rows take a warp long, so
+// narrow warps pay: 32^3 cells at density 150 292 -> 137 us a step, 96^3 2942 -> 2743.
+// The row members are numbered 0 .. N-1 in cell order (a warp prefix sum of the row
 // counts); a byte map gives each member's cell.
 //   pass 1   the (v, tag) words of up to 192 members are copied into shared
 //            memory asynchronously in member order (neighbouring lanes,
